@@ -265,3 +265,77 @@ def tolerance(case):
         return {"rel": 1e-5, "differ": 5e-3}
     tol = {"rel": 1e-2, "max": 0.12} if case["bf16"] else {"rel": 5e-6, "max": 3e-5}
     return tol if kind == "steps" else dict(tol, differ=5e-3)
+
+
+# ---- the same pass in 64 bits, in plain torch -----------------------------------------------------------------------
+
+def _unpack(W13p, I):
+    """Rows of W1 and of W3 inside the packed array: blocks of 128 channels of W1, then the same channels of W3."""
+    i = torch.arange(I, device=W13p.device)
+    gate = i // 128 * 256 + i % 128
+    return gate, gate + torch.clamp(I - i // 128 * 128, max=128)
+
+
+def _expert(x, W13, W2, rows, s, g):
+    """s silu(x W1^T) (x W3^T) W2^T for rows x and, with g = dL/dY, also dx, dW13 (packed), dW2 and s <g, expert(x)>."""
+    W13, W2 = W13.double(), W2.double()
+    gate, up = rows
+    a, b = x @ W13[gate].T, x @ W13[up].T
+    sg = torch.sigmoid(a)
+    h = a * sg * b
+    y = s[:, None] * (h @ W2.T)
+    if g is None:
+        return y, None
+    dh = s[:, None] * (g @ W2)
+    da, db = dh * b * sg * (1 + a * (1 - sg)), dh * a * sg
+    dW13 = torch.empty_like(W13)
+    dW13[gate], dW13[up] = da.T @ x, db.T @ x
+    return y, (da @ W13[gate] + db @ W13[up], dW13, g.T @ (s[:, None] * h), (dh * h).sum(1))
+
+
+def exact(case, seed):
+    s = prepare(case, seed)
+    kind, E, K, I, I_s = case["kind"], case["E"], case["K"], case["I"], case["I_s"]
+    if kind == "calibrate":
+        return {"L": s["X"].double() @ s["Wg"].double().T, "idx": None, "C": None, "I_T": None}
+    t = s if kind == "dispatch" else s["lay"].t
+    X = t["X"].double()
+    L = t["L"].double() if kind in ("dispatch", "steps") else X @ t["Wg"].double().T
+    # Sec. 3.3 step 2: the best expert of all, then the K - 1 best inside its collaborator set (ties: lower index)
+    top = L.argmax(1)
+    member = ((t["mask"][:, None] >> torch.arange(E, device="cuda")[None, :]) & 1).bool()[top]
+    rest = L.masked_fill(~member, -math.inf).scatter(1, top[:, None], -math.inf)
+    idx = torch.cat([top[:, None], rest.sort(dim=1, descending=True, stable=True).indices[:, :K - 1]], 1)
+    w = torch.softmax(L.gather(1, idx), 1)
+    if kind == "dispatch":
+        return {"w": w}
+    dY = t["dY"].double() if kind == "train" else None
+    Y, out = torch.zeros_like(X), {}
+    dX, q = torch.zeros_like(X), torch.zeros_like(w)
+    if kind == "train":
+        out["dW13p"] = torch.zeros(t["W13p"].shape, dtype=torch.float64, device="cuda")
+        out["dW2"] = torch.zeros(t["W2"].shape, dtype=torch.float64, device="cuda")
+    rows = _unpack(t["W13p"], I)
+    for e in range(E):
+        tok, k = (idx == e).nonzero(as_tuple=True)
+        if len(tok) == 0:
+            continue
+        y, back = _expert(X[tok], t["W13p"][e], t["W2"][e], rows, w[tok, k], None if dY is None else dY[tok])
+        Y.index_add_(0, tok, y)
+        if back is not None:
+            dX.index_add_(0, tok, back[0])
+            out["dW13p"][e], out["dW2"][e], q[tok, k] = back[1:]
+        del y, back
+    if I_s:
+        gs = torch.sigmoid(X @ t["wsg"].double())
+        y, back = _expert(X, t["Ws13p"][0], t["Ws2"][0], _unpack(t["Ws13p"], I_s), gs, dY)
+        Y += y
+        if back is not None:
+            dz = back[3] * (1 - gs)
+            dX += back[0] + dz[:, None] * t["wsg"].double()
+            out.update(dWs13p=back[1][None], dWs2=back[2][None], dwsg=dz @ X)
+    if kind == "train":
+        dL = torch.zeros_like(L).scatter(1, idx, q - w * q.sum(1, keepdim=True))
+        dX += dL @ t["Wg"].double()
+        out.update(dX=dX, dWg=dL.T @ X)
+    return dict(out, Y=Y, w=w)
