@@ -90,7 +90,8 @@ static int apply_opts(const c2r_config* cfg, const c2r_expert_opts* o, SwigluCal
 static int swiglu_fwd_dispatch(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) {
   if (a.R == 0) return C2R_OK;
   if (cfg->dtype == C2R_F32) return simt_swiglu_fwd<float>(cfg, a, s);
-  if (tc_supported(cfg, a.nE, a.I, a.R)) return tc_swiglu_fwd(cfg, a, s);
+  if (tc_supported(cfg, a.nE, a.I, a.R))
+    return skinny_supported(cfg, a, SKINNY_ROWS) ? skinny_swiglu_fwd(cfg, &a, 1, s) : tc_swiglu_fwd(cfg, a, s);
   return simt_swiglu_fwd<__nv_bfloat16>(cfg, a, s);
 }
 
@@ -219,7 +220,22 @@ extern "C" int c2r_layer_fwd(const c2r_config* cfg, const c2r_layer_buffers* b, 
   const LayerWs ws = layer_ws(cfg, b->ws);
   const SideStream ss(b, stream, shared);
   C2R_TRY(gate_logits_impl(cfg, b->X, b->Wg, shared ? b->wsg : nullptr, b->L, b->z, b->status, stream));
-  if (shared) {
+  // With a few rows per expert the shared expert rides along with the routed ones: calls[0] shared, calls[1] routed.
+  SwigluCall calls[2] = {};
+  bool paired = false;
+  if (shared && !fcomb && !ss.on && !gather_fused(cfg, b->X) && cfg->N > 0 && cfg->I > 0) {
+    SwigluCall &sh = calls[0], &ro = calls[1];
+    sh.nE = 1; sh.I = cfg->I_s; sh.R = cfg->N; sh.Xp = b->X; sh.counts = b->s_counts; sh.offsets = b->s_offsets;
+    sh.W13p = b->Ws13p; sh.W2 = b->Ws2; sh.row_scale = b->z; sh.scale_kind = C2R_SCALE_SIGMOID; sh.AB = b->ABs; sh.H = b->Hs;
+    sh.Yp = b->Ys; sh.status = b->status;
+    ro.nE = cfg->E; ro.I = cfg->I; ro.R = R; ro.Xp = b->Xp; ro.counts = b->counts; ro.offsets = b->offsets;
+    ro.W13p = b->W13p; ro.W2 = b->W2; ro.row_scale = b->w_row; ro.scale_kind = C2R_SCALE_ROW; ro.AB = b->AB; ro.H = b->H;
+    ro.Yp = b->Yp; ro.status = b->status;
+    paired = sh.Xp && ro.counts && ro.offsets && ro.W13p && ro.W2 && ro.H && tc_supported(cfg, 1, sh.I, sh.R) &&
+             tc_supported(cfg, ro.nE, ro.I, R) && skinny_supported(cfg, sh, SKINNY_ROWS_PAIRED) &&
+             skinny_supported(cfg, ro, SKINNY_ROWS);
+  }
+  if (shared && !paired) {
     // shared expert, its sigmoid gate applied to H inside the GEMM: Ys = sigmoid(z) * Shared(x).  With the fused
     // combine its output initialises the per-token accumulator the routed experts then add to.
     c2r_expert_opts o{};
@@ -227,7 +243,7 @@ extern "C" int c2r_layer_fwd(const c2r_config* cfg, const c2r_layer_buffers* b, 
     C2R_TRY(ss.fork());
     C2R_TRY(c2r_grouped_swiglu_fwd(cfg, 1, cfg->I_s, cfg->N, b->X, b->s_counts, b->s_offsets, b->Ws13p, b->Ws2, b->ABs,
                                    b->Hs, fcomb ? (void*)b->Yacc : b->Ys, &o, b->status, ss.work()));
-  } else if (fcomb) {
+  } else if (!shared && fcomb) {
     C2R_CUDA(cudaMemsetAsync(b->Yacc, 0, sizeof(float) * (size_t)cfg->N * cfg->d, as_stream(stream)));
   }
   // routing leaves the dispatch's per-block histogram in the workspace; the dispatch also spreads the weights
@@ -244,8 +260,11 @@ extern "C" int c2r_layer_fwd(const c2r_config* cfg, const c2r_layer_buffers* b, 
     o.token_acc = b->Yacc; o.slot_of_row = b->slot_of_row;
     C2R_TRY(ss.join());  // the accumulator holds the shared expert's term before the routed rows are added
   }
-  C2R_TRY(c2r_grouped_swiglu_fwd(cfg, cfg->E, cfg->I, R, gfused ? nullptr : b->Xp, b->counts, b->offsets, b->W13p, b->W2,
-                                 b->AB, b->H, fcomb ? nullptr : b->Yp, &o, b->status, stream));
+  if (paired)
+    C2R_TRY(skinny_swiglu_fwd(cfg, calls, 2, as_stream(stream)));
+  else
+    C2R_TRY(c2r_grouped_swiglu_fwd(cfg, cfg->E, cfg->I, R, gfused ? nullptr : b->Xp, b->counts, b->offsets, b->W13p, b->W2,
+                                   b->AB, b->H, fcomb ? nullptr : b->Yp, &o, b->status, stream));
   if (!fcomb) C2R_TRY(ss.join());
   // the weights are already inside Yp and Ys: a plain sum over the token's K rows plus the shared term
   // (fused combine: the sum is complete, what is left is the conversion to the storage type)

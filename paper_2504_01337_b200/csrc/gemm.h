@@ -78,6 +78,15 @@ enum { TC_EPI_SWIGLU_FWD = 0, TC_EPI_F32 = 1, TC_EPI_SWIGLU_BWD = 2, TC_EPI_WGRA
 bool tc_supported(const c2r_config* cfg, int nE, int I, int64_t R);
 int tc_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
 int tc_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
+// Weight-streaming forward for a handful of rows per expert (bf16, nothing kept for a backward pass).
+// The line: with the routed experts' rows spread evenly, up to 48 rows per expert (Qwen-MoE shape, us, pair tiles against
+// this: 237 / 183 at 4 rows, 238 / 202 at 34, 238 / 226 at 68; LLaMA-MoE shape 105 / 95 at 32, 105 / 107 at 64; 12 experts of
+// 512: 36 / 34 at 43, 36 / 44 at 85).  A dense group that rides along with the routed ones may have 128 rows: the
+// launches it saves and the SMs it fills are worth more than its own loss (Qwen shape, 128 tokens, whole forward 382 / 319).
+constexpr int SKINNY_ROWS = 48, SKINNY_ROWS_PAIRED = 128;
+bool skinny_supported(const c2r_config* cfg, const SwigluCall& a, int max_rows);
+// One or two such calls in one launch per product (the routed experts and the shared expert).
+int skinny_swiglu_fwd(const c2r_config* cfg, const SwigluCall* calls, int n, cudaStream_t s);
 // Rows of the partial-dot buffer the backward call writes for this shape (depends on which kernel serves it).
 int swiglu_qparts(const c2r_config* cfg, int nE, int I, int64_t R);
 
