@@ -30,7 +30,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[GT_STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[2 * GT_STAGES]), tempty0 = smem_u32(&bars[2 * GT_STAGES + 2]);
   if (threadIdx.x == 0) {
@@ -48,7 +48,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = tmem_slot;
+  const uint32_t tmem_base = warp_uniform(tmem_slot);
   volatile int* abort_flag = &s_abort;
 
   const int tiles = (N + BM - 1) / BM;
