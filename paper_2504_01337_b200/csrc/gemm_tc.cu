@@ -91,7 +91,9 @@ __device__ __forceinline__ bool decode_tile(const TcParams& p, const int* s_off,
     e_hint = e;
     ti.expert = warp_uniform(e);
     ti.m0 = warp_uniform(s_off[e] + TILE_M * (mp - s_pt[e]));
-    ti.m_end = warp_uniform(min(p.R, s_off[e] + (s_cnt[e] + BM - 1) / BM * BM));
+    // the rows that close an expert's 128-aligned segment are written (as zeros) where a backward pass contracts over them;
+    // nothing reads them in the fp32 results
+    ti.m_end = warp_uniform(min(p.R, s_off[e] + (p.epi == TC_EPI_F32 ? s_cnt[e] : (s_cnt[e] + BM - 1) / BM * BM)));
     ti.kblocks = (p.K + BK - 1) / BK;
     ti.krow0 = 0;
     return true;
