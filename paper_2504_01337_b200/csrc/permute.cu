@@ -63,6 +63,25 @@ __device__ __forceinline__ void layout_order(const int32_t* __restrict__ expert_
   __syncthreads();
 }
 
+// Segment offsets in layout order, by the first warp: lane l owns layout positions 2l and 2l + 1.  off[e] = start of expert e,
+// off[E] = end of the layout.  (One thread walking 60 experts took about 3 us of every dispatch.)
+__device__ __forceinline__ void segment_offsets(const int* s_by_rank, const int* s_total, int E, int row_align, int* off) {
+  if (threadIdx.x >= 32) return;
+  const int l = threadIdx.x;
+  const int e0 = 2 * l < E ? s_by_rank[2 * l] : -1, e1 = 2 * l + 1 < E ? s_by_rank[2 * l + 1] : -1;
+  const int v0 = e0 >= 0 ? (s_total[e0] + row_align - 1) / row_align * row_align : 0;
+  const int v1 = e1 >= 0 ? (s_total[e1] + row_align - 1) / row_align * row_align : 0;
+  int incl = v0 + v1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (l >= o) incl += x;
+  }
+  if (e0 >= 0) off[e0] = incl - v0 - v1;
+  if (e1 >= 0) off[e1] = incl - v1;
+  if (l == 31) off[E] = incl;
+}
+
 __global__ void __launch_bounds__(PERM_THREADS) perm_hist_kernel(const int32_t* __restrict__ idx, long long NK, int E,
                                                                  int slots_per_block, int32_t* __restrict__ block_counts,
                                                                  int32_t* __restrict__ status, int skip_negative) {
@@ -108,16 +127,8 @@ __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ b
     if (lane == 0) s_counts[e] = running;
   }
   layout_order(expert_rank, E, s_by_rank, &s_bad);
-  if (threadIdx.x == 0) {
-    int cursor = 0;
-    for (int r = 0; r < E; ++r) {
-      const int e = s_by_rank[r];
-      offsets[e] = cursor;
-      cursor += (s_counts[e] + row_align - 1) / row_align * row_align;
-    }
-    offsets[E] = cursor;
-    if (s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
-  }
+  segment_offsets(s_by_rank, s_counts, E, row_align, offsets);
+  if (threadIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
   if (threadIdx.x < E) counts[threadIdx.x] = s_counts[threadIdx.x];
 }
 
@@ -216,16 +227,8 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
     s_total[e] = total;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int cursor = 0;
-    for (int r = 0; r < E; ++r) {
-      const int e = s_by_rank[r];
-      s_off[e] = cursor;
-      cursor += (s_total[e] + row_align - 1) / row_align * row_align;
-    }
-    s_off[E] = cursor;
-    if (blockIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
-  }
+  segment_offsets(s_by_rank, s_total, E, row_align, s_off);
+  if (threadIdx.x == 0 && blockIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
   int flags = 0;
   const int e_mine = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, 0);
   __syncthreads();
@@ -235,47 +238,56 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
       if (e < E) counts[e] = s_total[e];
     }
   }
-  // rows without a slot: expert x's padding is written by block x mod gridDim.x, the tail by the last block
-  for (int x = blockIdx.x; x < E; x += gridDim.x) {
-    const int r0 = s_off[x] + s_total[x], r1 = s_off[x] + (s_total[x] + row_align - 1) / row_align * row_align;
-    for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
+  // rows without a slot: the padding that closes each segment and the rows past the layout, all blocks together
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < (long long)E * row_align; i += stride) {
+    const int x = (int)(i / row_align), r = s_off[x] + s_total[x] + (int)(i - (long long)x * row_align);
+    if (r < s_off[x] + (s_total[x] + row_align - 1) / row_align * row_align) {
       slot_of_row[r] = -1;
       if (w_row != nullptr) w_row[r] = 0.f;
     }
   }
-  if (blockIdx.x == gridDim.x - 1) {
-    for (long long r = s_off[E] + threadIdx.x; r < R; r += blockDim.x) {
-      slot_of_row[r] = -1;
-      if (w_row != nullptr) w_row[r] = 0.f;
-    }
+  for (long long r = s_off[E] + first; r < R; r += stride) {
+    slot_of_row[r] = -1;
+    if (w_row != nullptr) w_row[r] = 0.f;
   }
   for (int e = threadIdx.x; e < E; e += blockDim.x) s_start[e] += s_off[e];
   __syncthreads();
   rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, w, w_row);
 }
 
-// Row gather, one warp per token: the token's row is read once and written to its K rows.  Blocks past the
-// token blocks zero the padding rows that close each expert's aligned segment (block j: expert j).
+// Warps over which a token's row is spread where there are few tokens: enough for 32 warps per SM, each with at least one
+// 16-byte chunk per lane.  With a warp per token, 1021 tokens of d = 4096 left most of the chip idle (combine 38 us, row
+// gather 20 us) and a single token took 23 us in the combine, 16 loads one after another.
+inline int row_parts(long long tokens, int chunks_per_warp) {
+  const long long want = (148 * 32 + tokens - 1) / (tokens > 0 ? tokens : 1);
+  return (int)(want < 1 ? 1 : want > chunks_per_warp ? chunks_per_warp : want);
+}
+
+// Row gather: a token's row is read once and written to its K rows by `parts` warps.  Blocks past the token blocks zero the
+// padding rows that close each expert's aligned segment (PAD_BLOCKS blocks per expert).
+constexpr int PAD_BLOCKS = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__ X,
                                                            const int32_t* __restrict__ row_of_slot, T* __restrict__ Xp,
                                                            int N, int d, int K, const int32_t* __restrict__ counts,
                                                            const int32_t* __restrict__ offsets, int token_blocks,
-                                                           int row_align) {
+                                                           int row_align, int parts) {
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= token_blocks) {
-    const int e = blockIdx.x - token_blocks;
+    const int e = (blockIdx.x - token_blocks) / PAD_BLOCKS, sub = (blockIdx.x - token_blocks) % PAD_BLOCKS;
     const int n = counts[e];
     const int r0 = offsets[e] + n, r1 = offsets[e] + (n + row_align - 1) / row_align * row_align;
     V zero;
     float zf[V::N] = {};
     zero.from_float(zf);
-    for (int r = r0 + (threadIdx.x >> 5); r < r1; r += blockDim.x >> 5)
+    for (int r = r0 + sub * (blockDim.x >> 5) + (threadIdx.x >> 5); r < r1; r += PAD_BLOCKS * (blockDim.x >> 5))
       for (int c = lane; c < d / V::N; c += 32) zero.store(Xp + (size_t)r * d + (size_t)c * V::N);
     return;
   }
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int t = (int)(wid / parts), part = (int)(wid - (long long)t * parts);
   if (t >= N) return;  // warp-uniform
   const int my_row = (lane < K) ? row_of_slot[(size_t)t * K + lane] : 0;
   int rows[8];
@@ -283,18 +295,19 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__
   for (int k = 0; k < 8; ++k) rows[k] = __shfl_sync(0xffffffffu, my_row, k);
   const int chunks = d / V::N;
   const T* src = X + (size_t)t * d;
-  for (int c0 = lane; c0 < chunks; c0 += 32 * 4) {
+  const int step = 32 * parts;  // the part's chunks: every parts-th group of 32
+  for (int c0 = 32 * part + lane; c0 < chunks; c0 += step * 4) {
     V v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (c0 + 32 * u < chunks) v[u].load(src + (size_t)(c0 + 32 * u) * V::N);
+      if (c0 + step * u < chunks) v[u].load(src + (size_t)(c0 + step * u) * V::N);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (k >= K) break;
       T* dst = Xp + (size_t)rows[k] * d;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (c0 + 32 * u < chunks) v[u].store(dst + (size_t)(c0 + 32 * u) * V::N);
+        if (c0 + step * u < chunks) v[u].store(dst + (size_t)(c0 + step * u) * V::N);
     }
   }
 }
@@ -339,17 +352,18 @@ __device__ __forceinline__ void load_as_float(const S* p, float* f) {
 //          + sum_k dl[t,k] * Wg[idx[t,k],:] + dz[t] * wsg[:] (gate terms, optional)
 //          + out[t,:] if accumulate.
 // src == NULL: no such term (the producer already added its rows into extra).  src / extra are the fp32 partial results of the expert GEMMs; out has the storage type.
-// One warp per token, fp32 accumulation in k order.  Serves the combine and the gradient un-permute.
+// `parts` warps per token, fp32 accumulation in k order.  Serves the combine and the gradient un-permute.
 template <typename T>
 __global__ void __launch_bounds__(256) gather_sum_kernel(const float* __restrict__ src, const int32_t* __restrict__ rows_g,
                                                          const float* __restrict__ coef, const float* __restrict__ extra,
                                                          const float* __restrict__ z, const int32_t* __restrict__ idx,
                                                          const float* __restrict__ dl, const T* __restrict__ Wg,
                                                          const float* __restrict__ dz, const T* __restrict__ wsg,
-                                                         T* __restrict__ out, int accumulate, int N, int d, int K) {
+                                                         T* __restrict__ out, int accumulate, int N, int d, int K, int parts) {
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int t = (int)(wid / parts), part = (int)(wid - (long long)t * parts);
   if (t >= N) return;  // warp-uniform
   int my_row = 0, my_idx = 0;
   float my_coef = 1.f, my_dl = 0.f;
@@ -370,7 +384,7 @@ __global__ void __launch_bounds__(256) gather_sum_kernel(const float* __restrict
   const float ecoef = (extra && z) ? 1.0f / (1.0f + expf(-z[t])) : 1.0f;
   const float dzt = (dz && wsg) ? dz[t] : 0.f;
   const int chunks = d / V::N;
-  for (int c = lane; c < chunks; c += 32) {
+  for (int c = 32 * part + lane; c < chunks; c += 32 * parts) {
     const size_t col = (size_t)c * V::N;
     float acc[V::N];
 #pragma unroll
@@ -677,6 +691,20 @@ size_t gate_bwd_ws_bytes(const c2r_config* cfg) {
   return simt > tc ? simt : tc;
 }
 
+// The row gather, plus the blocks that zero the padding rows closing the aligned segments.
+template <typename T>
+static int permute_rows_launch(const c2r_config* cfg, const T* X, const int32_t* row_of_slot, const int32_t* counts,
+                               const int32_t* offsets, T* Xp, cudaStream_t s) {
+  const int parts = row_parts(cfg->N, (cfg->d / Vec16<T>::N + 31) / 32);
+  const int token_blocks = (int)(((long long)cfg->N * parts + 7) / 8);
+  const int pad_blocks = cfg->row_align > 1 ? cfg->E * PAD_BLOCKS : 0;
+  if (token_blocks + pad_blocks == 0) return C2R_OK;
+  permute_rows_kernel<T><<<token_blocks + pad_blocks, 256, 0, s>>>(X, row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts, offsets,
+                                                                token_blocks, cfg->row_align, parts);
+  C2R_LAUNCH_CHECK();
+  return C2R_OK;
+}
+
 // have_hist: block_counts already holds the per-block expert counts of idx in this blocking (the routing
 // kernel wrote them), so the histogram launch is skipped.  w / w_row (both or neither): see rank_and_write.
 template <typename T>
@@ -709,14 +737,8 @@ int permute_impl(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
     }
   }
   if (X != nullptr) {
-    // the gather, plus one block per expert that zeroes the padding rows closing its aligned segment
-    const int token_blocks = (cfg->N + 7) / 8;
-    const int pad_blocks = cfg->row_align > 1 ? cfg->E : 0;
-    if (token_blocks + pad_blocks > 0) {
-      permute_rows_kernel<T><<<token_blocks + pad_blocks, 256, 0, s>>>(X, row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts,
-                                                                    offsets, token_blocks, cfg->row_align);
-      C2R_LAUNCH_CHECK();
-    }
+    int rc = permute_rows_launch<T>(cfg, X, row_of_slot, counts, offsets, Xp, s);
+    if (rc) return rc;
   }
   return C2R_OK;
 }
@@ -754,20 +776,9 @@ extern "C" int c2r_permute_rows(const c2r_config* cfg, const void* X, const int3
   int rc = check_config(cfg);
   if (rc) return rc;
   C2R_REQUIRE(X && row_of_slot && counts && offsets && Xp, C2R_ERR_INVALID_ARG);
-  const int token_blocks = (cfg->N + 7) / 8;
-  const int pad_blocks = cfg->row_align > 1 ? cfg->E : 0;
-  if (token_blocks + pad_blocks == 0) return C2R_OK;
-  cudaStream_t s = as_stream(stream);
   if (cfg->dtype == C2R_BF16)
-    permute_rows_kernel<__nv_bfloat16><<<token_blocks + pad_blocks, 256, 0, s>>>(
-        (const __nv_bfloat16*)X, row_of_slot, (__nv_bfloat16*)Xp, cfg->N, cfg->d, cfg->K, counts, offsets, token_blocks,
-        cfg->row_align);
-  else
-    permute_rows_kernel<float><<<token_blocks + pad_blocks, 256, 0, s>>>((const float*)X, row_of_slot, (float*)Xp, cfg->N,
-                                                                         cfg->d, cfg->K, counts, offsets, token_blocks,
-                                                                         cfg->row_align);
-  C2R_LAUNCH_CHECK();
-  return C2R_OK;
+    return permute_rows_launch(cfg, (const __nv_bfloat16*)X, row_of_slot, counts, offsets, (__nv_bfloat16*)Xp, as_stream(stream));
+  return permute_rows_launch(cfg, (const float*)X, row_of_slot, counts, offsets, (float*)Xp, as_stream(stream));
 }
 
 template <typename T>
@@ -775,9 +786,11 @@ static int gather_sum_launch(const c2r_config* cfg, const void* src, const int32
                              const void* extra, const float* z, const int32_t* idx, const float* dl, const void* Wg,
                              const float* dz, const void* wsg, void* out, int accumulate, cudaStream_t s) {
   if (cfg->N == 0) return C2R_OK;
-  gather_sum_kernel<T><<<(cfg->N + 7) / 8, 256, 0, s>>>((const float*)src, rows, coef, (const float*)extra, z, idx, dl,
-                                                        (const T*)Wg, dz, (const T*)wsg, (T*)out, accumulate, cfg->N,
-                                                        cfg->d, cfg->K);
+  const int parts = row_parts(cfg->N, (cfg->d / Vec16<T>::N + 31) / 32);
+  const long long warps = (long long)cfg->N * parts;
+  gather_sum_kernel<T><<<(unsigned)((warps + 7) / 8), 256, 0, s>>>((const float*)src, rows, coef, (const float*)extra, z, idx, dl,
+                                                                   (const T*)Wg, dz, (const T*)wsg, (T*)out, accumulate, cfg->N,
+                                                                   cfg->d, cfg->K, parts);
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
