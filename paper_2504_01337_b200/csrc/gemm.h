@@ -34,6 +34,11 @@ struct SimtGemm {
   const int32_t* offsets;
   long long sam, sak, sbn, sbk, sB, sC, ldc;
   int mode, epi, Mdim, Ndim, Kdim, I, accumulate;
+  // counts == NULL: one group of Mdim rows.  B_last / C_last (may be NULL): row Ndim - 1 of B comes from there, and column
+  // Ndim - 1 of C goes there ([m], SIMT_EPI_STORE).  n_groups and vec are filled in by the launch.
+  const void* B_last;
+  void* C_last;
+  int n_groups, vec;
 };
 
 // One grouped SwiGLU evaluation (forward or backward); members a direction does not use stay NULL.
@@ -71,6 +76,8 @@ template <typename T>
 int simt_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
 template <typename T>
 int simt_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
+template <typename T>
+int simt_gate_logits(const c2r_config* cfg, const void* X, const void* Wg, const void* wsg, float* L, float* z, cudaStream_t s);
 
 // Tensor-core (tcgen05) path, bf16 only.
 enum { TC_ROWS = 0, TC_WGRAD = 1 };

@@ -41,88 +41,208 @@ __global__ void pack_kernel(const T* __restrict__ W1, const T* __restrict__ W3, 
   }
 }
 
-constexpr int ST = 64;  // tile M = N
-constexpr int SK = 16;  // tile K
+constexpr int SIMT_THREADS = 256;
+
+// Four consecutive elements as floats; `vec`: base pointers and strides are known to be aligned for one vector load.
+__device__ __forceinline__ float4 load4(const float* p, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p, bool vec) {
+  if (vec) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+  }
+  return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+}
+
+// Operand tiles are [SK][W] floats.  The 4-wide column groups of row k are permuted by ^ ((k >> 2) & 7): a thread that
+// loaded four consecutive k of one row stores them down a column without bank conflicts, and four consecutive columns
+// still lie in 16 aligned bytes.
+template <int W>
+__device__ __forceinline__ int tile_at(int k, int m) {
+  return k * W + ((((m >> 2) ^ ((k >> 2) & 7)) & (W / 4 - 1)) << 2) + (m & 3);
+}
+
+// A W x SK operand tile on its way from global memory to shared memory, held in registers while the previous tile is used.
+template <typename T, int W, int SK>
+struct TileLoad {
+  static constexpr int V = W * SK / 4;                                       // four-element pieces
+  static constexpr int PER = (V + SIMT_THREADS - 1) / SIMT_THREADS;
+  float4 v[PER];
+  // row(m): address of element (m, 0); element (m, k) lies k * sk (and m * sm for sk != 1) further
+  template <typename Row>
+  __device__ __forceinline__ void load(Row row, long long sk, int m_left, int k0, int Kd, bool vec) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int x = threadIdx.x + i * SIMT_THREADS;
+      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (V % SIMT_THREADS != 0 && x >= V) continue;
+      if (sk == 1) {  // contraction contiguous
+        const int k = 4 * (x % (SK / 4)), m = x / (SK / 4);
+        if (m < m_left && k0 + k < Kd) v[i] = load4(row(m) + k0 + k, vec);
+      } else {        // rows contiguous
+        const int m = 4 * (x % (W / 4)), k = x / (W / 4);
+        if (m < m_left && k0 + k < Kd) v[i] = load4(row(m) + (k0 + k) * sk, vec);
+      }
+    }
+  }
+  __device__ __forceinline__ void store(float* tile, long long sk) const {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int x = threadIdx.x + i * SIMT_THREADS;
+      if (V % SIMT_THREADS != 0 && x >= V) continue;
+      if (sk == 1) {
+        const int k = 4 * (x % (SK / 4)), m = x / (SK / 4);
+        tile[tile_at<W>(k, m)] = v[i].x;
+        tile[tile_at<W>(k + 1, m)] = v[i].y;
+        tile[tile_at<W>(k + 2, m)] = v[i].z;
+        tile[tile_at<W>(k + 3, m)] = v[i].w;
+      } else {
+        const int m = 4 * (x % (W / 4)), k = x / (W / 4);
+        *reinterpret_cast<float4*>(&tile[tile_at<W>(k, m)]) = v[i];
+      }
+    }
+  }
+};
 
 // C_g(m,n) = sum_k A_g(m,k) B_g(n,k) with arbitrary strides; see SimtGemm for the two modes.
-template <typename T, typename TC>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(SimtGemm g) {
-  __shared__ float sa[SK][ST + 4];
-  __shared__ float sb[SK][ST + 4];
-  __shared__ float sb2[SK][ST + 4];  // up-projection tile of the fused SwiGLU forward
-  __shared__ float sred[ST][17];     // per-row partial dots of the SwiGLU backward, one column per thread column
-  const bool dual = g.epi == SIMT_EPI_SWIGLU_FWD;
-  const int grp = blockIdx.z;
-  int M, Kd;
-  long long a_off, b_off, c_off;
-  const int cnt = g.counts[grp], r0 = g.offsets[grp];
-  if (g.mode == SIMT_ROWS) {
-    M = cnt; Kd = g.Kdim;
-    a_off = (long long)r0 * g.sam; b_off = (long long)grp * g.sB; c_off = (long long)r0 * g.ldc;
+//
+// A block computes TM x TN outputs; (TM / 4)(TN / 4) threads hold a 4 x 4 share each, and where that is fewer than the
+// block has, groups of threads split every k-tile and their sums are added in group order.  The next k-tile is loaded into
+// registers while the current one is used (two shared-memory buffers, one barrier per tile).  The small configurations
+// this serves are bound by latency: a chain of 16-deep tiles, each waiting for its own loads, took 80 us for K = 256
+// where this takes 16.5 (1024 rows, 128 dual columns; weight gradients of 375 rows 158 -> 28; whole fp32 training step of
+// 1500 tokens 502 -> 206).  64 x 64 tiles where they fill the chip, else 32-wide ones.
+// Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
+// (SIMT_WGRAD).
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL>
+__global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
+  constexpr int GROUP = (TM / 4) * (TN / 4), G = SIMT_THREADS / GROUP;  // threads per group, groups
+  constexpr int MR = G == 1 ? 4 : TM * TN / (4 * SIMT_THREADS);         // output rows a thread finishes, four columns each
+  constexpr int TILES = 2 * SK * (TM + TN * (DUAL ? 2 : 1)), RED = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4);
+  __shared__ __align__(16) float smem[TILES > RED ? TILES : RED];
+  __shared__ float sred[TM][TN / 4 + 1];  // per-row partial dots of the SwiGLU backward, one column per thread column
+  const int tid = threadIdx.x, lane = tid & 31;
+  int grp, m0, M, Kd;
+  long long a_off, b_off, c_off, r0 = 0;
+  if (g.counts == nullptr) {  // one group whose size the host knows
+    grp = 0; m0 = blockIdx.x * TM; M = g.Mdim; Kd = g.Kdim;
+    a_off = b_off = c_off = 0;
+  } else if (g.mode == SIMT_ROWS) {
+    // row tiles are numbered through the groups; every warp finds the group of tile blockIdx.x by a scan over the counts
+    const int n0 = lane < g.n_groups ? (max(g.counts[lane], 0) + TM - 1) / TM : 0;
+    const int n1 = lane + 32 < g.n_groups ? (max(g.counts[lane + 32], 0) + TM - 1) / TM : 0;
+    int s0 = n0, s1 = n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x0 = __shfl_up_sync(0xffffffffu, s0, o), x1 = __shfl_up_sync(0xffffffffu, s1, o);
+      if (lane >= o) { s0 += x0; s1 += x1; }
+    }
+    s1 += __shfl_sync(0xffffffffu, s0, 31);
+    const int y = blockIdx.x;
+    const uint32_t in0 = __ballot_sync(0xffffffffu, y >= s0 - n0 && y < s0), in1 = __ballot_sync(0xffffffffu, y >= s1 - n1 && y < s1);
+    if (!(in0 | in1)) return;
+    const int src = in0 ? __ffs(in0) - 1 : __ffs(in1) - 1;
+    grp = in0 ? src : 32 + src;
+    m0 = (y - __shfl_sync(0xffffffffu, in0 ? s0 - n0 : s1 - n1, src)) * TM;
+    M = g.counts[grp]; r0 = g.offsets[grp]; Kd = g.Kdim;
+    a_off = r0 * g.sam; b_off = (long long)grp * g.sB; c_off = r0 * g.ldc;
   } else {
-    M = g.Mdim; Kd = cnt;
-    a_off = (long long)r0 * g.sak; b_off = (long long)r0 * g.sbk; c_off = (long long)grp * g.sC;
+    grp = blockIdx.z; m0 = blockIdx.x * TM; M = g.Mdim;
+    Kd = g.counts[grp]; r0 = g.offsets[grp];
+    a_off = r0 * g.sak; b_off = r0 * g.sbk; c_off = (long long)grp * g.sC;
   }
-  const int m0 = blockIdx.y * ST, n0 = blockIdx.x * ST;
+  const int n0 = blockIdx.y * TN;
   if (m0 >= M || n0 >= g.Ndim) return;
-  const T* A = (const T*)g.A + a_off;
+  const T* A = (const T*)g.A + a_off + (long long)m0 * g.sam;
   const T* B = (const T*)g.B + b_off;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  float acc[4][4] = {};
-  float acc2[4][4] = {};
-  for (int k0 = 0; k0 < Kd; k0 += SK) {
-    for (int i = tid; i < ST * SK; i += 256) {
-      int m, k;
-      if (g.sak == 1) { k = i % SK; m = i / SK; } else { m = i % ST; k = i / ST; }
-      float v = 0.f;
-      if (m0 + m < M && k0 + k < Kd) v = to_f32(A[(long long)(m0 + m) * g.sam + (long long)(k0 + k) * g.sak]);
-      sa[k][m] = v;
-    }
-    for (int i = tid; i < ST * SK; i += 256) {
-      int n, k;
-      if (g.sbk == 1) { k = i % SK; n = i / SK; } else { n = i % ST; k = i / ST; }
-      float v = 0.f, v2 = 0.f;
-      if (n0 + n < g.Ndim && k0 + k < Kd) {
-        if (!dual) {
-          v = to_f32(B[(long long)(n0 + n) * g.sbn + (long long)(k0 + k) * g.sbk]);
-        } else {  // column n of H pairs packed rows pg (gate) and pu (up) of W13p
-          const int pg = pack_col(n0 + n, g.I), pu = pg + pack_width(n0 + n, g.I);
-          v = to_f32(B[(long long)pg * g.sbn + (long long)(k0 + k) * g.sbk]);
-          v2 = to_f32(B[(long long)pu * g.sbn + (long long)(k0 + k) * g.sbk]);
-        }
-      }
-      sb[k][n] = v;
-      if (dual) sb2[k][n] = v2;
-    }
+  const bool vec = g.vec != 0;
+  auto rowA = [&](int m) { return A + (long long)m * g.sam; };
+  auto rowB = [&](int n) {
+    if (g.B_last != nullptr && n0 + n == g.Ndim - 1) return (const T*)g.B_last;
+    return B + (long long)(DUAL ? pack_col(n0 + n, g.I) : n0 + n) * g.sbn;
+  };
+  auto rowB2 = [&](int n) { return B + (long long)(pack_col(n0 + n, g.I) + pack_width(n0 + n, g.I)) * g.sbn; };
+
+  const int grp_k = tid / GROUP, tg = tid % GROUP;
+  const int tx = tg % (TN / 4), ty = tg / (TN / 4);
+  float acc[4][4] = {}, acc2[DUAL ? 4 : 1][4] = {};
+  TileLoad<T, TM, SK> la;
+  TileLoad<T, TN, SK> lb, lb2;
+  auto fetch = [&](int k0) {
+    la.load(rowA, g.sak, M - m0, k0, Kd, vec);
+    lb.load(rowB, g.sbk, g.Ndim - n0, k0, Kd, vec);
+    if (DUAL) lb2.load(rowB2, g.sbk, g.Ndim - n0, k0, Kd, vec);
+  };
+  constexpr int BUF = SK * (TM + TN * (DUAL ? 2 : 1));
+  fetch(0);
+  for (int k0 = 0, buf = 0; k0 < Kd; k0 += SK, buf ^= 1) {
+    float* sa = smem + buf * BUF;
+    float* sb = sa + SK * TM;
+    float* sb2 = sb + SK * TN;
+    la.store(sa, g.sak);
+    lb.store(sb, g.sbk);
+    if (DUAL) lb2.store(sb2, g.sbk);
     __syncthreads();
+    if (k0 + SK < Kd) fetch(k0 + SK);
 #pragma unroll
-    for (int k = 0; k < SK; ++k) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { av[i] = sa[k][ty * 4 + i]; bv[i] = sb[k][tx * 4 + i]; }
+    for (int kk = 0; kk < SK / G; ++kk) {
+      const int k = grp_k * (SK / G) + kk;
+      const float4 av = *reinterpret_cast<const float4*>(&sa[tile_at<TM>(k, 4 * ty)]);
+      const float4 bv = *reinterpret_cast<const float4*>(&sb[tile_at<TN>(k, 4 * tx)]);
+      const float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-      if (dual) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) bv[i] = sb2[k][tx * 4 + i];
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
+      if (DUAL) {
+        const float4 cv = *reinterpret_cast<const float4*>(&sb2[tile_at<TN>(k, 4 * tx)]);
+        const float cr[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(av[i], bv[j], acc2[i][j]);
+          for (int j = 0; j < 4; ++j) acc2[DUAL ? i : 0][j] = fmaf(ar[i], cr[j], acc2[DUAL ? i : 0][j]);
       }
     }
+  }
+  // this thread's outputs: rows m_of(i), columns nc .. nc + 3
+  const int nc = n0 + 4 * (G == 1 ? tx : tid % (TN / 4));
+  auto m_of = [&](int i) { return G == 1 ? 4 * ty + i : tid / (TN / 4) + i * (SIMT_THREADS / (TN / 4)); };
+  if (G > 1) {  // add the groups' partial sums, in group order
+    constexpr int P = TN + 4;
     __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      *reinterpret_cast<float4*>(&smem[(grp_k * TM + 4 * ty + i) * P + 4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      if (DUAL)
+        *reinterpret_cast<float4*>(&smem[((G + grp_k) * TM + 4 * ty + i) * P + 4 * tx]) =
+            make_float4(acc2[DUAL ? i : 0][0], acc2[DUAL ? i : 0][1], acc2[DUAL ? i : 0][2], acc2[DUAL ? i : 0][3]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < MR; ++i) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float v = 0.f, v2 = 0.f;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+          v += smem[(q * TM + m_of(i)) * P + nc - n0 + j];
+          if (DUAL) v2 += smem[((G + q) * TM + m_of(i)) * P + nc - n0 + j];
+        }
+        acc[i][j] = v;
+        if (DUAL) acc2[DUAL ? i : 0][j] = v2;
+      }
+    }
   }
   TC* C = (TC*)g.C + c_off;
   const bool want_q = g.epi == SIMT_EPI_SWIGLU_BWD && g.qpart != nullptr;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
+  for (int i = 0; i < MR; ++i) {
+    const int lm = m_of(i), m = m0 + lm;
     float qrow = 0.f;
-    if (want_q) sred[ty * 4 + i][tx] = 0.f;
+    if (want_q) sred[lm][(nc - n0) / 4] = 0.f;
     if (m >= M) continue;
     float sc = 1.f;  // per-row scale of H (SwiGLU forms)
     if (g.scale_kind != 0 && g.row_scale != nullptr) {
@@ -131,22 +251,14 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(SimtGemm g) {
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
+      const int n = nc + j;
       if (n >= g.Ndim) continue;
       float v = acc[i][j];
-      if (g.epi == SIMT_EPI_STORE && g.token_acc != nullptr) {
-        // fused combine: the row is added into its token's accumulator (fp32 atomics, order not fixed)
-        const int sl = g.slot_of_row[r0 + m];
-        if (sl >= 0) atomicAdd(g.token_acc + (long long)(sl / g.slots_per_token) * g.ldc + n, v);
-      } else if (g.epi == SIMT_EPI_STORE) {
-        TC* o = C + (long long)m * g.ldc + n;
-        if (g.accumulate) v += to_f32(*o);
-        *o = from_f32<TC>(v);
-      } else if (g.epi == SIMT_EPI_SWIGLU_FWD) {
+      if (DUAL) {
         // v = A[r,n], acc2 = B[r,n]: H = silu(A) * B; the backward pass needs only the two local
         // derivatives dH/dA = B silu'(A) and dH/dB = silu(A), which are what is kept (packed columns)
         const int pg = pack_col(n, g.I), pu = pg + pack_width(n, g.I);
-        const float b = acc2[i][j];
+        const float b = acc2[DUAL ? i : 0][j];
         const float sg = 1.0f / (1.0f + expf(-v));
         const float as = v * sg;
         if (g.C != nullptr) {  // inference: nothing is kept for a backward pass
@@ -155,6 +267,14 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(SimtGemm g) {
           sv[pu] = from_f32<T>(as);
         }
         ((T*)g.aux_out)[(long long)(r0 + m) * g.I + n] = from_f32<T>(sc * (as * b));
+      } else if (g.epi == SIMT_EPI_STORE && g.token_acc != nullptr) {
+        // fused combine: the row is added into its token's accumulator (fp32 atomics, order not fixed)
+        const int sl = g.slot_of_row[r0 + m];
+        if (sl >= 0) atomicAdd(g.token_acc + (long long)(sl / g.slots_per_token) * g.ldc + n, v);
+      } else if (g.epi == SIMT_EPI_STORE) {
+        TC* o = (g.C_last != nullptr && n == g.Ndim - 1) ? (TC*)g.C_last + m : C + (long long)m * g.ldc + n;
+        if (g.accumulate) v += to_f32(*o);
+        *o = from_f32<TC>(v);
       } else {  // SIMT_EPI_SWIGLU_BWD: v = dH[r, n]; dA = dH * (dH/dA), dB = dH * (dH/dB) at the packed columns
         const int pg = pack_col(n, g.I), pu = pg + pack_width(n, g.I);
         const T* sv = (const T*)g.aux + (long long)(r0 + m) * 2 * g.I;
@@ -164,32 +284,66 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(SimtGemm g) {
         if (want_q) qrow = fmaf(v, to_f32(((const T*)g.aux2)[(long long)(r0 + m) * g.I + n]), qrow);
       }
     }
-    if (want_q) sred[ty * 4 + i][tx] = qrow;
+    if (want_q) sred[lm][(nc - n0) / 4] = qrow;
   }
   if (want_q) {  // (uniform across the block) row dots <dH_r, H_r> over this block's 64 columns, in column order
     __syncthreads();
-    if (tid < ST && m0 + tid < M) {
+    if (tid < TM && m0 + tid < M) {
       float q = 0.f;
 #pragma unroll
-      for (int x = 0; x < 16; ++x) q += sred[tid][x];
-      g.qpart[(long long)blockIdx.x * g.R + r0 + m0 + tid] = q;
+      for (int x = 0; x < TN / 4; ++x) q += sred[tid][x];
+      g.qpart[(long long)blockIdx.y * g.R + r0 + m0 + tid] = q;
     }
   }
 }
 
-template <typename T, typename TC = T>
-int simt_launch(const SimtGemm& g, int n_groups, int max_m, cudaStream_t s) {
-  if (n_groups == 0 || max_m == 0 || g.Ndim == 0) return C2R_OK;
-  dim3 grid((g.Ndim + ST - 1) / ST, (max_m + ST - 1) / ST, n_groups);
-  simt_gemm_kernel<T, TC><<<grid, 256, 0, s>>>(g);
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL>
+static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
+  simt_gemm_kernel<T, TC, TM, TN, SK, DUAL><<<dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s>>>(g);
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
 
+// max_m: rows (SIMT_ROWS: of all groups together) or Mdim.
+template <typename T, typename TC = T>
+int simt_launch(SimtGemm g, int n_groups, int64_t max_m, cudaStream_t s) {
+  if (n_groups == 0 || max_m == 0 || g.Ndim == 0) return C2R_OK;
+  g.n_groups = n_groups;
+  const uintptr_t align = 4 * sizeof(T) - 1;
+  const uintptr_t bits = (uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last;
+  g.vec = (bits & align) == 0 && (g.sak == 1 ? g.sam : g.sak) % 4 == 0 && (g.sbk == 1 ? g.sbn : g.sbk) % 4 == 0 && g.sB % 4 == 0;
+  const bool rows = g.mode == SIMT_ROWS && g.counts != nullptr;
+  const int z = rows ? 1 : n_groups;
+  // SIMT_ROWS: whole tiles of all groups, and one more per group for its remainder
+  auto m_tiles = [&](int tm) { return (int)((max_m + tm - 1) / tm) + (rows ? n_groups : 0); };
+  const int64_t blocks64 = (int64_t)((max_m + 63) / 64) * ((g.Ndim + 63) / 64) * z;
+  const bool dual = g.epi == SIMT_EPI_SWIGLU_FWD;
+  if (blocks64 >= 2 * 148)
+    return dual ? simt_launch_tile<T, TC, 64, 64, 16, true>(g, m_tiles(64), z, s)
+                : simt_launch_tile<T, TC, 64, 64, 16, false>(g, m_tiles(64), z, s);
+  if (dual) return simt_launch_tile<T, TC, 32, 32, 32, true>(g, m_tiles(32), z, s);
+  // the backward's partial row dots cover 64 columns each
+  return g.epi == SIMT_EPI_SWIGLU_BWD ? simt_launch_tile<T, TC, 32, 64, 32, false>(g, m_tiles(32), z, s)
+                                      : simt_launch_tile<T, TC, 32, 32, 32, false>(g, m_tiles(32), z, s);
+}
+
+// Gate logits (Eq. 1) in fp32 arithmetic: L = X Wg^T and, as one more row of the other operand, z = X wsg.
+template <typename T>
+int simt_gate_logits(const c2r_config* cfg, const void* X, const void* Wg, const void* wsg, float* L, float* z, cudaStream_t s) {
+  SimtGemm g{};
+  g.mode = SIMT_ROWS; g.epi = SIMT_EPI_STORE;
+  g.A = X; g.sam = cfg->d; g.sak = 1; g.B = Wg; g.sbn = cfg->d; g.sbk = 1; g.B_last = wsg;
+  g.C = L; g.C_last = wsg ? z : nullptr; g.ldc = cfg->E;
+  g.Mdim = cfg->N; g.Ndim = cfg->E + (wsg ? 1 : 0); g.Kdim = cfg->d;
+  return simt_launch<T, float>(g, 1, cfg->N, s);
+}
+template int simt_gate_logits<float>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);
+template int simt_gate_logits<__nv_bfloat16>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);
+
 template <typename T>
 int simt_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) {
   const int d = cfg->d, I = a.I;
-  const int max_m = (int)a.R;
+  const int64_t max_m = a.R;
   SimtGemm g{};
   g.counts = a.counts; g.offsets = a.offsets; g.mode = SIMT_ROWS; g.I = I; g.R = a.R;
   // A = Xp W1^T, B = Xp W3^T in one pass over Xp; epilogue stores H = s silu(A) * B and the two local derivatives
@@ -210,7 +364,7 @@ int simt_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) 
 template <typename T>
 int simt_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) {
   const int d = cfg->d, I = a.I, nE = a.nE;
-  const int max_m = (int)a.R;
+  const int64_t max_m = a.R;
   SimtGemm g{};
   g.counts = a.counts; g.offsets = a.offsets; g.I = I; g.R = a.R;
   // dH = dYp W2  (epilogue turns it into dA, dB at the packed columns, and the row dots with H)

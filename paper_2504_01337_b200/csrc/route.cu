@@ -10,67 +10,6 @@ thread_local int g_last_cuda_error = 0;
 unsigned long long g_launch_count = 0;
 
 // ---------------------------------------------------------------------------------------------
-// Gate logits (Eq. 1): L = X Wg^T, z = X wsg.  CUDA-core kernel: a block owns TM tokens and all
-// E (+1) gate columns, streams d in chunks through shared memory; X is read from HBM once.
-// ---------------------------------------------------------------------------------------------
-constexpr int GL_TM = 32;   // tokens per block
-constexpr int GL_DK = 64;   // d-chunk
-constexpr int GL_COLS = 64; // gate columns held (E routed + optional shared gate)
-
-template <typename T>
-__global__ void __launch_bounds__(256) gate_logits_kernel(const T* __restrict__ X, const T* __restrict__ Wg,
-                                                          const T* __restrict__ wsg, float* __restrict__ L,
-                                                          float* __restrict__ z, int N, int d, int E) {
-  __shared__ float sx[GL_TM][GL_DK + 1];
-  __shared__ float sw[GL_COLS][GL_DK + 1];
-  const int tid = threadIdx.x;
-  const int t0 = blockIdx.x * GL_TM;
-  const int cols = E + (wsg != nullptr ? 1 : 0);
-  const int tx = tid & 15;  // column group: columns tx, tx+16, tx+32, tx+48
-  const int ty = tid >> 4;  // token group: tokens ty, ty+16
-  float acc[2][4] = {};
-  for (int k0 = 0; k0 < d; k0 += GL_DK) {
-    for (int i = tid; i < GL_TM * GL_DK; i += 256) {
-      int r = i / GL_DK, c = i % GL_DK;
-      int t = t0 + r;
-      sx[r][c] = (t < N && k0 + c < d) ? to_f32(X[(size_t)t * d + k0 + c]) : 0.f;
-    }
-    for (int i = tid; i < GL_COLS * GL_DK; i += 256) {
-      int r = i / GL_DK, c = i % GL_DK;
-      float v = 0.f;
-      if (k0 + c < d) {
-        if (r < E) v = to_f32(Wg[(size_t)r * d + k0 + c]);
-        else if (r == E && wsg != nullptr) v = to_f32(wsg[k0 + c]);
-      }
-      sw[r][c] = v;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < GL_DK; ++k) {
-      float xa = sx[ty][k], xb = sx[ty + 16][k];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float wv = sw[tx + 16 * j][k];
-        acc[0][j] = fmaf(xa, wv, acc[0][j]);
-        acc[1][j] = fmaf(xb, wv, acc[1][j]);
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    int t = t0 + ty + 16 * i;
-    if (t >= N) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int c = tx + 16 * j;
-      if (c < E) L[(size_t)t * E + c] = acc[i][j];
-      else if (c == E && c < cols) z[t] = acc[i][j];
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
 // Routing (Sec. 3.3 step 2).  One warp per token; lane l holds logits l and l+32.  K rounds of an
 // arg-max under the total order (value desc, index asc); after round 0 the candidate set
 // is intersected with the top-1 expert's collaborator mask.  A round is one warp-wide integer maximum over
@@ -368,19 +307,12 @@ int c2r::gate_logits_impl(const c2r_config* cfg, const void* X, const void* Wg, 
   if (rc) return rc;
   C2R_REQUIRE(X && Wg && L, C2R_ERR_INVALID_ARG);
   C2R_REQUIRE(!wsg || z, C2R_ERR_INVALID_ARG);
-  C2R_REQUIRE(cfg->E + (wsg ? 1 : 0) <= GL_COLS, C2R_ERR_UNSUPPORTED_SHAPE);
+  C2R_REQUIRE(cfg->E + (wsg ? 1 : 0) <= 64, C2R_ERR_UNSUPPORTED_SHAPE);
   if (cfg->N == 0) return C2R_OK;
   const bool aligned = (((uintptr_t)X | (uintptr_t)Wg | (uintptr_t)wsg | (uintptr_t)L) & 15u) == 0;
   if (aligned && gate_tc_supported(cfg)) return gate_tc_launch(cfg, X, Wg, wsg, L, z, status, as_stream(stream));
-  dim3 grid((cfg->N + GL_TM - 1) / GL_TM);
-  if (cfg->dtype == C2R_BF16)
-    gate_logits_kernel<__nv_bfloat16><<<grid, 256, 0, as_stream(stream)>>>(
-        (const __nv_bfloat16*)X, (const __nv_bfloat16*)Wg, (const __nv_bfloat16*)wsg, L, z, cfg->N, cfg->d, cfg->E);
-  else
-    gate_logits_kernel<float><<<grid, 256, 0, as_stream(stream)>>>((const float*)X, (const float*)Wg,
-                                                                   (const float*)wsg, L, z, cfg->N, cfg->d, cfg->E);
-  C2R_LAUNCH_CHECK();
-  return C2R_OK;
+  return cfg->dtype == C2R_BF16 ? simt_gate_logits<__nv_bfloat16>(cfg, X, Wg, wsg, L, z, as_stream(stream))
+                                : simt_gate_logits<float>(cfg, X, Wg, wsg, L, z, as_stream(stream));
 }
 
 extern "C" int c2r_gate_logits(const c2r_config* cfg, const void* X, const void* Wg, const void* wsg, float* L,
