@@ -7,11 +7,6 @@
 // 16 k-elements (N = 64 for the routed gate, N = 80 when the shared-expert gate's block rides along) into tensor
 // memory, and four warps write the fp32 accumulators out.  Waits are bounded like in the grouped
 // GEMM kernel.
-//
-// Few tokens are few tiles, and one CTA streams a tile at a small part of the chip's bandwidth: a cluster of 2, 4 or 8 CTAs
-// then splits the contraction of a tile, and each adds up a share of the tile's rows from the partial results in the
-// others' shared memory, in rank order (us, one CTA per tile against this: 13.3 / 8.6 for 1 token of d = 2048, 21.0 / 8.5 for
-// 1021 of d = 4096, 14.0 / 11.8 for 4096 of d = 2048).
 #include "gemm.h"
 #include "tc_common.cuh"
 
@@ -25,19 +20,10 @@ constexpr int GT_STAGE_BYTES = GT_X_BYTES + GT_W_BYTES + GT_S_BYTES;
 constexpr int GT_THREADS = 192;
 constexpr int GT_TMEM_COLS = 256;          // two accumulators of 128 columns (64 logits | 16 shared gate | unused)
 
-constexpr int GT_SPLIT_STAGES = 4;         // a split has few k-blocks, and two CTAs then share an SM
-constexpr int GT_PART_PITCH = 81;          // floats per row of a split's partial result (odd: no bank conflicts)
-
-__device__ __forceinline__ float ld_cluster(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-
 __global__ void __launch_bounds__(GT_THREADS, 1)
 gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_s, float* __restrict__ L, float* __restrict__ z, int N, int d,
-               int E, int has_shared, int splits, int stages, int32_t* __restrict__ status) {
+               int E, int has_shared, int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ uint64_t bars[2 * GT_STAGES + 4];
@@ -49,7 +35,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   const uint32_t tfull0 = smem_u32(&bars[2 * GT_STAGES]), tempty0 = smem_u32(&bars[2 * GT_STAGES + 2]);
   if (threadIdx.x == 0) {
     s_abort = 0;
-    for (int s = 0; s < stages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+    for (int s = 0; s < GT_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull0 + 8 * b, 1); mbar_init(tempty0 + 8 * b, 4); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -64,83 +50,68 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = warp_uniform(tmem_slot);
   volatile int* abort_flag = &s_abort;
-  float* part = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)));  // [128][GT_PART_PITCH], splits > 1
 
   const int tiles = (N + BM - 1) / BM;
-  const int rank = splits > 1 ? (int)cluster_ctarank() : 0;
   const int kblocks = (d + BK - 1) / BK;
-  const int kb0 = rank * kblocks / splits, kb1 = (rank + 1) * kblocks / splits;  // k-blocks of this split
-  const int tile0 = blockIdx.x / splits, tile_step = gridDim.x / splits;  // splits > 1: one tile per cluster
   const int n_mma = (E + 15) / 16 * 16;  // MMA-N of the routed gate
   const uint32_t tx_bytes = GT_X_BYTES + GT_W_BYTES + (has_shared ? GT_S_BYTES : 0);
 
   if (warp == 0) {
-    uint32_t stage = 0, phase = 0;
-    bool ok = true;
-    for (int t = tile0; t < tiles && ok; t += tile_step) {
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!__all_sync(0xffffffffu, mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort_flag))) { ok = false; break; }
-        const uint32_t fb = full0 + 8 * stage;
-        const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
-        if (elect_one()) {
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
+          const uint32_t fb = full0 + 8 * stage;
+          const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
           mbar_expect_tx(fb, tx_bytes);
           tma_load_2d(sx, &map_x, fb, kb * BK, t * BM);
           tma_load_2d(sx + GT_X_BYTES, &map_w, fb, kb * BK, 0);
           if (has_shared) tma_load_2d(sx + GT_X_BYTES + GT_W_BYTES, &map_s, fb, kb * BK, 0);
+          if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
     }
-    if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
   } else if (warp == 1) {
-    uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
-    // with a shared gate, its [16 x 64] block follows the [64 x 64] block of Wg in shared memory (same 128-byte
-    // swizzle rows), so one MMA of N = 80 covers both: accumulator columns 0..63 logits, 64 the shared gate
-    const uint32_t idesc_w = instr_desc(has_shared ? 80 : n_mma, false, false);
-    bool ok = true;
-    for (int t = tile0; t < tiles && ok; t += tile_step) {
-      if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag))) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + acc * 128;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, abort_flag))) { ok = false; break; }
+    if (lane == 0) {
+      uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
+      // with a shared gate, its [16 x 64] block follows the [64 x 64] block of Wg in shared memory (same 128-byte
+      // swizzle rows), so one MMA of N = 80 covers both: accumulator columns 0..63 logits, 64 the shared gate
+      const uint32_t idesc_w = instr_desc(has_shared ? 80 : n_mma, false, false);
+      bool ok = true;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
-        const uint32_t sw = sx + GT_X_BYTES;
-        if (elect_one()) {
+        const uint32_t d_tmem = tmem_base + acc * 128;
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
+          const uint32_t sw = sx + GT_X_BYTES;
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k)
-            tc_mma(d_tmem, smem_desc(sx + k * 32, 16, 1024), smem_desc(sw + k * 32, 16, 1024), idesc_w, (kb > kb0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < BK / UMMA_K; ++k) {
+            const uint64_t da = smem_desc(sx + k * 32, 16, 1024);
+            const uint32_t accum = (kb > 0 || k > 0) ? 1u : 0u;
+            tc_mma(d_tmem, da, smem_desc(sw + k * 32, 16, 1024), idesc_w, accum);
+          }
           tc_commit(empty0 + 8 * stage);
+          if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
+        if (!ok) break;
+        tc_commit(tfull0 + 8 * acc);
+        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
-      if (!ok) break;
-      if (elect_one()) tc_commit(tfull0 + 8 * acc);
-      __syncwarp();
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      if (!ok) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
     }
-    if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
   } else {
     const int q = warp & 3;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
-    for (int t = tile0; t < tiles && ok; t += tile_step) {
-      if (!__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag))) { ok = false; break; }
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      if (splits > 1) {  // this split's partial rows go to shared memory: its stages are free, every MMA has read them
-        float* mine = part + (32 * q + lane) * GT_PART_PITCH;
-        for (int c = 0; c < (has_shared ? 80 : n_mma); c += 16) {
-          uint32_t r[16];
-          tc_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + c, r);
-          tc_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 16; ++i) mine[c + i] = __uint_as_float(r[i]);
-        }
-        continue;
-      }
       const uint32_t taddr = tmem_base + acc * 128 + ((uint32_t)(32 * q) << 16);
       const long long tok = (long long)t * BM + 32 * q + lane;
       for (int c = 0; c < n_mma; c += 16) {
@@ -174,30 +145,6 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
-  }
-
-  if (splits > 1) {
-    cluster_sync_all();  // the partial rows of all splits are written
-    const int rows = BM / splits, cols = E + (has_shared ? 1 : 0);
-    const uint32_t local = smem_u32(part);
-    uint32_t peer[8];
-#pragma unroll
-    for (int x = 0; x < 8; ++x) peer[x] = map_to_cta(local, x < splits ? x : 0);
-    for (int i = threadIdx.x; i < rows * cols; i += GT_THREADS) {
-      const int r = rank * rows + i / cols, c = i % cols;
-      const long long tok = (long long)tile0 * BM + r;
-      const int at = r * GT_PART_PITCH + (c < E ? c : 64);
-      float v[8], sum = 0.f;
-#pragma unroll
-      for (int x = 0; x < 8; ++x) v[x] = x < splits ? ld_cluster(peer[x] + 4 * at) : 0.f;
-#pragma unroll
-      for (int x = 0; x < 8; ++x) sum += v[x];
-      if (tok < N) {
-        if (c < E) L[tok * E + c] = sum;
-        else z[tok] = sum;
-      }
-    }
-    cluster_sync_all();  // nobody leaves while its rows are being read
   }
 
   // after a wait gave up, let TMA loads still in flight land before the CTA (and its shared memory) goes away
@@ -237,24 +184,9 @@ int gate_tc_launch(const c2r_config* cfg, const void* X, const void* Wg, const v
     C2R_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     __atomic_store_n(&sms_of_device[dev], sms, __ATOMIC_RELEASE);
   }
-  const int tiles = (cfg->N + BM - 1) / BM, kblocks = (cfg->d + BK - 1) / BK;
-  int splits = 8;  // the most that leaves every split two k-blocks and every CTA an SM
-  while (splits > 1 && (tiles * splits > sms || kblocks < 2 * splits)) splits >>= 1;
-  cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = splits;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  lc.gridDim = dim3(splits > 1 ? tiles * splits : tiles < sms ? tiles : sms);
-  lc.blockDim = dim3(GT_THREADS);
-  lc.stream = s;
-  lc.attrs = attr;
-  lc.numAttrs = splits > 1 ? 1 : 0;
-  const int stages = splits > 1 ? GT_SPLIT_STAGES : GT_STAGES;
-  lc.dynamicSmemBytes = stages * GT_STAGE_BYTES + 1024;
-  C2R_CUDA(cudaLaunchKernelEx(&lc, gate_tc_kernel, mx, mw, ms, L, z, (int)cfg->N, (int)cfg->d, (int)cfg->E, (int)(wsg != nullptr), splits,
-                              stages, status));
+  const int tiles = (cfg->N + BM - 1) / BM;
+  const int grid = tiles < sms ? tiles : sms;
+  gate_tc_kernel<<<grid, GT_THREADS, smem, s>>>(mx, mw, ms, L, z, cfg->N, cfg->d, cfg->E, wsg != nullptr, status);
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

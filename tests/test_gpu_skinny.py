@@ -73,21 +73,3 @@ def test_uneven_counts_take_the_same_kernel(counts):
         assert_close_rms(host(Yp)[rows], (s * Yref)[rows], 3e-2, "Yp", out_bf16=False)
     other = np.setdiff1d(np.arange(R), rows)  # rows that belong to no expert are left alone
     assert (host(Yp)[other] == 7.0).all() and (host(H)[other] == 7.0).all()
-
-
-@pytest.mark.parametrize("N,d,E,shared", [(1, 2048, 60, True), (127, 1088, 33, False), (129, 1040, 7, True), (1021, 4096, 16, False),
-                                          (2200, 336, 63, True), (4737, 272, 64, False), (5, 240, 12, True)])
-def test_gate_logits_with_a_split_contraction(N, d, E, shared):
-    """Clusters of 8, 4, 2 and 1 CTAs per token tile, splits of unequal k-blocks, a partial last k-block, a partial last tile.
-    1e-4 as for the unsplit kernel: sums of d products of magnitude 0.02 in fp32 are off by well under 1e-5."""
-    from paper_2504_01337_b200 import binding as B
-    X, Wg, wsg = (G.round_bf16(G.normal(1, s, shp, sd)) for s, shp, sd in
-                  ((G.S_X, (N, d), 1.0), (G.S_WG, (E, d), 0.02), (G.S_WSG, (d,), 0.02)))
-    bf = torch.bfloat16
-    cfg = B.make_config(N, d, E, 16, 2, 3, 1, 16 if shared else 0, B.BF16, 1)
-    L = torch.full((N, E), 7.0, device="cuda")
-    z = torch.full((N,), 7.0, device="cuda")
-    B.gate_logits(cfg, dev(X, bf), dev(Wg, bf), dev(wsg, bf) if shared else None, L, z if shared else None)
-    assert np.abs(host(L) - O.gate_logits(X, Wg)).max() <= 1e-4
-    if shared:
-        assert np.abs(host(z) - X.astype(np.float64) @ wsg.astype(np.float64)).max() <= 1e-4
