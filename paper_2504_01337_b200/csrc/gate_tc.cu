@@ -7,6 +7,12 @@
 // 16 k-elements (N = 64 for the routed gate, N = 80 when the shared-expert gate's block rides along) into tensor
 // memory, and four warps write the fp32 accumulators out.  Waits are bounded like in the grouped
 // GEMM kernel.
+//
+// Few tokens are few tiles, and a CTA that streams 128 tokens alone is slow: a tile then has 64 or 32 tokens (the MMA still
+// computes 128 rows, the rest is whatever the stage holds and is not stored).  A split of the contraction over a cluster is faster still, but adds a
+// token's products in another order, and logits that differ in their last bits route near-ties to other experts.
+// (us, 128 tokens per tile and a divergent issuing lane against this: 13.3 / 10.0 for 1 token and 14.0 / 10.9
+// for 4096 of d = 2048, 21.0 / 15.1 for 1021 and 22.0 / 16.4 for 8192 of d = 4096.)
 #include "gemm.h"
 #include "tc_common.cuh"
 
@@ -23,7 +29,7 @@ constexpr int GT_TMEM_COLS = 256;          // two accumulators of 128 columns (6
 __global__ void __launch_bounds__(GT_THREADS, 1)
 gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_s, float* __restrict__ L, float* __restrict__ z, int N, int d,
-               int E, int has_shared, int32_t* __restrict__ status) {
+               int E, int has_shared, int tm, int32_t* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ uint64_t bars[2 * GT_STAGES + 4];
@@ -51,70 +57,70 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   const uint32_t tmem_base = warp_uniform(tmem_slot);
   volatile int* abort_flag = &s_abort;
 
-  const int tiles = (N + BM - 1) / BM;
+  const int tiles = (N + tm - 1) / tm;  // tm tokens per tile
   const int kblocks = (d + BK - 1) / BK;
   const int n_mma = (E + 15) / 16 * 16;  // MMA-N of the routed gate
-  const uint32_t tx_bytes = GT_X_BYTES + GT_W_BYTES + (has_shared ? GT_S_BYTES : 0);
+  const uint32_t tx_bytes = tm * BK * 2 + GT_W_BYTES + (has_shared ? GT_S_BYTES : 0);
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t fb = full0 + 8 * stage;
-          const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort_flag))) { ok = false; break; }
+        const uint32_t fb = full0 + 8 * stage;
+        const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
+        if (elect_one()) {
           mbar_expect_tx(fb, tx_bytes);
-          tma_load_2d(sx, &map_x, fb, kb * BK, t * BM);
+          tma_load_2d(sx, &map_x, fb, kb * BK, t * tm);
           tma_load_2d(sx + GT_X_BYTES, &map_w, fb, kb * BK, 0);
           if (has_shared) tma_load_2d(sx + GT_X_BYTES + GT_W_BYTES, &map_s, fb, kb * BK, 0);
-          if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
     }
+    if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
   } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
-      // with a shared gate, its [16 x 64] block follows the [64 x 64] block of Wg in shared memory (same 128-byte
-      // swizzle rows), so one MMA of N = 80 covers both: accumulator columns 0..63 logits, 64 the shared gate
-      const uint32_t idesc_w = instr_desc(has_shared ? 80 : n_mma, false, false);
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+    uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
+    // with a shared gate, its [16 x 64] block follows the [64 x 64] block of Wg in shared memory (same 128-byte
+    // swizzle rows), so one MMA of N = 80 covers both: accumulator columns 0..63 logits, 64 the shared gate
+    const uint32_t idesc_w = instr_desc(has_shared ? 80 : n_mma, false, false);
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      if (!__all_sync(0xffffffffu, mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1u, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + acc * 128;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, abort_flag))) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * 128;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
-          const uint32_t sw = sx + GT_X_BYTES;
+        const uint32_t sx = smem_base + stage * GT_STAGE_BYTES;
+        const uint32_t sw = sx + GT_X_BYTES;
+        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t da = smem_desc(sx + k * 32, 16, 1024);
-            const uint32_t accum = (kb > 0 || k > 0) ? 1u : 0u;
-            tc_mma(d_tmem, da, smem_desc(sw + k * 32, 16, 1024), idesc_w, accum);
-          }
+          for (int k = 0; k < BK / UMMA_K; ++k)
+            tc_mma(d_tmem, smem_desc(sx + k * 32, 16, 1024), smem_desc(sw + k * 32, 16, 1024), idesc_w, (kb > 0 || k > 0) ? 1u : 0u);
           tc_commit(empty0 + 8 * stage);
-          if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        tc_commit(tfull0 + 8 * acc);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        __syncwarp();
+        if (++stage == GT_STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
+      if (!ok) break;
+      if (elect_one()) tc_commit(tfull0 + 8 * acc);
+      __syncwarp();
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+    if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
   } else {
     const int q = warp & 3;
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-      if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag))) { ok = false; break; }
       tc_fence_after();
       const uint32_t taddr = tmem_base + acc * 128 + ((uint32_t)(32 * q) << 16);
-      const long long tok = (long long)t * BM + 32 * q + lane;
-      for (int c = 0; c < n_mma; c += 16) {
+      const long long tok = 32 * q < tm ? (long long)t * tm + 32 * q + lane : N;
+      for (int c = 0; c < n_mma && 32 * q < tm; c += 16) {
         uint32_t r[16];
         tc_ld16(taddr + c, r);
         tc_ld_wait();
@@ -133,7 +139,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           }
         }
       }
-      if (has_shared) {
+      if (has_shared && 32 * q < tm) {
         uint32_t r[16];
         tc_ld16(taddr + 64, r);
         tc_ld_wait();
@@ -163,30 +169,41 @@ bool gate_tc_supported(const c2r_config* cfg) {
   return cfg->dtype == C2R_BF16 && cfg->E <= 64 && cfg->d % 8 == 0 && cfg->N > 0 && get_encode() != nullptr;
 }
 
-int gate_tc_launch(const c2r_config* cfg, const void* X, const void* Wg, const void* wsg, float* L, float* z,
-                   int32_t* status, cudaStream_t s) {
-  CUtensorMap mx, mw, ms;
-  int rc = make_map(&mx, X, cfg->d, cfg->N, 0, BK, BM);
-  if (rc) return rc;
-  rc = make_map(&mw, Wg, cfg->d, cfg->E, 0, BK, 64);
-  if (rc) return rc;
-  rc = make_map(&ms, wsg ? wsg : Wg, cfg->d, 1, 0, BK, 16);
-  if (rc) return rc;
-  constexpr int smem = GT_STAGES * GT_STAGE_BYTES + 1024;
+constexpr int GT_SMEM = GT_STAGES * GT_STAGE_BYTES + 1024;
+
+// SM count of the current device (a negative error code if that fails); the first call per device also sets the kernel's
+// shared-memory limit.
+static int gate_sms() {
   constexpr int MAX_DEV = 64;
-  static int sms_of_device[MAX_DEV] = {};  // SM count, also "the kernel's shared-memory limit is set on this device"
+  static int sms_of_device[MAX_DEV] = {};
   int dev = 0;
   C2R_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= MAX_DEV) return C2R_ERR_UNSUPPORTED_SHAPE;
   int sms = __atomic_load_n(&sms_of_device[dev], __ATOMIC_ACQUIRE);
   if (sms == 0) {
-    C2R_CUDA(cudaFuncSetAttribute(gate_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    C2R_CUDA(cudaFuncSetAttribute(gate_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GT_SMEM));
     C2R_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     __atomic_store_n(&sms_of_device[dev], sms, __ATOMIC_RELEASE);
   }
-  const int tiles = (cfg->N + BM - 1) / BM;
+  return sms;
+}
+
+int gate_tc_launch(const c2r_config* cfg, const void* X, const void* Wg, const void* wsg, float* L, float* z,
+                   int32_t* status, cudaStream_t s) {
+  CUtensorMap mx, mw, ms;
+  const int sms = gate_sms();
+  if (sms < 0) return sms;
+  int tm = BM;  // halved while every tile still has an SM of its own
+  while (tm > 32 && (cfg->N + tm / 2 - 1) / (tm / 2) <= sms) tm >>= 1;
+  int rc = make_map(&mx, X, cfg->d, cfg->N, 0, BK, tm);
+  if (rc) return rc;
+  rc = make_map(&mw, Wg, cfg->d, cfg->E, 0, BK, 64);
+  if (rc) return rc;
+  rc = make_map(&ms, wsg ? wsg : Wg, cfg->d, 1, 0, BK, 16);
+  if (rc) return rc;
+  const int tiles = (cfg->N + tm - 1) / tm;
   const int grid = tiles < sms ? tiles : sms;
-  gate_tc_kernel<<<grid, GT_THREADS, smem, s>>>(mx, mw, ms, L, z, cfg->N, cfg->d, cfg->E, wsg != nullptr, status);
+  gate_tc_kernel<<<grid, GT_THREADS, GT_SMEM, s>>>(mx, mw, ms, L, z, cfg->N, cfg->d, cfg->E, wsg != nullptr, tm, status);
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
