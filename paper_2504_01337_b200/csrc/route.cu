@@ -10,11 +10,13 @@ thread_local int g_last_cuda_error = 0;
 unsigned long long g_launch_count = 0;
 
 // ---------------------------------------------------------------------------------------------
-// Routing (Sec. 3.3 step 2).  One warp per token; lane l holds logits l and l+32.  K rounds of an
-// arg-max under the total order (value desc, index asc); after round 0 the candidate set
-// is intersected with the top-1 expert's collaborator mask.  A round is one warp-wide integer maximum over
-// order-preserving keys and a ballot for its lowest index: the kernel is bound by this chain, and ten dependent shuffles
-// per round took 13.5 us where this takes 10.6 (16384 tokens, 60 experts, top-4; the sets of 60 experts 5.7 -> 3.7).
+// Routing (Sec. 3.3 step 2).  A thread per token over logits staged in shared memory as order-preserving integer keys: K
+// scans, each for the best remaining candidate under the total order (value desc, index asc); after the first the candidates
+// are those in the top-1 expert's collaborator mask.  The kernel is bound by the instructions of the blocks it has -- their number is
+// fixed by the dispatch's blocking -- and a scan costs an instruction or two per logit for 32 tokens at once; a warp per token with
+// a warp-wide arg-max per round took several times as many
+// (16384 tokens, 60 experts, top-4: 13.5 us with a shuffle arg-max, 10.6 with an integer one, 8.8 here; 512 tokens, 8 experts,
+// top-2: 17.4, 13.2, 4.4).
 // ---------------------------------------------------------------------------------------------
 // Order-preserving map of a logit to an unsigned key above 0 (-0 and +0 share one, as they compare equal); 0 marks an
 // expert that is not a candidate.
@@ -24,103 +26,181 @@ __device__ __forceinline__ uint32_t logit_key(float v) {
 }
 __device__ __forceinline__ float key_logit(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k); }
 
-constexpr int ROUTE_WARPS = 32;
+// Keys per token in shared memory: whole groups of four, and odd, so that the threads of a warp read one expert's keys
+// without bank conflicts.
+__host__ __device__ inline int route_pitch(int E) { return (E + 3) / 4 * 4 + 1; }
 
-// A block owns tokens_per_block consecutive tokens (the blocking of the dispatch's counting sort), a warp
-// every ROUTE_WARPS-th of them.  block_counts (optional): [blocks][E] experts' slot counts of the block's
-// tokens -- the histogram the dispatch starts from, so it need not read idx again to build it.  A token's
-// K experts are distinct, hence lanes 0..K-1 bump different counters of the warp's private row: no atomics.
-__global__ void __launch_bounds__(ROUTE_WARPS * 32) route_kernel(const float* __restrict__ L, const uint64_t* __restrict__ mask,
-                                                                 int32_t* __restrict__ idx, float* __restrict__ w,
-                                                                 float* __restrict__ p, int32_t* __restrict__ status, int N,
-                                                                 int E, int K, int renorm, int tokens_per_block,
-                                                                 int32_t* __restrict__ block_counts) {
-  __shared__ int warp_cnt[ROUTE_WARPS][64];
-  __shared__ uint64_t s_mask[64];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (block_counts != nullptr)
-    for (int i = threadIdx.x; i < ROUTE_WARPS * 64; i += blockDim.x) (&warp_cnt[0][0])[i] = 0;
-  if ((int)threadIdx.x < E) s_mask[threadIdx.x] = mask != nullptr ? mask[threadIdx.x] : ~0ull;
-  __syncthreads();
-  const float NEG_INF = -INFINITY;
-  const int t_end = min(N, (int)(blockIdx.x + 1) * tokens_per_block);
-  int flags = 0;
-  int t = blockIdx.x * tokens_per_block + warp;
-  float n0 = NEG_INF, n1 = NEG_INF;  // the next token's logits, requested one token ahead
-  if (t < t_end) {
-    if (lane < E) n0 = L[(size_t)t * E + lane];
-    if (lane + 32 < E) n1 = L[(size_t)t * E + lane + 32];
-  }
-  for (; t < t_end; t += ROUTE_WARPS) {
-    float v0 = n0, v1 = n1;
-    if (t + ROUTE_WARPS < t_end) {
-      if (lane < E) n0 = L[(size_t)(t + ROUTE_WARPS) * E + lane];
-      if (lane + 32 < E) n1 = L[(size_t)(t + ROUTE_WARPS) * E + lane + 32];
+// The largest key among the candidates (bits of avail), lowest index first; key 0 and index -1 if there are none.  Four
+// interleaved chains of compare-and-select.
+__device__ __forceinline__ void best_candidate(const uint32_t* row, uint64_t avail, int E, uint32_t& key, int& sel) {
+  uint32_t b[4] = {0u, 0u, 0u, 0u};
+  int at[4] = {64, 64, 64, 64};
+  uint32_t bits = (uint32_t)avail;
+#pragma unroll 2
+  for (int e0 = 0; e0 < E; e0 += 4, bits >>= 4) {
+    if (e0 == 32) bits = (uint32_t)(avail >> 32);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t k = row[e0 + q] & (uint32_t)((int32_t)(bits << (31 - q)) >> 31);
+      at[q] = k > b[q] ? e0 + q : at[q];
+      b[q] = max(k, b[q]);
     }
-    if (v0 != v0) { v0 = NEG_INF; flags |= C2R_STATUS_NAN_LOGIT; }
-    if (v1 != v1) { v1 = NEG_INF; flags |= C2R_STATUS_NAN_LOGIT; }
-    uint64_t avail = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
-    const uint64_t valid = avail;
-    uint64_t chosen = 0;
-    float my_sel = NEG_INF;  // lane k keeps the logit picked in round k
-    int my_idx = 0;
-    const uint32_t key0 = logit_key(v0), key1 = logit_key(v1);
-    for (int k = 0; k < K; ++k) {
-      const uint32_t c0 = ((avail >> lane) & 1ull) ? key0 : 0u, c1 = ((avail >> (lane + 32)) & 1ull) ? key1 : 0u;
-      const uint32_t best = __reduce_max_sync(0xffffffffu, max(c0, c1));
-      const uint32_t at0 = __ballot_sync(0xffffffffu, c0 == best), at1 = __ballot_sync(0xffffffffu, c1 == best);
-      int bi = at0 ? __ffs(at0) - 1 : 31 + __ffs(at1);
-      float bv = key_logit(best);
-      if (best == 0u) {  // candidate set exhausted: fall back to the lowest unselected expert
-        flags |= C2R_STATUS_SET_TOO_SMALL;
-        bi = __ffsll((long long)(valid & ~chosen)) - 1;
-        bv = NEG_INF;
+  }
+  key = b[0]; sel = at[0];
+#pragma unroll
+  for (int q = 1; q < 4; ++q)
+    if (b[q] > key || (b[q] == key && at[q] < sel)) { key = b[q]; sel = at[q]; }
+  if (key == 0u) sel = -1;
+}
+
+// A block owns tokens_per_block consecutive tokens (the blocking of the dispatch's counting sort).  block_counts (optional):
+// [blocks][E] experts' slot counts of the block's tokens -- the histogram the dispatch starts from, so it need not read
+// idx again to build it.
+template <int K>
+__global__ void __launch_bounds__(512) route_kernel(const float* __restrict__ L, const uint64_t* __restrict__ mask,
+                                                    int32_t* __restrict__ idx, float* __restrict__ w, float* __restrict__ p,
+                                                    int32_t* __restrict__ status, int N, int E, int renorm, int tokens_per_block,
+                                                    int32_t* __restrict__ block_counts) {
+  extern __shared__ uint32_t s_key[];  // [tokens][route_pitch(E)]
+  __shared__ uint64_t s_mask[64];
+  __shared__ int s_cnt[64];
+  const int tid = threadIdx.x;
+  const int t_begin = blockIdx.x * tokens_per_block, tokens = min(N - t_begin, tokens_per_block);
+  const int pitch = route_pitch(E);
+  if (tid < 64) {
+    s_cnt[tid] = 0;
+    s_mask[tid] = (tid < E && mask != nullptr) ? mask[tid] : ~0ull;
+  }
+  int flags = 0;
+  {
+    // eight loads in flight per thread (clamped, not predicated: a load under a condition waits for the one before it)
+    const float* src = L + (size_t)t_begin * E;
+    auto put = [&](int at, float v) {
+      if (v != v) { v = -INFINITY; flags |= C2R_STATUS_NAN_LOGIT; }
+      s_key[at] = logit_key(v);
+    };
+    if ((E & 3) == 0 && ((uintptr_t)L & 15u) == 0) {
+      const int per = E >> 2, n = tokens * per;
+      for (int i0 = tid; i0 < n; i0 += 8 * blockDim.x) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = reinterpret_cast<const float4*>(src)[min(i0 + u * (int)blockDim.x, n - 1)];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = i0 + u * blockDim.x, at = 4 * i + i / per;  // pitch E + 1
+          if (i < n) { put(at, v[u].x); put(at + 1, v[u].y); put(at + 2, v[u].z); put(at + 3, v[u].w); }
+        }
       }
-      chosen |= 1ull << bi;
-      avail &= ~(1ull << bi);
-      if (k == 0) avail &= s_mask[bi];
-      if (lane == k) { my_sel = bv; my_idx = bi; }
+    } else {
+      const int n = tokens * E;
+      for (int i0 = tid; i0 < n; i0 += 8 * blockDim.x) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[min(i0 + u * (int)blockDim.x, n - 1)];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = i0 + u * blockDim.x;
+          if (i < n) put(i / E * pitch + i % E, v[u]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < tokens) {
+    uint32_t* row = s_key + tid * pitch;
+    uint32_t key[K];
+    int sel[K];
+    uint64_t avail = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      best_candidate(row, avail, E, key[j], sel[j]);
+      if (sel[j] >= 0) avail &= ~(1ull << sel[j]);
+      if (j == 0) avail &= s_mask[sel[0]];
     }
     // Eq. 1 weights.  The round-0 logit is the row maximum, so it is the softmax shift for both forms.
-    const float top = __shfl_sync(0xffffffffu, my_sel, 0);
-    float denom;
-    if (renorm) {
-      const float ek = (lane < K) ? expf(my_sel - top) : 0.f;  // K <= 8: the sum stays inside groups of eight lanes
-      denom = ek;
+    float lg[K], ek[8];
 #pragma unroll
-      for (int off = 4; off > 0; off >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, off);
-      if (lane < K) w[(size_t)t * K + lane] = ek / denom;
-    }
-    if (!renorm || p != nullptr) {
-      float e0 = (lane < E) ? expf(v0 - top) : 0.f;
-      float e1 = (lane + 32 < E) ? expf(v1 - top) : 0.f;
-      float s = e0 + e1;
+    for (int j = 0; j < K; ++j) lg[j] = sel[j] >= 0 ? key_logit(key[j]) : -INFINITY;
+    uint64_t chosen = 0;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (p != nullptr) {
-        if (lane < E) p[(size_t)t * E + lane] = e0 / s;
-        if (lane + 32 < E) p[(size_t)t * E + lane + 32] = e1 / s;
+    for (int j = 0; j < K; ++j) {
+      if (sel[j] < 0) {  // candidate set exhausted: fall back to the lowest unselected expert
+        flags |= C2R_STATUS_SET_TOO_SMALL;
+        const uint64_t valid = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
+        sel[j] = __ffsll((long long)(valid & ~chosen)) - 1;
       }
-      if (!renorm && lane < K) w[(size_t)t * K + lane] = expf(my_sel - top) / s;
+      chosen |= 1ull << sel[j];
     }
-    if (lane < K) {
-      idx[(size_t)t * K + lane] = my_idx;
-      if (block_counts != nullptr) warp_cnt[warp][my_idx] += 1;
+    const size_t o = (size_t)(t_begin + tid) * K;
+    const float top = lg[0];
+    if (renorm) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) ek[j] = j < K ? expf(lg[j < K ? j : 0] - top) : 0.f;
+      const float denom = ((ek[0] + ek[4]) + (ek[2] + ek[6])) + ((ek[1] + ek[5]) + (ek[3] + ek[7]));
+#pragma unroll
+      for (int j = 0; j < K; ++j) w[o + j] = ek[j] / denom;
+    }
+    if (!renorm || p != nullptr) {  // the full softmax, summed as a binary tree over the expert index
+      float s16[16];
+#pragma unroll
+      for (int x = 0; x < 16; ++x) {
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = x + 16 * q < E ? expf(key_logit(row[x + 16 * q]) - top) : 0.f;
+        s16[x] = (v[0] + v[2]) + (v[1] + v[3]);
+      }
+#pragma unroll
+      for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          if (x < h) s16[x] += s16[x + h];
+      if (p != nullptr)
+        for (int e = 0; e < E; ++e) row[e] = __float_as_uint(expf(key_logit(row[e]) - top) / s16[0]);
+      if (!renorm) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[o + j] = expf(lg[j] - top) / s16[0];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      idx[o + j] = sel[j];
+      if (block_counts != nullptr) atomicAdd(&s_cnt[sel[j]], 1);  // integer counts: the order does not matter
     }
   }
-  if (block_counts != nullptr) {
+  if (block_counts != nullptr || p != nullptr) {
     __syncthreads();
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-      int s = 0;
-#pragma unroll
-      for (int x = 0; x < ROUTE_WARPS; ++x) s += warp_cnt[x][e];
-      block_counts[(size_t)blockIdx.x * E + e] = s;
-    }
+    if (block_counts != nullptr && tid < E) block_counts[(size_t)blockIdx.x * E + tid] = s_cnt[tid];
+    if (p != nullptr)
+      for (int i = tid; i < tokens * E; i += blockDim.x) p[(size_t)t_begin * E + i] = __uint_as_float(s_key[i / E * pitch + i % E]);
   }
   if (status != nullptr) {
     flags = __reduce_or_sync(0xffffffffu, flags);
-    if (flags && lane == 0) atomicOr(status, flags);
+    if (flags && (tid & 31) == 0) atomicOr(status, flags);
   }
+}
+
+template <int K>
+static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
+                        int32_t* status, int32_t* block_counts, cudaStream_t s) {
+  const int tpb = perm_tokens_per_block(K);
+  const int threads = tpb < 128 ? 128 : (tpb + 31) / 32 * 32;
+  const int smem = tpb * route_pitch(cfg->E) * (int)sizeof(uint32_t);
+  if (smem > 48 * 1024) {
+    constexpr int MAX_DEV = 64;
+    static int done[MAX_DEV] = {};  // the kernel's shared-memory limit is set on this device
+    int dev = 0;
+    C2R_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= MAX_DEV) return C2R_ERR_UNSUPPORTED_SHAPE;
+    if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
+      C2R_CUDA(cudaFuncSetAttribute(route_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    perm_tokens_per_block(K) * route_pitch(64) * (int)sizeof(uint32_t)));
+      __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
+    }
+  }
+  route_kernel<K><<<(cfg->N + tpb - 1) / tpb, threads, smem, s>>>(L, mask, idx, w, p, status, cfg->N, cfg->E, cfg->renorm, tpb,
+                                                                 block_counts);
+  C2R_LAUNCH_CHECK();
+  return C2R_OK;
 }
 
 __global__ void route_bwd_kernel(const float* __restrict__ w, const float* __restrict__ dw, float* __restrict__ dl,
@@ -327,11 +407,17 @@ int c2r::route_impl(const c2r_config* cfg, const float* L, const uint64_t* mask,
   C2R_REQUIRE(L && idx && w, C2R_ERR_INVALID_ARG);
   if (mask) C2R_REQUIRE(cfg->T >= cfg->K - 1 && cfg->T <= cfg->E - 1, C2R_ERR_INVALID_ARG);
   if (cfg->N == 0) return C2R_OK;
-  const int tpb = perm_tokens_per_block(cfg->K);
-  route_kernel<<<(cfg->N + tpb - 1) / tpb, ROUTE_WARPS * 32, 0, as_stream(stream)>>>(L, mask, idx, w, p, status, cfg->N, cfg->E,
-                                                                                   cfg->K, cfg->renorm, tpb, block_counts);
-  C2R_LAUNCH_CHECK();
-  return C2R_OK;
+  cudaStream_t s = as_stream(stream);
+  switch (cfg->K) {
+    case 1: return route_launch<1>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 2: return route_launch<2>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 3: return route_launch<3>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 4: return route_launch<4>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 5: return route_launch<5>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 6: return route_launch<6>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    case 7: return route_launch<7>(cfg, L, mask, idx, w, p, status, block_counts, s);
+    default: return route_launch<8>(cfg, L, mask, idx, w, p, status, block_counts, s);
+  }
 }
 
 extern "C" int c2r_route(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
