@@ -41,7 +41,6 @@ __global__ void pack_kernel(const T* __restrict__ W1, const T* __restrict__ W3, 
   }
 }
 
-constexpr int SIMT_THREADS = 256;
 
 // Four consecutive elements as floats; `vec`: base pointers and strides are known to be aligned for one vector load.
 __device__ __forceinline__ float4 load4(const float* p, bool vec) {
@@ -66,42 +65,58 @@ __device__ __forceinline__ int tile_at(int k, int m) {
 }
 
 // A W x SK operand tile on its way from global memory to shared memory, held in registers while the previous tile is used.
-template <typename T, int W, int SK>
+// Addresses are worked out once and advanced by a k-tile: the small problems are bound by instructions as much as by latency.
+template <typename T, int W, int SK, int SIMT_THREADS>
 struct TileLoad {
-  static constexpr int V = W * SK / 4;                                       // four-element pieces
-  static constexpr int PER = (V + SIMT_THREADS - 1) / SIMT_THREADS;
+  static constexpr int PER = W * SK / 4 / SIMT_THREADS;  // four-element pieces per thread
+  static_assert(W * SK / 4 % SIMT_THREADS == 0, "every thread loads the same number of pieces");
   float4 v[PER];
-  // row(m): address of element (m, 0); element (m, k) lies k * sk (and m * sm for sk != 1) further
+  const T* src[PER];   // next piece; NULL where the tile has no such row
+  int k_of[PER], at[PER];
+  long long step;
+  int lane_step;       // distance of a piece's elements in the shared tile
+  // row(m): address of element (m, 0); element (m, k) lies k * sk further, and for sk != 1 rows lie next to each other
   template <typename Row>
-  __device__ __forceinline__ void load(Row row, long long sk, int m_left, int k0, int Kd, bool vec) {
+  __device__ __forceinline__ void init(Row row, long long sk, int m_left) {
+    step = SK * sk;
+    lane_step = sk == 1 ? W : 1;
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
       const int x = threadIdx.x + i * SIMT_THREADS;
-      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (V % SIMT_THREADS != 0 && x >= V) continue;
-      if (sk == 1) {  // contraction contiguous
-        const int k = 4 * (x % (SK / 4)), m = x / (SK / 4);
-        if (m < m_left && k0 + k < Kd) v[i] = load4(row(m) + k0 + k, vec);
-      } else {        // rows contiguous
-        const int m = 4 * (x % (W / 4)), k = x / (W / 4);
-        if (m < m_left && k0 + k < Kd) v[i] = load4(row(m) + (k0 + k) * sk, vec);
-      }
+      const int k = sk == 1 ? 4 * (x % (SK / 4)) : x / (W / 4), m = sk == 1 ? x / (SK / 4) : 4 * (x % (W / 4));
+      k_of[i] = k;
+      at[i] = tile_at<W>(k, m);
+      src[i] = m < m_left ? row(m) + k * sk : nullptr;
     }
   }
-  __device__ __forceinline__ void store(float* tile, long long sk) const {
+  __device__ __forceinline__ void load(int k_left, bool vec) {
+    if (vec) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (src[i] != nullptr && k_of[i] < k_left) v[i] = load4(src[i], true);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (src[i] != nullptr && k_of[i] < k_left) v[i] = load4(src[i], false);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+      if (src[i] != nullptr) src[i] += step;
+  }
+  __device__ __forceinline__ void store(float* tile) const {
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-      const int x = threadIdx.x + i * SIMT_THREADS;
-      if (V % SIMT_THREADS != 0 && x >= V) continue;
-      if (sk == 1) {
-        const int k = 4 * (x % (SK / 4)), m = x / (SK / 4);
-        tile[tile_at<W>(k, m)] = v[i].x;
-        tile[tile_at<W>(k + 1, m)] = v[i].y;
-        tile[tile_at<W>(k + 2, m)] = v[i].z;
-        tile[tile_at<W>(k + 3, m)] = v[i].w;
-      } else {
-        const int m = 4 * (x % (W / 4)), k = x / (W / 4);
-        *reinterpret_cast<float4*>(&tile[tile_at<W>(k, m)]) = v[i];
+      if (lane_step == 1) {
+        *reinterpret_cast<float4*>(&tile[at[i]]) = v[i];
+      } else {  // the four k of a piece share a column group: W floats apart
+        tile[at[i]] = v[i].x;
+        tile[at[i] + W] = v[i].y;
+        tile[at[i] + 2 * W] = v[i].z;
+        tile[at[i] + 3 * W] = v[i].w;
       }
     }
   }
@@ -114,10 +129,10 @@ struct TileLoad {
 // registers while the current one is used (two shared-memory buffers, one barrier per tile).  The small configurations
 // this serves are bound by latency: a chain of 16-deep tiles, each waiting for its own loads, took 80 us for K = 256
 // where this takes 16.5 (1024 rows, 128 dual columns; weight gradients of 375 rows 158 -> 28; whole fp32 training step of
-// 1500 tokens 502 -> 206).  64 x 64 tiles where they fill the chip, else 32-wide ones.
+// 1500 tokens 500 -> 200).  64 x 64 tiles where they fill the chip, else 32-wide ones.
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL>
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS>
 __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   constexpr int GROUP = (TM / 4) * (TN / 4), G = SIMT_THREADS / GROUP;  // threads per group, groups
   constexpr int MR = G == 1 ? 4 : TM * TN / (4 * SIMT_THREADS);         // output rows a thread finishes, four columns each
@@ -169,12 +184,15 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   const int grp_k = tid / GROUP, tg = tid % GROUP;
   const int tx = tg % (TN / 4), ty = tg / (TN / 4);
   float acc[4][4] = {}, acc2[DUAL ? 4 : 1][4] = {};
-  TileLoad<T, TM, SK> la;
-  TileLoad<T, TN, SK> lb, lb2;
+  TileLoad<T, TM, SK, SIMT_THREADS> la;
+  TileLoad<T, TN, SK, SIMT_THREADS> lb, lb2;
+  la.init(rowA, g.sak, M - m0);
+  lb.init(rowB, g.sbk, g.Ndim - n0);
+  if (DUAL) lb2.init(rowB2, g.sbk, g.Ndim - n0);
   auto fetch = [&](int k0) {
-    la.load(rowA, g.sak, M - m0, k0, Kd, vec);
-    lb.load(rowB, g.sbk, g.Ndim - n0, k0, Kd, vec);
-    if (DUAL) lb2.load(rowB2, g.sbk, g.Ndim - n0, k0, Kd, vec);
+    la.load(Kd - k0, vec);
+    lb.load(Kd - k0, vec);
+    if (DUAL) lb2.load(Kd - k0, vec);
   };
   constexpr int BUF = SK * (TM + TN * (DUAL ? 2 : 1));
   fetch(0);
@@ -182,12 +200,12 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
     float* sa = smem + buf * BUF;
     float* sb = sa + SK * TM;
     float* sb2 = sb + SK * TN;
-    la.store(sa, g.sak);
-    lb.store(sb, g.sbk);
-    if (DUAL) lb2.store(sb2, g.sbk);
+    la.store(sa);
+    lb.store(sb);
+    if (DUAL) lb2.store(sb2);
     __syncthreads();
     if (k0 + SK < Kd) fetch(k0 + SK);
-#pragma unroll
+#pragma unroll 8  // a kernel this short is bound by instruction fetch if the body is longer
     for (int kk = 0; kk < SK / G; ++kk) {
       const int k = grp_k * (SK / G) + kk;
       const float4 av = *reinterpret_cast<const float4*>(&sa[tile_at<TM>(k, 4 * ty)]);
@@ -297,11 +315,19 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   }
 }
 
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL>
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS = 256>
 static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
-  simt_gemm_kernel<T, TC, TM, TN, SK, DUAL><<<dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s>>>(g);
+  simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, SIMT_THREADS><<<dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s>>>(g);
   C2R_LAUNCH_CHECK();
   return C2R_OK;
+}
+
+// Whether every group of four elements the kernel loads lies on a four-element boundary.
+template <typename T>
+static int simt_vec(const SimtGemm& g) {
+  const uintptr_t bits = (uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last;
+  return (bits & (4 * sizeof(T) - 1)) == 0 && (g.sak == 1 ? g.sam : g.sak) % 4 == 0 &&
+         (g.sbk == 1 ? g.sbn : g.sbk) % 4 == 0 && g.sB % 4 == 0;
 }
 
 // max_m: rows (SIMT_ROWS: of all groups together) or Mdim.
@@ -309,9 +335,7 @@ template <typename T, typename TC = T>
 int simt_launch(SimtGemm g, int n_groups, int64_t max_m, cudaStream_t s) {
   if (n_groups == 0 || max_m == 0 || g.Ndim == 0) return C2R_OK;
   g.n_groups = n_groups;
-  const uintptr_t align = 4 * sizeof(T) - 1;
-  const uintptr_t bits = (uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last;
-  g.vec = (bits & align) == 0 && (g.sak == 1 ? g.sam : g.sak) % 4 == 0 && (g.sbk == 1 ? g.sbn : g.sbk) % 4 == 0 && g.sB % 4 == 0;
+  g.vec = simt_vec<T>(g);
   const bool rows = g.mode == SIMT_ROWS && g.counts != nullptr;
   const int z = rows ? 1 : n_groups;
   // SIMT_ROWS: whole tiles of all groups, and one more per group for its remainder
@@ -335,7 +359,10 @@ int simt_gate_logits(const c2r_config* cfg, const void* X, const void* Wg, const
   g.A = X; g.sam = cfg->d; g.sak = 1; g.B = Wg; g.sbn = cfg->d; g.sbk = 1; g.B_last = wsg;
   g.C = L; g.C_last = wsg ? z : nullptr; g.ldc = cfg->E;
   g.Mdim = cfg->N; g.Ndim = cfg->E + (wsg ? 1 : 0); g.Kdim = cfg->d;
-  return simt_launch<T, float>(g, 1, cfg->N, s);
+  // a tile without thread groups: one chain of products in k order, whatever the batch (near-ties must not move with it)
+  g.n_groups = 1;
+  g.vec = simt_vec<T>(g);
+  return simt_launch_tile<T, float, 32, 32, 32, false, 64>(g, (cfg->N + 31) / 32, 1, s);
 }
 template int simt_gate_logits<float>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);
 template int simt_gate_logits<__nv_bfloat16>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);
