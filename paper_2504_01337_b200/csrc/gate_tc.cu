@@ -52,6 +52,7 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  chain_wait();  // before the first access to global memory
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = warp_uniform(tmem_slot);
@@ -111,6 +112,9 @@ gate_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     if (!ok && lane == 0) { *abort_flag = 1; if (status) atomicOr(status, C2R_STATUS_WAIT_TIMEOUT); }
+    // Late: the routing kernel's blocks do not fit beside this kernel's, and released early all of them would be placed on
+    // the few SMs without a token tile (calibration pass 43 us, released here 35).
+    chain_release();
   } else {
     const int q = warp & 3;
     uint32_t acc = 0, acc_phase = 0;
@@ -203,7 +207,7 @@ int gate_tc_launch(const c2r_config* cfg, const void* X, const void* Wg, const v
   if (rc) return rc;
   const int tiles = (cfg->N + tm - 1) / tm;
   const int grid = tiles < sms ? tiles : sms;
-  gate_tc_kernel<<<grid, GT_THREADS, GT_SMEM, s>>>(mx, mw, ms, L, z, cfg->N, cfg->d, cfg->E, wsg != nullptr, tm, status);
+  C2R_CUDA(launch_chained(gate_tc_kernel, grid, GT_THREADS, GT_SMEM, s, mx, mw, ms, L, z, cfg->N, cfg->d, cfg->E, wsg != nullptr, tm, status));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

@@ -119,6 +119,9 @@ int permute_call(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
                  int32_t* offsets, int32_t* row_of_slot, int32_t* slot_of_row, void* Xp, int32_t* status, void* ws,
                  size_t ws_bytes, void* stream, bool have_hist, const float* w, float* w_row);
 
+// Sets up to three arrays of 32-bit words (NULL with 0 words for fewer) to a value, in the chain of kernels on the stream.
+int fill_words(uint32_t* a, int64_t na, uint32_t* b, int64_t nb, uint32_t* c, int64_t nc, uint32_t value, cudaStream_t s);
+
 size_t permute_ws_bytes(const c2r_config* cfg);
 size_t layer_ws_bytes(const c2r_config* cfg);
 size_t gate_bwd_ws_bytes(const c2r_config* cfg);

@@ -19,6 +19,7 @@ __host__ __device__ inline int pack_width(int i, int I) {
 template <typename T>
 __global__ void pack_kernel(const T* __restrict__ W1, const T* __restrict__ W3, T* __restrict__ W13p, int I, int d,
                             int unpack, T* __restrict__ W1o, T* __restrict__ W3o) {
+  chain_begin();
   using V = Vec16<T>;
   const int e = blockIdx.y;
   const int i = blockIdx.x;
@@ -134,6 +135,7 @@ struct TileLoad {
 // (SIMT_WGRAD).
 template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS>
 __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
+  chain_begin();
   constexpr int GROUP = (TM / 4) * (TN / 4), G = SIMT_THREADS / GROUP;  // threads per group, groups
   constexpr int MR = G == 1 ? 4 : TM * TN / (4 * SIMT_THREADS);         // output rows a thread finishes, four columns each
   constexpr int TILES = 2 * SK * (TM + TN * (DUAL ? 2 : 1)), RED = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4);
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
 
 template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS = 256>
 static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
-  simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, SIMT_THREADS><<<dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s>>>(g);
+  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s, g));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -438,12 +440,12 @@ static int pack_common(const c2r_config* cfg, int nE, int I, const void* W1, con
   if (nE == 0) return C2R_OK;
   dim3 grid(I, nE);
   if (cfg->dtype == C2R_BF16)
-    pack_kernel<__nv_bfloat16><<<grid, 128, 0, as_stream(stream)>>>((const __nv_bfloat16*)W1, (const __nv_bfloat16*)W3,
-                                                                    (__nv_bfloat16*)W13p, I, cfg->d, unpack,
-                                                                    (__nv_bfloat16*)W1o, (__nv_bfloat16*)W3o);
+    C2R_CUDA(launch_chained(pack_kernel<__nv_bfloat16>, grid, 128, 0, as_stream(stream), (const __nv_bfloat16*)W1, (const __nv_bfloat16*)W3,
+                          (__nv_bfloat16*)W13p, I, cfg->d, unpack,
+                          (__nv_bfloat16*)W1o, (__nv_bfloat16*)W3o));
   else
-    pack_kernel<float><<<grid, 128, 0, as_stream(stream)>>>((const float*)W1, (const float*)W3, (float*)W13p, I, cfg->d,
-                                                            unpack, (float*)W1o, (float*)W3o);
+    C2R_CUDA(launch_chained(pack_kernel<float>, grid, 128, 0, as_stream(stream), (const float*)W1, (const float*)W3, (float*)W13p, I, cfg->d,
+                          unpack, (float*)W1o, (float*)W3o));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

@@ -131,14 +131,6 @@ skinny_kernel(const __grid_constant__ SkinnyMaps maps0, const __grid_constant__ 
   const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[SK_MAX_STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[2 * SK_MAX_STAGES]), tempty0 = smem_u32(&bars[2 * SK_MAX_STAGES + 2]);
-  for (int i = threadIdx.x; i < 64 * p.n_problems; i += blockDim.x) {
-    const int q = i >> 6, e = i & 63;
-    if (e < p.pr[q].nE) {
-      const int off = p.pr[q].offsets[e];
-      s_off[q][e] = off;
-      s_cnt[q][e] = (int)max(0ll, min((long long)p.pr[q].counts[e], p.pr[q].R - off));
-    }
-  }
   if (threadIdx.x == 0) {
     s_abort = 0;
     for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
@@ -149,6 +141,16 @@ skinny_kernel(const __grid_constant__ SkinnyMaps maps0, const __grid_constant__ 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    chain_release();  // not before: a block of the next kernel must not take the tensor memory this one waits for
+  }
+  chain_wait();  // before the first access to global memory
+  for (int i = threadIdx.x; i < 64 * p.n_problems; i += blockDim.x) {
+    const int q = i >> 6, e = i & 63;
+    if (e < p.pr[q].nE) {
+      const int off = p.pr[q].offsets[e];
+      s_off[q][e] = off;
+      s_cnt[q][e] = (int)max(0ll, min((long long)p.pr[q].counts[e], p.pr[q].R - off));
+    }
   }
   __syncthreads();
   if (warp < p.n_problems) {  // a warp per problem: exclusive scan of the experts' unit counts
@@ -420,7 +422,7 @@ static int skinny_launch(const c2r_config* cfg, const SwigluCall* calls, int n, 
     }
   }
   if (n == 1) maps[1] = maps[0];
-  skinny_kernel<<<sms, SK_THREADS, SK_SMEM, s>>>(maps[0], maps[1], p);
+  C2R_CUDA(launch_chained(skinny_kernel, sms, SK_THREADS, SK_SMEM, s, maps[0], maps[1], p));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

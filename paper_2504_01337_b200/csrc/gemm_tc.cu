@@ -274,29 +274,38 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
 
-  for (int i = threadIdx.x; i <= p.n_experts; i += blockDim.x) s_off[i] = p.offsets[i];
-  for (int i = threadIdx.x; i < p.n_experts; i += blockDim.x) s_cnt[i] = p.counts[i];
   if (threadIdx.x == 0) {
     s_abort = 0;
     for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull0 + 8 * b, 1); mbar_init(tempty0 + 8 * b, 2 * EPI_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int e = 0; e < p.n_experts; ++e) {
-      s_pt[e] = run;
-      const int rows = min(s_cnt[e], max(p.R - s_off[e], 0));
-      run += (rows + TILE_M - 1) / TILE_M;
-    }
-    s_pt[p.n_experts] = run;
-  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                  "r"(TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    chain_release();  // not before: a block of the next kernel must not take the tensor memory this one waits for
+  }
+  chain_wait();  // before the first access to global memory
+  for (int i = threadIdx.x; i <= p.n_experts; i += blockDim.x) s_off[i] = p.offsets[i];
+  for (int i = threadIdx.x; i < p.n_experts; i += blockDim.x) s_cnt[i] = p.counts[i];
+  __syncthreads();
+  if (warp == 0) {  // pair tiles before each expert
+    int run = 0;
+    for (int e0 = 0; e0 < p.n_experts; e0 += 32) {
+      const int e = e0 + lane;
+      const int v = e < p.n_experts ? (min(s_cnt[e], max(p.R - s_off[e], 0)) + TILE_M - 1) / TILE_M : 0;
+      int incl = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+      }
+      if (e < p.n_experts) s_pt[e] = run + incl - v;
+      run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_pt[p.n_experts] = run;
   }
   tc_fence_before();
   __syncthreads();
@@ -736,11 +745,13 @@ static int launch(const CUtensorMap& ma, const CUtensorMap& mb, const TcParams& 
   C2R_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= MAX_DEV) return C2R_ERR_UNSUPPORTED_SHAPE;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_chained
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(TC_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -758,6 +769,7 @@ static int launch(const CUtensorMap& ma, const CUtensorMap& mb, const TcParams& 
     __atomic_store_n(&grid_of_device[dev], grid, __ATOMIC_RELEASE);
   }
   cfg.gridDim = dim3(grid);
+  cfg.numAttrs = 2;
   C2R_CUDA(cudaLaunchKernelEx(&cfg, tc_gemm_kernel<A_MN, B_MN, GATHER, EPI>, ma, mb, p));
   C2R_LAUNCH_CHECK();
   return C2R_OK;

@@ -85,6 +85,7 @@ __device__ __forceinline__ void segment_offsets(const int* s_by_rank, const int*
 __global__ void __launch_bounds__(PERM_THREADS) perm_hist_kernel(const int32_t* __restrict__ idx, long long NK, int E,
                                                                  int slots_per_block, int32_t* __restrict__ block_counts,
                                                                  int32_t* __restrict__ status, int skip_negative) {
+  chain_begin();
   __shared__ int grp_cnt[PERM_GROUPS][64];
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) (&grp_cnt[0][0])[i] = 0;
   __syncthreads();
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ b
                                                          const int32_t* __restrict__ expert_rank, int row_align,
                                                          int32_t* __restrict__ counts, int32_t* __restrict__ offsets,
                                                          int32_t* __restrict__ status) {
+  chain_begin();
   __shared__ int s_counts[64];
   __shared__ int s_by_rank[64];
   __shared__ int s_bad;
@@ -167,6 +169,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_kernel(const int32_t* 
                                                                  int32_t* __restrict__ row_of_slot,
                                                                  int32_t* __restrict__ slot_of_row, int skip_negative,
                                                                  const float* __restrict__ w, float* __restrict__ w_row) {
+  chain_begin();
   __shared__ int grp_cnt[PERM_GROUPS][64];
   __shared__ int s_start[64];
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) (&grp_cnt[0][0])[i] = 0;
@@ -198,6 +201,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
                                                                        const float* __restrict__ w,
                                                                        float* __restrict__ w_row,
                                                                        int32_t* __restrict__ status) {
+  chain_begin();
   constexpr int PARTS = PERM_THREADS / 64;
   __shared__ int grp_cnt[PERM_GROUPS][64];
   __shared__ int s_start[64], s_total[64], s_by_rank[64], s_off[65];
@@ -273,6 +277,7 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__
                                                            int N, int d, int K, const int32_t* __restrict__ counts,
                                                            const int32_t* __restrict__ offsets, int token_blocks,
                                                            int row_align, int parts) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= token_blocks) {
@@ -316,6 +321,7 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__
 template <typename T>
 __global__ void __launch_bounds__(256) zero_pad_rows_kernel(const int32_t* __restrict__ slot_of_row, T* __restrict__ Xp,
                                                             long long R, int d) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   const int chunks = d / V::N;
@@ -360,6 +366,7 @@ __global__ void __launch_bounds__(256) gather_sum_kernel(const float* __restrict
                                                          const float* __restrict__ dl, const T* __restrict__ Wg,
                                                          const float* __restrict__ dz, const T* __restrict__ wsg,
                                                          T* __restrict__ out, int accumulate, int N, int d, int K, int parts) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -444,6 +451,7 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const T* __restrict__ 
                                                           T* __restrict__ dYp, float* __restrict__ dw,
                                                           T* __restrict__ dYs, float* __restrict__ dz, int N, int d,
                                                           int K) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -511,6 +519,7 @@ __global__ void __launch_bounds__(GW_WARPS * 32) gate_wgrad_kernel(const T* __re
                                                                    const int32_t* __restrict__ slot_of_row,
                                                                    const float* __restrict__ dl, float* __restrict__ dWg, int d,
                                                                    int accumulate) {
+  chain_begin();
   using V = Vec16<T>;
   __shared__ float part[GW_WARPS][32 * V::N + 4];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -557,6 +566,7 @@ constexpr int GWS_SPLITS = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) shared_gate_wgrad_kernel(const T* __restrict__ X, const float* __restrict__ dz,
                                                                 float* __restrict__ ws, int N, int d) {
+  chain_begin();
   using V = Vec16<T>;
   __shared__ float part[8][32 * V::N];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -590,6 +600,7 @@ __global__ void __launch_bounds__(256) shared_gate_wgrad_kernel(const T* __restr
 }
 
 __global__ void sum_splits_kernel(const float* __restrict__ ws, float* __restrict__ out, int d, int accumulate) {
+  chain_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d) return;
   float s = 0.f;
@@ -640,6 +651,7 @@ __global__ void __launch_bounds__(256) gate_dl_scatter_kernel(const int32_t* __r
                                                               const int32_t* __restrict__ slot_of_row,
                                                               const float* __restrict__ dl,
                                                               __nv_bfloat16* __restrict__ dLd, int K) {
+  chain_begin();
   const int e = blockIdx.x;
   const int r0 = offsets[e], n = counts[e];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -655,6 +667,7 @@ __global__ void __launch_bounds__(256) gate_dl_dense_kernel(const int32_t* __res
                                                             int N, int E, int K, int per, int splits,
                                                             int32_t* __restrict__ split_counts,
                                                             int32_t* __restrict__ split_offsets) {
+  chain_begin();
   if (blockIdx.x == 0 && (int)threadIdx.x <= splits) {
     const int lo = min(N, (int)threadIdx.x * per);
     split_offsets[threadIdx.x] = lo;
@@ -676,6 +689,7 @@ __global__ void __launch_bounds__(256) gate_dl_dense_kernel(const int32_t* __res
 __global__ void __launch_bounds__(256) gate_dz_kernel(const float* __restrict__ dz, __nv_bfloat16* __restrict__ dLd, int N,
                                                       int E, int per, int splits, int32_t* __restrict__ split_counts,
                                                       int32_t* __restrict__ split_offsets) {
+  chain_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (dz != nullptr && t < N) dLd[(size_t)t * GW_COLS + E] = __float2bfloat16_rn(dz[t]);
   if (blockIdx.x == 0 && threadIdx.x <= splits) {
@@ -687,6 +701,7 @@ __global__ void __launch_bounds__(256) gate_dz_kernel(const float* __restrict__ 
 __global__ void __launch_bounds__(256) gate_wgrad_reduce_kernel(const float* __restrict__ partial, int splits, int E, int d,
                                                                 float* __restrict__ dWg, float* __restrict__ dwsg,
                                                                 int accumulate) {
+  chain_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int e = blockIdx.y;  // 0..E: row E is the shared gate
   if (c >= d) return;
@@ -710,8 +725,8 @@ static int permute_rows_launch(const c2r_config* cfg, const T* X, const int32_t*
   const int token_blocks = (int)(((long long)cfg->N * parts + 7) / 8);
   const int pad_blocks = cfg->row_align > 1 ? cfg->E * PAD_BLOCKS : 0;
   if (token_blocks + pad_blocks == 0) return C2R_OK;
-  permute_rows_kernel<T><<<token_blocks + pad_blocks, 256, 0, s>>>(X, row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts, offsets,
-                                                                token_blocks, cfg->row_align, parts);
+  C2R_CUDA(launch_chained(permute_rows_kernel<T>, token_blocks + pad_blocks, 256, 0, s, X, row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts, offsets,
+                          token_blocks, cfg->row_align, parts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -729,21 +744,21 @@ int permute_impl(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
   int32_t* block_counts = (int32_t*)ws;
   if (w == nullptr) w_row = nullptr;
   if (nb > 0 && !have_hist) {
-    perm_hist_kernel<<<nb, PERM_THREADS, 0, s>>>(idx, NK, cfg->E, spb, block_counts, status, 0);
+    C2R_CUDA(launch_chained(perm_hist_kernel, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, status, 0));
     C2R_LAUNCH_CHECK();
   }
   if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
-    perm_rank_fused_kernel<<<nb, PERM_THREADS, 0, s>>>(idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
-                                                       R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status);
+    C2R_CUDA(launch_chained(perm_rank_fused_kernel, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
+                          R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status));
     C2R_LAUNCH_CHECK();
   } else {
     C2R_CUDA(cudaMemsetAsync(slot_of_row, 0xFF, sizeof(int32_t) * R, s));
     if (w_row != nullptr) C2R_CUDA(cudaMemsetAsync(w_row, 0, sizeof(float) * R, s));
-    perm_scan_kernel<<<1, 1024, 0, s>>>(block_counts, nb, cfg->E, expert_rank, cfg->row_align, counts, offsets, status);
+    C2R_CUDA(launch_chained(perm_scan_kernel, 1, 1024, 0, s, block_counts, nb, cfg->E, expert_rank, cfg->row_align, counts, offsets, status));
     C2R_LAUNCH_CHECK();
     if (nb > 0) {
-      perm_rank_kernel<<<nb, PERM_THREADS, 0, s>>>(idx, NK, cfg->E, spb, block_counts, offsets, row_of_slot, slot_of_row, 0,
-                                                   w, w_row);
+      C2R_CUDA(launch_chained(perm_rank_kernel, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, offsets, row_of_slot, slot_of_row, 0,
+                          w, w_row));
       C2R_LAUNCH_CHECK();
     }
   }
@@ -799,9 +814,9 @@ static int gather_sum_launch(const c2r_config* cfg, const void* src, const int32
   if (cfg->N == 0) return C2R_OK;
   const int parts = row_parts(cfg->N, (cfg->d / Vec16<T>::N + 31) / 32);
   const long long warps = (long long)cfg->N * parts;
-  gather_sum_kernel<T><<<(unsigned)((warps + 7) / 8), 256, 0, s>>>((const float*)src, rows, coef, (const float*)extra, z, idx, dl,
-                                                                   (const T*)Wg, dz, (const T*)wsg, (T*)out, accumulate, cfg->N,
-                                                                   cfg->d, cfg->K, parts);
+  C2R_CUDA(launch_chained(gather_sum_kernel<T>, (unsigned)((warps + 7) / 8), 256, 0, s, (const float*)src, rows, coef, (const float*)extra, z, idx, dl,
+                          (const T*)Wg, dz, (const T*)wsg, (T*)out, accumulate, cfg->N,
+                          cfg->d, cfg->K, parts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -839,14 +854,14 @@ static int combine_bwd_launch(const c2r_config* cfg, const void* dY, const void*
                               void* dYp, float* dw, void* dYs, float* dz, cudaStream_t s) {
   const long long R = permuted_rows(cfg);
   if (cfg->N > 0) {
-    combine_bwd_kernel<T><<<(cfg->N + 7) / 8, 256, 0, s>>>((const T*)dY, (const float*)Yp, w, rows, (const float*)Ys, z,
-                                                           (T*)dYp, dw, (T*)dYs, dz, cfg->N, cfg->d, cfg->K);
+    C2R_CUDA(launch_chained(combine_bwd_kernel<T>, (cfg->N + 7) / 8, 256, 0, s, (const T*)dY, (const float*)Yp, w, rows, (const float*)Ys, z,
+                          (T*)dYp, dw, (T*)dYs, dz, cfg->N, cfg->d, cfg->K));
     C2R_LAUNCH_CHECK();
   }
   if (R > (long long)cfg->N * cfg->K) {
     int blocks = (int)((R + 7) / 8);
     if (blocks > 1184) blocks = 1184;
-    zero_pad_rows_kernel<T><<<blocks, 256, 0, s>>>(slot_of_row, (T*)dYp, R, cfg->d);
+    C2R_CUDA(launch_chained(zero_pad_rows_kernel<T>, blocks, 256, 0, s, slot_of_row, (T*)dYp, R, cfg->d));
     C2R_LAUNCH_CHECK();
   }
   return C2R_OK;
@@ -879,31 +894,31 @@ static int gate_bwd_launch(const c2r_config* cfg, const void* X, const void* Xp,
     int32_t* sc = (int32_t*)((char*)ws + g.off_counts);
     int32_t* so = sc + g.splits;
     if (idx != nullptr) {
-      gate_dl_dense_kernel<<<(cfg->N + 7) / 8, 256, 0, s>>>(idx, dl, dz, dLd, cfg->N, cfg->E, cfg->K, g.per, g.splits, sc, so);
+      C2R_CUDA(launch_chained(gate_dl_dense_kernel, (cfg->N + 7) / 8, 256, 0, s, idx, dl, dz, dLd, cfg->N, cfg->E, cfg->K, g.per, g.splits, sc, so));
       C2R_LAUNCH_CHECK();
     } else {
       C2R_CUDA(cudaMemsetAsync(dLd, 0, (size_t)cfg->N * GW_COLS * 2, s));
-      gate_dl_scatter_kernel<<<cfg->E, 256, 0, s>>>(counts, offsets, slot_of_row, dl, dLd, cfg->K);
+      C2R_CUDA(launch_chained(gate_dl_scatter_kernel, cfg->E, 256, 0, s, counts, offsets, slot_of_row, dl, dLd, cfg->K));
       C2R_LAUNCH_CHECK();
-      gate_dz_kernel<<<(cfg->N + 255) / 256, 256, 0, s>>>(dz, dLd, cfg->N, cfg->E, g.per, g.splits, sc, so);
+      C2R_CUDA(launch_chained(gate_dz_kernel, (cfg->N + 255) / 256, 256, 0, s, dz, dLd, cfg->N, cfg->E, g.per, g.splits, sc, so));
       C2R_LAUNCH_CHECK();
     }
     int rc = tc_gate_wgrad(cfg, X, dLd, partial, g.splits, sc, so, nullptr, s);
     if (rc) return rc;
-    gate_wgrad_reduce_kernel<<<dim3((cfg->d + 255) / 256, cfg->E + 1), 256, 0, s>>>(partial, g.splits, cfg->E, cfg->d,
-                                                                                   dWg, dz ? dwsg : nullptr, accumulate);
+    C2R_CUDA(launch_chained(gate_wgrad_reduce_kernel, dim3((cfg->d + 255) / 256, cfg->E + 1), 256, 0, s, partial, g.splits, cfg->E, cfg->d,
+                          dWg, dz ? dwsg : nullptr, accumulate));
     C2R_LAUNCH_CHECK();
     return C2R_OK;
   }
   C2R_REQUIRE(Xp != nullptr, C2R_ERR_INVALID_ARG);  // the row-serial form walks the permuted rows
   const int colblocks = (cfg->d + 32 * V::N - 1) / (32 * V::N);
-  gate_wgrad_kernel<T><<<dim3(colblocks, cfg->E), GW_WARPS * 32, 0, s>>>((const T*)Xp, counts, offsets, slot_of_row, dl, dWg,
-                                                               cfg->d, accumulate);
+  C2R_CUDA(launch_chained(gate_wgrad_kernel<T>, dim3(colblocks, cfg->E), GW_WARPS * 32, 0, s, (const T*)Xp, counts, offsets, slot_of_row, dl, dWg,
+                          cfg->d, accumulate));
   C2R_LAUNCH_CHECK();
   if (dz) {
-    shared_gate_wgrad_kernel<T><<<dim3(colblocks, GWS_SPLITS), 256, 0, s>>>((const T*)X, dz, (float*)ws, cfg->N, cfg->d);
+    C2R_CUDA(launch_chained(shared_gate_wgrad_kernel<T>, dim3(colblocks, GWS_SPLITS), 256, 0, s, (const T*)X, dz, (float*)ws, cfg->N, cfg->d));
     C2R_LAUNCH_CHECK();
-    sum_splits_kernel<<<(cfg->d + 255) / 256, 256, 0, s>>>((const float*)ws, dwsg, cfg->d, accumulate);
+    C2R_CUDA(launch_chained(sum_splits_kernel, (cfg->d + 255) / 256, 256, 0, s, (const float*)ws, dwsg, cfg->d, accumulate));
     C2R_LAUNCH_CHECK();
   }
   return C2R_OK;
@@ -990,6 +1005,7 @@ namespace c2r {
 // key[t,k] = partition of slot (t,k) if no earlier slot of the token maps to that partition, else -1.
 __global__ void __launch_bounds__(256) dedup_keys_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ part,
                                                          int32_t* __restrict__ key, int N, int E, int K, int P) {
+  chain_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N) return;
   int q[8];
@@ -1006,6 +1022,7 @@ __global__ void __launch_bounds__(256) dedup_keys_kernel(const int32_t* __restri
 __global__ void __launch_bounds__(256) dedup_fill_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ part,
                                                          const int32_t* __restrict__ key,
                                                          int32_t* __restrict__ recv_row_of_slot, int N, int E, int K, int P) {
+  chain_begin();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N) return;
   for (int k = 1; k < K; ++k) {
@@ -1018,6 +1035,7 @@ __global__ void __launch_bounds__(256) dedup_fill_kernel(const int32_t* __restri
 
 __global__ void __launch_bounds__(256) dedup_tokens_kernel(const int32_t* __restrict__ slot_of_recv_row,
                                                            int32_t* __restrict__ token_of_recv_row, long long cap, int K) {
+  chain_begin();
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= cap) return;
   const int s = slot_of_recv_row[r];
@@ -1030,6 +1048,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) dedup_send_kernel(const T* __restrict__ X, const int32_t* __restrict__ key,
                                                          const int32_t* __restrict__ recv_row_of_slot, T* __restrict__ Xr,
                                                          int N, int d, int K) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1055,6 +1074,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) dedup_replicate_kernel(const T* __restrict__ Xr, const int32_t* __restrict__ slot_of_row,
                                                               const int32_t* __restrict__ recv_row_of_slot,
                                                               T* __restrict__ Xp, long long R, int d) {
+  chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
   const long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1103,29 +1123,29 @@ static int dispatch_dedup_impl(const c2r_config* cfg, const int32_t* idx, const 
   const int nb = perm_blocks(cfg);
   const int spb = perm_tokens_per_block(K) * K;
   if (N > 0) {
-    dedup_keys_kernel<<<(N + 255) / 256, 256, 0, s>>>(idx, part, key, N, E, K, P);
+    C2R_CUDA(launch_chained(dedup_keys_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, N, E, K, P));
     C2R_LAUNCH_CHECK();
-    C2R_CUDA(cudaMemsetAsync(slot_of_recv_row, 0xFF, sizeof(int32_t) * NK, s));
-    perm_hist_kernel<<<nb, PERM_THREADS, 0, s>>>(key, NK, P, spb, block_counts, status, 1);
+    if ((rc = fill_words((uint32_t*)slot_of_recv_row, NK, nullptr, 0, nullptr, 0, ~0u, s))) return rc;
+    C2R_CUDA(launch_chained(perm_hist_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, status, 1));
     C2R_LAUNCH_CHECK();
   }
-  perm_scan_kernel<<<1, 1024, 0, s>>>(block_counts, nb, P, nullptr, 1, recv_counts, recv_offsets, nullptr);
+  C2R_CUDA(launch_chained(perm_scan_kernel, 1, 1024, 0, s, block_counts, nb, P, nullptr, 1, recv_counts, recv_offsets, nullptr));
   C2R_LAUNCH_CHECK();
   if (N > 0) {
-    perm_rank_kernel<<<nb, PERM_THREADS, 0, s>>>(key, NK, P, spb, block_counts, recv_offsets, recv_row_of_slot,
-                                                 slot_of_recv_row, 1, nullptr, nullptr);
+    C2R_CUDA(launch_chained(perm_rank_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, recv_offsets, recv_row_of_slot,
+                          slot_of_recv_row, 1, nullptr, nullptr));
     C2R_LAUNCH_CHECK();
-    dedup_fill_kernel<<<(N + 255) / 256, 256, 0, s>>>(idx, part, key, recv_row_of_slot, N, E, K, P);
+    C2R_CUDA(launch_chained(dedup_fill_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, recv_row_of_slot, N, E, K, P));
     C2R_LAUNCH_CHECK();
-    dedup_tokens_kernel<<<(int)((cap + 255) / 256), 256, 0, s>>>(slot_of_recv_row, token_of_recv_row, cap, K);
+    C2R_CUDA(launch_chained(dedup_tokens_kernel, (int)((cap + 255) / 256), 256, 0, s, slot_of_recv_row, token_of_recv_row, cap, K));
     C2R_LAUNCH_CHECK();
     if (X != nullptr) {
-      dedup_send_kernel<T><<<(N + 7) / 8, 256, 0, s>>>(X, key, recv_row_of_slot, Xr, N, cfg->d, K);
+      C2R_CUDA(launch_chained(dedup_send_kernel<T>, (N + 7) / 8, 256, 0, s, X, key, recv_row_of_slot, Xr, N, cfg->d, K));
       C2R_LAUNCH_CHECK();
     }
   }
   if (X != nullptr && R > 0) {
-    dedup_replicate_kernel<T><<<(int)((R + 7) / 8), 256, 0, s>>>(Xr, slot_of_row, recv_row_of_slot, Xp, R, cfg->d);
+    C2R_CUDA(launch_chained(dedup_replicate_kernel<T>, (int)((R + 7) / 8), 256, 0, s, Xr, slot_of_row, recv_row_of_slot, Xp, R, cfg->d));
     C2R_LAUNCH_CHECK();
   }
   return C2R_OK;

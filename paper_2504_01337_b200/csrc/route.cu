@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(512) route_kernel(const float* __restrict__ L,
                                                     int32_t* __restrict__ idx, float* __restrict__ w, float* __restrict__ p,
                                                     int32_t* __restrict__ status, int N, int E, int renorm, int tokens_per_block,
                                                     int32_t* __restrict__ block_counts) {
+  chain_begin();
   extern __shared__ uint32_t s_key[];  // [tokens][route_pitch(E)]
   __shared__ uint64_t s_mask[64];
   __shared__ int s_cnt[64];
@@ -197,14 +198,15 @@ static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* m
       __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
     }
   }
-  route_kernel<K><<<(cfg->N + tpb - 1) / tpb, threads, smem, s>>>(L, mask, idx, w, p, status, cfg->N, cfg->E, cfg->renorm, tpb,
-                                                                 block_counts);
+  C2R_CUDA(launch_chained(route_kernel<K>, (cfg->N + tpb - 1) / tpb, threads, smem, s, L, mask, idx, w, p, status, cfg->N, cfg->E, cfg->renorm, tpb,
+                          block_counts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
 
 __global__ void route_bwd_kernel(const float* __restrict__ w, const float* __restrict__ dw, float* __restrict__ dl,
                                  int N, int K) {
+  chain_begin();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N) return;
   float s = 0.f;
@@ -225,6 +227,7 @@ __global__ void __launch_bounds__(RBS_TOKENS * 8) route_bwd_scaled_kernel(const 
                                                                           const float* __restrict__ qspart, int nqs,
                                                                           float* __restrict__ dw, float* __restrict__ dl,
                                                                           float* __restrict__ dz, int N, int K) {
+  chain_begin();
   __shared__ float s_q[RBS_TOKENS * 8];
   const int lt = threadIdx.x / K, k = threadIdx.x - lt * K;  // token of the block, slot of the token
   const int t = blockIdx.x * RBS_TOKENS + lt;
@@ -249,11 +252,22 @@ __global__ void __launch_bounds__(RBS_TOKENS * 8) route_bwd_scaled_kernel(const 
   }
 }
 
+// Up to three arrays of 32-bit words set to a value: a kernel, because a memset between two kernels would end their chain
+// (see launch_chained), and one launch instead of three memsets where the arrays are separate.
+__global__ void __launch_bounds__(256) fill_words_kernel(uint32_t* __restrict__ a, long long na, uint32_t* __restrict__ b, long long nb,
+                                                         uint32_t* __restrict__ c, long long nc, uint32_t value) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < na; i += step) a[i] = value;
+  for (long long i = first; i < nb; i += step) b[i] = value;
+  for (long long i = first; i < nc; i += step) c[i] = value;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Collaboration matrix (Eq. 2): per-block table in shared memory, merged with integer adds.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) collab_count_kernel(const int32_t* __restrict__ idx, long long n_tokens,
                                                            int32_t* __restrict__ C, int E, int K) {
+  chain_begin();
   extern __shared__ int32_t tab[];
   for (int i = threadIdx.x; i < E * E; i += blockDim.x) tab[i] = 0;
   __syncthreads();
@@ -275,6 +289,7 @@ __global__ void __launch_bounds__(256) collab_count_kernel(const int32_t* __rest
 // Top-T sets (Eq. 4): one warp per row; T rounds of arg-max under (count desc, index asc), self excluded.
 __global__ void collab_sets_kernel(const int32_t* __restrict__ C, int32_t* __restrict__ I_T,
                                    uint64_t* __restrict__ mask, int E, int T) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= E) return;
@@ -303,6 +318,7 @@ __global__ void collab_sets_kernel(const int32_t* __restrict__ C, int32_t* __res
 // columns, and a fixed-order sum over rows for the layer mean.
 __global__ void __launch_bounds__(1024) collab_degree_kernel(const int32_t* __restrict__ C, float* __restrict__ degree,
                                                              float* __restrict__ mean, int E) {
+  chain_begin();
   __shared__ float s_deg[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = warp; i < E; i += 32) {
@@ -338,6 +354,7 @@ __global__ void __launch_bounds__(256) dispatch_volume_kernel(const int32_t* __r
                                                               unsigned long long* __restrict__ send_naive,
                                                               unsigned long long* __restrict__ send_dedup, int N,
                                                               int E, int K, int P) {
+  chain_begin();
   extern __shared__ uint32_t sm[];
   uint32_t* s_naive = sm;           // [P*P]
   uint32_t* s_dedup = sm + P * P;   // [P*P]
@@ -376,6 +393,15 @@ __global__ void __launch_bounds__(256) dispatch_volume_kernel(const int32_t* __r
 }  // namespace c2r
 
 using namespace c2r;
+
+int c2r::fill_words(uint32_t* a, int64_t na, uint32_t* b, int64_t nb, uint32_t* c, int64_t nc, uint32_t value, cudaStream_t s) {
+  const int64_t most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
+  if (most <= 0) return C2R_OK;
+  const int blocks = (int)(most > 592 * 1024 ? 592 : (most + 1023) / 1024);
+  C2R_CUDA(launch_chained(fill_words_kernel, blocks, 256, 0, s, a, na, b, nb, c, nc, value));
+  C2R_LAUNCH_CHECK();
+  return C2R_OK;
+}
 
 extern "C" int c2r_last_cuda_error(void) { return g_last_cuda_error; }
 
@@ -434,8 +460,8 @@ extern "C" int c2r_route_bwd_scaled(const c2r_config* cfg, const float* w, const
   C2R_REQUIRE(!dz || (z && qspart && nqs >= 0), C2R_ERR_INVALID_ARG);
   C2R_REQUIRE(cfg->renorm == 1, C2R_ERR_UNSUPPORTED_SHAPE);
   if (cfg->N == 0) return C2R_OK;
-  route_bwd_scaled_kernel<<<(cfg->N + RBS_TOKENS - 1) / RBS_TOKENS, RBS_TOKENS * cfg->K, 0, as_stream(stream)>>>(w, row_of_slot, qpart, nq, permuted_rows(cfg),
-                                                                              z, qspart, nqs, dw, dl, dz, cfg->N, cfg->K);
+  C2R_CUDA(launch_chained(route_bwd_scaled_kernel, (cfg->N + RBS_TOKENS - 1) / RBS_TOKENS, RBS_TOKENS * cfg->K, 0, as_stream(stream), w, row_of_slot, qpart, nq, permuted_rows(cfg),
+                          z, qspart, nqs, dw, dl, dz, cfg->N, cfg->K));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -446,7 +472,7 @@ extern "C" int c2r_route_bwd(const c2r_config* cfg, const float* w, const float*
   C2R_REQUIRE(w && dw && dl, C2R_ERR_INVALID_ARG);
   C2R_REQUIRE(cfg->renorm == 1, C2R_ERR_UNSUPPORTED_SHAPE);
   if (cfg->N == 0) return C2R_OK;
-  route_bwd_kernel<<<(cfg->N + 255) / 256, 256, 0, as_stream(stream)>>>(w, dw, dl, cfg->N, cfg->K);
+  C2R_CUDA(launch_chained(route_bwd_kernel, (cfg->N + 255) / 256, 256, 0, as_stream(stream), w, dw, dl, cfg->N, cfg->K));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -457,12 +483,12 @@ extern "C" int c2r_collab_count(const c2r_config* cfg, const int32_t* idx, int64
   if (rc) return rc;
   C2R_REQUIRE(idx && C && n_tokens >= 0, C2R_ERR_INVALID_ARG);
   const int E = cfg->E;
-  if (!accumulate) C2R_CUDA(cudaMemsetAsync(C, 0, sizeof(int32_t) * E * E, as_stream(stream)));
+  if (!accumulate && (rc = fill_words((uint32_t*)C, E * E, nullptr, 0, nullptr, 0, 0u, as_stream(stream)))) return rc;
   if (n_tokens == 0) return C2R_OK;
   int blocks = (int)((n_tokens + 255) / 256);
   if (blocks > 296) blocks = 296;
-  collab_count_kernel<<<blocks, 256, sizeof(int32_t) * E * E, as_stream(stream)>>>(idx, (long long)n_tokens, C, E,
-                                                                                 cfg->K);
+  C2R_CUDA(launch_chained(collab_count_kernel, blocks, 256, sizeof(int32_t) * E * E, as_stream(stream), idx, (long long)n_tokens, C, E,
+                          cfg->K));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -473,7 +499,7 @@ extern "C" int c2r_collab_sets(const c2r_config* cfg, const int32_t* C, int32_t*
   C2R_REQUIRE(C && I_T && mask, C2R_ERR_INVALID_ARG);
   C2R_REQUIRE(cfg->T >= 0 && cfg->T <= cfg->E - 1, C2R_ERR_INVALID_ARG);
   const int warps = 4;
-  collab_sets_kernel<<<(cfg->E + warps - 1) / warps, warps * 32, 0, as_stream(stream)>>>(C, I_T, mask, cfg->E, cfg->T);
+  C2R_CUDA(launch_chained(collab_sets_kernel, (cfg->E + warps - 1) / warps, warps * 32, 0, as_stream(stream), C, I_T, mask, cfg->E, cfg->T));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -482,7 +508,7 @@ extern "C" int c2r_collab_degree(const c2r_config* cfg, const int32_t* C, float*
   int rc = check_config(cfg);
   if (rc) return rc;
   C2R_REQUIRE(C && degree, C2R_ERR_INVALID_ARG);
-  collab_degree_kernel<<<1, 1024, 0, as_stream(stream)>>>(C, degree, mean, cfg->E);
+  C2R_CUDA(launch_chained(collab_degree_kernel, 1, 1024, 0, as_stream(stream), C, degree, mean, cfg->E));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -495,20 +521,14 @@ extern "C" int c2r_dispatch_volume(const c2r_config* cfg, const int32_t* idx, co
   const int P = cfg->P;
   C2R_REQUIRE(P >= 1 && P <= cfg->E, C2R_ERR_INVALID_ARG);
   cudaStream_t s = as_stream(stream);
-  if (send_naive == totals + 4 && send_dedup == send_naive + P * P) {  // one buffer (the layer drivers' layout)
-    C2R_CUDA(cudaMemsetAsync(totals, 0, sizeof(uint64_t) * (4 + 2 * P * P), s));
-  } else {
-    C2R_CUDA(cudaMemsetAsync(totals, 0, 4 * sizeof(uint64_t), s));
-    C2R_CUDA(cudaMemsetAsync(send_naive, 0, sizeof(uint64_t) * P * P, s));
-    C2R_CUDA(cudaMemsetAsync(send_dedup, 0, sizeof(uint64_t) * P * P, s));
-  }
+  if ((rc = fill_words((uint32_t*)totals, 8, (uint32_t*)send_naive, 2 * P * P, (uint32_t*)send_dedup, 2 * P * P, 0u, s))) return rc;
   if (cfg->N == 0) return C2R_OK;
   int blocks = (cfg->N + 255) / 256;
   if (blocks > 296) blocks = 296;
   size_t smem = sizeof(uint32_t) * (2 * P * P + cfg->E);
-  dispatch_volume_kernel<<<blocks, 256, smem, s>>>(idx, part, (unsigned long long*)totals,
-                                                   (unsigned long long*)send_naive, (unsigned long long*)send_dedup,
-                                                   cfg->N, cfg->E, cfg->K, P);
+  C2R_CUDA(launch_chained(dispatch_volume_kernel, blocks, 256, smem, s, idx, part, (unsigned long long*)totals,
+                          (unsigned long long*)send_naive, (unsigned long long*)send_dedup,
+                          cfg->N, cfg->E, cfg->K, P));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
