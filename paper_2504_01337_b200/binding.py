@@ -115,8 +115,6 @@ def make_config(N, d, E, I, K, T=0, P=1, I_s=0, dtype=BF16, row_align=1, renorm=
 
 
 def _ptr(t):
-    if t is None:
-        return None
     if isinstance(t, torch.Tensor):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("expected a contiguous CUDA tensor")
@@ -132,12 +130,23 @@ def _host_ptr(t):
     return t.data_ptr()
 
 
+# The current stream's handle without a Stream object around it: short calls (a calibration pass is four) are bound by what
+# happens here before the launch.
+_current_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else torch.cuda.current_device
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
+
+
+_FN = {name: getattr(lib, name) for name in _SIGS}
 
 
 def _call(name, *args):
-    rc = getattr(lib, name)(*args)
+    rc = _FN[name](*args)
     if rc != 0:
         raise C2RError(name, rc)
 
