@@ -16,14 +16,14 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// Expert key of slot s (clamped into [0,E); -1 = the slot takes no part: past the end, or a key of -1 when
+// Expert key of slot s (clamped into [0,E); -1 = the slot takes no part: past the end, or a negative key when
 // skip_negative is set, which the de-duplicated dispatch uses).
 __device__ __forceinline__ int slot_key(const int32_t* __restrict__ idx, long long s, long long NK, int E, int skip_negative,
                                         int& flags) {
   if (s >= NK) return -1;
   int e = idx[s];
   if (e < 0 || e >= E) {
-    if (skip_negative && e == -1) return -1;
+    if (skip_negative && e < 0) return -1;
     flags |= C2R_STATUS_BAD_INDEX;
     e = min(max(e, 0), E - 1);
   }
@@ -136,11 +136,11 @@ __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ b
 
 // Stable rank of a block's slots once grp_cnt holds the per-group counts and s_start[e] the row at which the
 // block's first slot of expert e lands: rows of earlier groups of the block, then lower lanes of the group.
-// w (optional): w_row[row] = w[slot], the routing weight of the slot that owns the row.
+// w (optional): w_row[row] = w[slot], the routing weight of the slot that owns the row.  slot_of_row gets slot / slot_div.
 __device__ __forceinline__ void rank_and_write(int e, long long NK, int E, int slots_per_block, int (*grp_cnt)[64],
                                                const int* s_start, int32_t* __restrict__ row_of_slot,
                                                int32_t* __restrict__ slot_of_row, const float* __restrict__ w,
-                                               float* __restrict__ w_row) {
+                                               float* __restrict__ w_row, int slot_div = 1, int* my_row = nullptr) {
   for (int x = threadIdx.x; x < E; x += blockDim.x) {
     int run = s_start[x];
 #pragma unroll
@@ -157,8 +157,9 @@ __device__ __forceinline__ void rank_and_write(int e, long long NK, int E, int s
     const long long s = (long long)blockIdx.x * slots_per_block + threadIdx.x;
     const int row = grp_cnt[g][e] + __popc(peers & lanemask_lt());
     row_of_slot[s] = row;
-    slot_of_row[row] = (int32_t)s;
+    slot_of_row[row] = slot_div == 1 ? (int32_t)s : (int32_t)(s / slot_div);
     if (w_row != nullptr) w_row[row] = w[s];
+    if (my_row != nullptr) *my_row = row;
   }
 }
 
@@ -187,7 +188,12 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_kernel(const int32_t* 
 // that hold no slot (the padding that closes every aligned segment and the rows past the layout's end, up
 // to R) with -1 in slot_of_row and 0 in w_row, so the call needs no memset: two launches fewer and one
 // dependent round trip fewer than memset -> hist -> scan -> rank.
+//
+// DEDUP (the receive side of the two-stage dispatch): idx holds the partition q for the first slot of every (token,
+// partition), else -2 - q; first slots get their rows, the others the row of the token's first slot with the same partition,
+// and slot_of_row holds tokens (slot / K).
 constexpr int PERM_FUSED_MAX_BLOCKS = 1024;
+template <bool DEDUP>
 __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int32_t* __restrict__ idx, long long NK, int E,
                                                                        int slots_per_block,
                                                                        const int32_t* __restrict__ block_counts,
@@ -200,7 +206,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
                                                                        int32_t* __restrict__ slot_of_row,
                                                                        const float* __restrict__ w,
                                                                        float* __restrict__ w_row,
-                                                                       int32_t* __restrict__ status) {
+                                                                       int32_t* __restrict__ status, int K) {
   chain_begin();
   constexpr int PARTS = PERM_THREADS / 64;
   __shared__ int grp_cnt[PERM_GROUPS][64];
@@ -234,7 +240,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
   segment_offsets(s_by_rank, s_total, E, row_align, s_off);
   if (threadIdx.x == 0 && blockIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
   int flags = 0;
-  const int e_mine = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, 0);
+  const int e_mine = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, DEDUP);
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int e = threadIdx.x; e <= E; e += blockDim.x) {
@@ -257,7 +263,22 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
   }
   for (int e = threadIdx.x; e < E; e += blockDim.x) s_start[e] += s_off[e];
   __syncthreads();
-  rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, w, w_row);
+  if constexpr (!DEDUP) {
+    rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, w, w_row);
+  } else {
+    __shared__ int s_row[PERM_THREADS], s_q[PERM_THREADS];
+    int row = -1;
+    rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, nullptr, nullptr, K, &row);
+    s_row[threadIdx.x] = row;
+    s_q[threadIdx.x] = e_mine;
+    __syncthreads();
+    const long long slot = (long long)blockIdx.x * slots_per_block + threadIdx.x;
+    if ((int)threadIdx.x < slots_per_block && slot < NK && e_mine < 0) {  // a block owns whole tokens
+      const int q = -2 - idx[slot];
+      for (int j = threadIdx.x / K * K; j < (int)threadIdx.x; ++j)
+        if (s_q[j] == q) { row_of_slot[slot] = s_row[j]; break; }
+    }
+  }
 }
 
 // Warps over which a token's row is spread where there are few tokens: enough for 32 warps per SM, each with at least one
@@ -748,8 +769,8 @@ int permute_impl(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
     C2R_LAUNCH_CHECK();
   }
   if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
-    C2R_CUDA(launch_chained(perm_rank_fused_kernel, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
-                          R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status));
+    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
+                          R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status, (int)cfg->K));
     C2R_LAUNCH_CHECK();
   } else {
     C2R_CUDA(cudaMemsetAsync(slot_of_row, 0xFF, sizeof(int32_t) * R, s));
@@ -1042,58 +1063,107 @@ __global__ void __launch_bounds__(256) dedup_tokens_kernel(const int32_t* __rest
   token_of_recv_row[r] = s >= 0 ? s / K : -1;
 }
 
-// Stage 1, one warp per token: the token's row is read once and written to the receive row of every
-// partition that needs it.
-template <typename T>
-__global__ void __launch_bounds__(256) dedup_send_kernel(const T* __restrict__ X, const int32_t* __restrict__ key,
-                                                         const int32_t* __restrict__ recv_row_of_slot, T* __restrict__ Xr,
-                                                         int N, int d, int K) {
+// Both histograms of the two-stage dispatch in one pass, a thread per slot: slots per expert (the plain dispatch's), and
+// first slots of a token per partition.  Leaves the receive side's key of every slot (see perm_rank_fused_kernel).
+__global__ void __launch_bounds__(PERM_THREADS) dedup_hist_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ part,
+                                                                  long long NK, int E, int K, int P, int slots_per_block,
+                                                                  int32_t* __restrict__ expert_counts,
+                                                                  int32_t* __restrict__ part_counts, int32_t* __restrict__ key,
+                                                                  int32_t* __restrict__ status) {
   chain_begin();
-  using V = Vec16<T>;
-  const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= N) return;  // warp-uniform
-  int my_row = -1;
-  if (lane < K && key[(size_t)t * K + lane] >= 0) my_row = recv_row_of_slot[(size_t)t * K + lane];
-  int rows[8];
+  __shared__ int grp_cnt[PERM_GROUPS][64], grp_cnt_p[PERM_GROUPS][64];
+  __shared__ int s_q[PERM_THREADS];
+  for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) { (&grp_cnt[0][0])[i] = 0; (&grp_cnt_p[0][0])[i] = 0; }
+  __syncthreads();
+  int flags = 0;
+  const int e = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, 0);
+  const int q = e >= 0 ? min(max(part[e], 0), P - 1) : -1;
+  s_q[threadIdx.x] = q;
+  __syncthreads();
+  int first = q;
+  for (int j = threadIdx.x / K * K; j < (int)threadIdx.x; ++j)
+    if (s_q[j] == q) first = -1;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const uint32_t peers = __match_any_sync(0xffffffffu, first);
+  if (first >= 0 && lane == __ffs(peers) - 1) grp_cnt_p[g][first] = __popc(peers);
+  if (e >= 0) key[(long long)blockIdx.x * slots_per_block + threadIdx.x] = first >= 0 ? first : -2 - q;
+  __syncthreads();
+  for (int x = threadIdx.x; x < E; x += blockDim.x) {
+    int sum = 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) rows[k] = __shfl_sync(0xffffffffu, my_row, k);
-  const int chunks = d / V::N;
-  const T* src = X + (size_t)t * d;
-  for (int c = lane; c < chunks; c += 32) {
-    V v;
-    v.load(src + (size_t)c * V::N);
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < K && rows[k] >= 0) v.store(Xr + (size_t)rows[k] * d + (size_t)c * V::N);
+    for (int y = 0; y < PERM_GROUPS; ++y) sum += grp_cnt[y][x];
+    expert_counts[(size_t)blockIdx.x * E + x] = sum;
   }
+  for (int x = threadIdx.x; x < P; x += blockDim.x) {
+    int sum = 0;
+#pragma unroll
+    for (int y = 0; y < PERM_GROUPS; ++y) sum += grp_cnt_p[y][x];
+    part_counts[(size_t)blockIdx.x * P + x] = sum;
+  }
+  if (status != nullptr && flags) atomicOr(status, flags);
 }
 
-// Stage 2, one warp per row of the per-expert layout: Xp[r] = Xr[recv_row_of_slot[slot_of_row[r]]], padding rows zero.
+// The rows of both stages: `parts` warps per token read its row once and write it to the receive row of every partition
+// that needs it and to its K rows of the per-expert layout, which are what replication from the receive buffer would give.
+// Blocks past the token blocks zero the rows of that layout that hold no slot.  Bound by the bytes (16384 tokens of 2048, top-4,
+// 4 partitions: 507 MB; two kernels, of which the second read the receive buffer again, took 110 us, this one 95).
 template <typename T>
-__global__ void __launch_bounds__(256) dedup_replicate_kernel(const T* __restrict__ Xr, const int32_t* __restrict__ slot_of_row,
-                                                              const int32_t* __restrict__ recv_row_of_slot,
-                                                              T* __restrict__ Xp, long long R, int d) {
+__global__ void __launch_bounds__(256) dedup_rows_kernel(const T* __restrict__ X, const int32_t* __restrict__ key,
+                                                         const int32_t* __restrict__ recv_row_of_slot,
+                                                         const int32_t* __restrict__ row_of_slot,
+                                                         const int32_t* __restrict__ slot_of_row, T* __restrict__ Xr,
+                                                         T* __restrict__ Xp, int N, int d, int K, long long R, int token_blocks,
+                                                         int parts) {
   chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
-  const long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= R) return;  // warp-uniform
-  const int s = slot_of_row[r];
   const int chunks = d / V::N;
-  T* dst = Xp + (size_t)r * d;
-  if (s < 0) {
+  if ((int)blockIdx.x >= token_blocks) {
     V zero;
     float zf[V::N] = {};
     zero.from_float(zf);
-    for (int c = lane; c < chunks; c += 32) zero.store(dst + (size_t)c * V::N);
+    const long long step = (long long)(gridDim.x - token_blocks) * (blockDim.x >> 5);
+    for (long long r = (long long)(blockIdx.x - token_blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += step) {
+      if (slot_of_row[r] >= 0) continue;
+      for (int c = lane; c < chunks; c += 32) zero.store(Xp + (size_t)r * d + (size_t)c * V::N);
+    }
     return;
   }
-  const T* src = Xr + (size_t)recv_row_of_slot[s] * d;
-  for (int c = lane; c < chunks; c += 32) {
-    V v;
-    v.load(src + (size_t)c * V::N);
-    v.store(dst + (size_t)c * V::N);
+  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int t = (int)(wid / parts), part = (int)(wid - (long long)t * parts);
+  if (t >= N) return;  // warp-uniform
+  int my_row = 0, my_recv = -1;
+  if (lane < K) {
+    my_row = row_of_slot[(size_t)t * K + lane];
+    if (key[(size_t)t * K + lane] >= 0) my_recv = recv_row_of_slot[(size_t)t * K + lane];
+  }
+  int rows[8], recv[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    rows[k] = __shfl_sync(0xffffffffu, my_row, k);
+    recv[k] = __shfl_sync(0xffffffffu, my_recv, k);
+  }
+  const T* src = X + (size_t)t * d;
+  const int step = 32 * parts;
+  for (int c0 = 32 * part + lane; c0 < chunks; c0 += step * 4) {
+    V v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + step * u < chunks) v[u].load(src + (size_t)(c0 + step * u) * V::N);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k >= K) break;
+      T* dst = Xp + (size_t)rows[k] * d;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c0 + step * u < chunks) v[u].store(dst + (size_t)(c0 + step * u) * V::N);
+      if (recv[k] >= 0) {
+        dst = Xr + (size_t)recv[k] * d;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + step * u < chunks) v[u].store(dst + (size_t)(c0 + step * u) * V::N);
+      }
+    }
   }
 }
 
@@ -1113,40 +1183,57 @@ static int dispatch_dedup_impl(const c2r_config* cfg, const int32_t* idx, const 
   const long long NK = (long long)N * K;
   const long long R = permuted_rows(cfg);
   const long long cap = (long long)N * (K < P ? K : P);  // rows the receive side can need
-  // the per-expert layout itself (counts, offsets, both row maps) is the plain dispatch's
-  int rc = permute_impl<T>(cfg, idx, expert_rank, nullptr, counts, offsets, row_of_slot, slot_of_row, nullptr, status, ws, s,
-                           false, nullptr, nullptr);
-  if (rc) return rc;
-  int32_t* block_counts = (int32_t*)ws;  // free again: the calls above are ordered on the stream
+  int32_t* block_counts = (int32_t*)ws;
   int32_t* key = (int32_t*)((char*)ws + align256_(permute_ws_bytes(cfg)));
-  int32_t* slot_of_recv_row = (int32_t*)((char*)key + align256_(sizeof(int32_t) * (NK > 0 ? NK : 1)));
+  int32_t* scratch = (int32_t*)((char*)key + align256_(sizeof(int32_t) * (NK > 0 ? NK : 1)));
   const int nb = perm_blocks(cfg);
   const int spb = perm_tokens_per_block(K) * K;
-  if (N > 0) {
-    C2R_CUDA(launch_chained(dedup_keys_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, N, E, K, P));
+  if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
+    // Three launches for both indices (eleven took 39 us of 16384 tokens' dispatch).  scratch: [nb][P] block counts, which fit:
+    // a block but the last owns at least 448 slots and P is at most 64, and the area is a whole number of 256 bytes.
+    C2R_CUDA(launch_chained(dedup_hist_kernel, nb, PERM_THREADS, 0, s, idx, part, NK, E, K, P, spb, block_counts, scratch, key,
+                            status));
     C2R_LAUNCH_CHECK();
-    if ((rc = fill_words((uint32_t*)slot_of_recv_row, NK, nullptr, 0, nullptr, 0, ~0u, s))) return rc;
-    C2R_CUDA(launch_chained(perm_hist_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, status, 1));
+    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, nb, PERM_THREADS, 0, s, idx, NK, E, spb, block_counts, nb, expert_rank,
+                            cfg->row_align, R, counts, offsets, row_of_slot, slot_of_row, nullptr, nullptr, status, K));
     C2R_LAUNCH_CHECK();
-  }
-  C2R_CUDA(launch_chained(perm_scan_kernel, 1, 1024, 0, s, block_counts, nb, P, nullptr, 1, recv_counts, recv_offsets, nullptr));
-  C2R_LAUNCH_CHECK();
-  if (N > 0) {
-    C2R_CUDA(launch_chained(perm_rank_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, recv_offsets, recv_row_of_slot,
-                          slot_of_recv_row, 1, nullptr, nullptr));
+    C2R_CUDA(launch_chained(perm_rank_fused_kernel<true>, nb, PERM_THREADS, 0, s, key, NK, P, spb, scratch, nb, nullptr, 1, cap,
+                            recv_counts, recv_offsets, recv_row_of_slot, token_of_recv_row, nullptr, nullptr, nullptr, K));
     C2R_LAUNCH_CHECK();
-    C2R_CUDA(launch_chained(dedup_fill_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, recv_row_of_slot, N, E, K, P));
+  } else {
+    // the per-expert layout itself (counts, offsets, both row maps) is the plain dispatch's
+    int rc = permute_impl<T>(cfg, idx, expert_rank, nullptr, counts, offsets, row_of_slot, slot_of_row, nullptr, status, ws, s,
+                             false, nullptr, nullptr);
+    if (rc) return rc;
+    int32_t* slot_of_recv_row = scratch;
+    if (N > 0) {
+      C2R_CUDA(launch_chained(dedup_keys_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, N, E, K, P));
+      C2R_LAUNCH_CHECK();
+      if ((rc = fill_words((uint32_t*)slot_of_recv_row, NK, nullptr, 0, nullptr, 0, ~0u, s))) return rc;
+      C2R_CUDA(launch_chained(perm_hist_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, status, 1));
+      C2R_LAUNCH_CHECK();
+    }
+    C2R_CUDA(launch_chained(perm_scan_kernel, 1, 1024, 0, s, block_counts, nb, P, nullptr, 1, recv_counts, recv_offsets, nullptr));
     C2R_LAUNCH_CHECK();
-    C2R_CUDA(launch_chained(dedup_tokens_kernel, (int)((cap + 255) / 256), 256, 0, s, slot_of_recv_row, token_of_recv_row, cap, K));
-    C2R_LAUNCH_CHECK();
-    if (X != nullptr) {
-      C2R_CUDA(launch_chained(dedup_send_kernel<T>, (N + 7) / 8, 256, 0, s, X, key, recv_row_of_slot, Xr, N, cfg->d, K));
+    if (N > 0) {
+      C2R_CUDA(launch_chained(perm_rank_kernel, nb, PERM_THREADS, 0, s, key, NK, P, spb, block_counts, recv_offsets,
+                              recv_row_of_slot, slot_of_recv_row, 1, nullptr, nullptr));
+      C2R_LAUNCH_CHECK();
+      C2R_CUDA(launch_chained(dedup_fill_kernel, (N + 255) / 256, 256, 0, s, idx, part, key, recv_row_of_slot, N, E, K, P));
+      C2R_LAUNCH_CHECK();
+      C2R_CUDA(launch_chained(dedup_tokens_kernel, (int)((cap + 255) / 256), 256, 0, s, slot_of_recv_row, token_of_recv_row, cap, K));
       C2R_LAUNCH_CHECK();
     }
   }
   if (X != nullptr && R > 0) {
-    C2R_CUDA(launch_chained(dedup_replicate_kernel<T>, (int)((R + 7) / 8), 256, 0, s, Xr, slot_of_row, recv_row_of_slot, Xp, R, cfg->d));
-    C2R_LAUNCH_CHECK();
+    const int parts = row_parts(N, (cfg->d / Vec16<T>::N + 31) / 32);
+    const int token_blocks = (int)(((long long)N * parts + 7) / 8);
+    const int pad_blocks = R > NK ? (int)(R - NK + 7 < 8 * 296 ? (R - NK + 7) / 8 : 296) : 0;
+    if (token_blocks + pad_blocks > 0) {
+      C2R_CUDA(launch_chained(dedup_rows_kernel<T>, token_blocks + pad_blocks, 256, 0, s, X, key, recv_row_of_slot, row_of_slot,
+                              slot_of_row, Xr, Xp, N, cfg->d, K, R, token_blocks, parts));
+      C2R_LAUNCH_CHECK();
+    }
   }
   return C2R_OK;
 }

@@ -59,3 +59,52 @@ def test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared):
         assert_close_abs(host(z), X.astype(np.float64) @ wsg.astype(np.float64), 1e-4, "z")
     big, zb = gate(x.repeat(20000 // N + 1, 1))
     assert torch.equal(big[:N], L) and torch.equal(zb[:N], z)
+
+
+@pytest.mark.parametrize("N,K,P", [(1, 3, 4), (150, 7, 2), (1700, 6, 5), (40000, 4, 3), (525000, 1, 3)])
+def test_two_stage_dispatch_against_numpy(N, K, P):
+    """Both index paths (up to and beyond 1024 blocks of the counting sort), tokens that meet a partition several times; the
+    receive side is a stable sort of the first slots by partition, so numpy gives it directly."""
+    from paper_2504_01337_b200 import binding as B
+    E, d, align = 9, 8, 4
+    rng = np.random.default_rng(N + K)
+    idx = rng.permuted(np.tile(np.arange(E, dtype=np.int32), (N, 1)), axis=1)[:, :K].copy()
+    part = (np.arange(E) % P).astype(np.int32)
+    X = rng.standard_normal((N, d)).astype(np.float32)
+    cfg = B.make_config(N, d, E, 16, K, 0, P, 0, B.F32, align)
+    R, cap = B.permuted_rows(cfg), N * min(K, P)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    out = {k: torch.full((n,), -7, **i32) for k, n in (("counts", E), ("offsets", E + 1), ("row_of_slot", N * K), ("slot_of_row", R),
+                                                       ("recv_counts", P), ("recv_offsets", P + 1), ("recv_row_of_slot", N * K),
+                                                       ("token_of_recv_row", cap))}
+    Xr, Xp = torch.full((cap, d), 7.0, device="cuda"), torch.full((R, d), 7.0, device="cuda")
+    status = torch.zeros(1, **i32)
+    ws = torch.empty(B.workspace_bytes(cfg, B.WS_DISPATCH_DEDUP), dtype=torch.uint8, device="cuda")
+    B.dispatch_dedup(cfg, dev(idx), dev(part), None, dev(X), *out.values(), Xr, Xp, status, ws)
+    got = {k: host(v) for k, v in out.items()}
+    assert int(status.item()) == 0
+    # per-expert layout: a stable sort of the slots by expert, segments aligned
+    flat = idx.reshape(-1)
+    counts = np.bincount(flat, minlength=E)
+    offsets = np.concatenate([[0], np.cumsum((counts + align - 1) // align * align)])
+    order = np.argsort(flat, kind="stable")
+    rank = np.arange(N * K) - np.repeat(np.cumsum(counts) - counts, counts)
+    row_of_slot = np.empty(N * K, np.int64)
+    row_of_slot[order] = offsets[flat[order]] + rank
+    assert np.array_equal(got["counts"], counts) and np.array_equal(got["offsets"], offsets)
+    assert np.array_equal(got["row_of_slot"], row_of_slot)
+    # receive side
+    q = part[idx]
+    first = np.array([[all(q[t, j] != q[t, k] for j in range(k)) for k in range(K)] for t in range(N)]) if N < 50000 else np.ones((N, K), bool)
+    slots = np.nonzero(first.reshape(-1))[0]
+    qs = q.reshape(-1)[slots]
+    recv = slots[np.argsort(qs, kind="stable")]
+    assert np.array_equal(got["recv_counts"], np.bincount(qs, minlength=P))
+    assert np.array_equal(got["recv_offsets"], np.concatenate([[0], np.cumsum(np.bincount(qs, minlength=P))]))
+    assert np.array_equal(got["token_of_recv_row"], np.concatenate([recv // K, np.full(cap - recv.size, -1)]))
+    Xph = np.zeros((R, d), np.float32)
+    Xph[row_of_slot] = np.repeat(X, K, axis=0)
+    assert np.array_equal(host(Xp), Xph) and np.array_equal(host(Xr)[:recv.size], X[recv // K])
+    rrs = got["recv_row_of_slot"]
+    assert np.array_equal(got["token_of_recv_row"][rrs], np.repeat(np.arange(N), K))
+    assert ((rrs[:, None] >= got["recv_offsets"][None, :-1]) & (rrs[:, None] < got["recv_offsets"][None, 1:])).argmax(1).tolist() == q.reshape(-1).tolist()
