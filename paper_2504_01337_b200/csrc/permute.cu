@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_kernel(const int32_t* 
 // partition), else -2 - q; first slots get their rows, the others the row of the token's first slot with the same partition,
 // and slot_of_row holds tokens (slot / K).
 constexpr int PERM_FUSED_MAX_BLOCKS = 1024;
+constexpr int PERM_MARK_BLOCKS = 16;
 template <bool DEDUP>
 __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int32_t* __restrict__ idx, long long NK, int E,
                                                                        int slots_per_block,
@@ -769,7 +770,9 @@ int permute_impl(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
     C2R_LAUNCH_CHECK();
   }
   if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
-    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, nb, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
+    // a batch of few blocks still has up to row_align - 1 padding rows per expert to mark: blocks without slots help with them
+    const int grid = nb < PERM_MARK_BLOCKS && cfg->row_align > 1 ? PERM_MARK_BLOCKS : nb;
+    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, grid, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
                           R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status, (int)cfg->K));
     C2R_LAUNCH_CHECK();
   } else {
