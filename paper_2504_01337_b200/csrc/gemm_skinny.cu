@@ -386,9 +386,12 @@ static int skinny_launch(const c2r_config* cfg, const SwigluCall* calls, int n, 
   const int wr = up ? p.ch : 2 * p.ch, parts = up ? 2 : 1;
   int nb_max = 16;
   for (int i = 0; i < n; ++i) {
-    // chunks of half as many tokens again as expected: most experts fit one, and few columns are empty
+    // Chunks of half as many tokens again as expected: most experts fit one, and few columns are empty.  In a shared launch
+    // all stages have the size of the larger problem's, so the shared expert's tokens come in chunks of 32 at most, whose weights
+    // the later chunks find in the L2 (64 tokens of the Qwen shape 235 us with one chunk of 64, 219 with two of 32; 128
+    // tokens 263 / 247).
     const int64_t rows = expected_rows(cfg, calls[i]), want = calls[i].nE == 1 ? rows : rows + rows / 2;
-    for (p.pr[i].nb = 16; p.pr[i].nb < want && p.pr[i].nb < 128; p.pr[i].nb <<= 1) {}
+    for (p.pr[i].nb = 16; p.pr[i].nb < want && p.pr[i].nb < (n > 1 ? 32 : 128); p.pr[i].nb <<= 1) {}
     if (p.pr[i].nb > nb_max) nb_max = p.pr[i].nb;
   }
   const int kb_bytes = (parts * wr + nb_max) * BK * 2;
