@@ -283,10 +283,11 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
 }
 
 // Warps over which a token's row is spread where there are few tokens: enough for 32 warps per SM, each with at least one
-// 16-byte chunk per lane.  With a warp per token, 1021 tokens of d = 4096 left most of the chip idle (combine 38 us, row
+// 16-byte chunk per lane, and no more, so that the combine's blocks (four to an SM) start together (1021 tokens of d = 4096: 5 parts
+// 22.8 us, 4 parts 15.8).  With a warp per token, 1021 tokens of d = 4096 left most of the chip idle (combine 38 us, row
 // gather 20 us) and a single token took 23 us in the combine, 16 loads one after another.
 inline int row_parts(long long tokens, int chunks_per_warp) {
-  const long long want = (148 * 32 + tokens - 1) / (tokens > 0 ? tokens : 1);
+  const long long want = 148 * 32 / (tokens > 0 ? tokens : 1);
   return (int)(want < 1 ? 1 : want > chunks_per_warp ? chunks_per_warp : want);
 }
 
