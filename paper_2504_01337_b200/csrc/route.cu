@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(RBS_TOKENS * 8) route_bwd_scaled_kernel(const 
 // (see launch_chained), and one launch instead of three memsets where the arrays are separate.
 __global__ void __launch_bounds__(256) fill_words_kernel(uint32_t* __restrict__ a, long long na, uint32_t* __restrict__ b, long long nb,
                                                          uint32_t* __restrict__ c, long long nc, uint32_t value) {
+  chain_begin();  // the arrays may still be in use by the kernel before, and the next one relies on this one having waited
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
   for (long long i = first; i < na; i += step) a[i] = value;
   for (long long i = first; i < nb; i += step) b[i] = value;
