@@ -125,18 +125,26 @@ struct TileLoad {
 
 // C_g(m,n) = sum_k A_g(m,k) B_g(n,k) with arbitrary strides; see SimtGemm for the two modes.
 //
-// A block computes TM x TN outputs; (TM / 4)(TN / 4) threads hold a 4 x 4 share each, and where that is fewer than the
-// block has, groups of threads split every k-tile and their sums are added in group order.  The next k-tile is loaded into
-// registers while the current one is used (two shared-memory buffers, one barrier per tile).  The small configurations
-// this serves are bound by latency: a chain of 16-deep tiles, each waiting for its own loads, took 80 us for K = 256
-// where this takes 16.5 (1024 rows, 128 dual columns; weight gradients of 375 rows 158 -> 28; whole fp32 training step of
-// 1500 tokens 500 -> 200).  64 x 64 tiles where they fill the chip, else 32-wide ones.
+// A block computes TM x TN outputs; (TM / 4)(TN / 4) threads hold a 4 x 4 share each.  A sum over k is kept as S partial sums,
+// part j over the j-th of S equal pieces of every SPAN consecutive k, added in part order at the end.  Groups of threads keep
+// a part each, or a thread keeps all: a result does not depend on the tile its batch was given, and is nearer to the
+// exact sum than one chain is.  The next k-tile is loaded into registers while the current one is used (two shared-memory
+// buffers, one barrier per tile).  The small configurations this serves are bound by latency: a chain of 16-deep tiles, each
+// waiting for its own loads, took 80 us for K = 256 where this takes 16.5 (1024 rows, 128 dual columns; weight gradients of
+// 375 rows 158 -> 28; whole fp32 training step of 1500 tokens 500 -> 190).  64 x 64 tiles where they fill the chip, else
+// 32-wide ones; the two SwiGLU products always take 32 x 32, since at 64 x 64 their parts are 128 registers of a thread and
+// one block per SM (forward of 4096 tokens of 512, top-4 of 8 experts of 512: 861 us with one chain per sum, 1018 with the
+// parts at 64 x 64, 980 so; 1250 before there were parts and prefetched tiles).
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS>
+constexpr int SPAN = 32;
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int S, int SIMT_THREADS>
 __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   chain_begin();
   constexpr int GROUP = (TM / 4) * (TN / 4), G = SIMT_THREADS / GROUP;  // threads per group, groups
+  constexpr int PART = SPAN / S, PARTS = SK / PART / G, O = S / G;      // length of a part; a thread's parts per k-tile, in all
+  static_assert(!DUAL || G > 1, "two products keep their parts in groups");
+  static_assert(SPAN % SK == 0 && PARTS * PART * G == SK && (G == 1 || O == 1), "a group of threads keeps one part, or a thread all of them");
   constexpr int MR = G == 1 ? 4 : TM * TN / (4 * SIMT_THREADS);         // output rows a thread finishes, four columns each
   constexpr int TILES = 2 * SK * (TM + TN * (DUAL ? 2 : 1)), RED = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4);
   __shared__ __align__(16) float smem[TILES > RED ? TILES : RED];
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
 
   const int grp_k = tid / GROUP, tg = tid % GROUP;
   const int tx = tg % (TN / 4), ty = tg / (TN / 4);
-  float acc[4][4] = {}, acc2[DUAL ? 4 : 1][4] = {};
+  float sum[O][4][4] = {}, sum2[DUAL ? O : 1][4][4] = {};
   TileLoad<T, TM, SK, SIMT_THREADS> la;
   TileLoad<T, TN, SK, SIMT_THREADS> lb, lb2;
   la.init(rowA, g.sak, M - m0);
@@ -198,61 +206,76 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   };
   constexpr int BUF = SK * (TM + TN * (DUAL ? 2 : 1));
   fetch(0);
-  for (int k0 = 0, buf = 0; k0 < Kd; k0 += SK, buf ^= 1) {
-    float* sa = smem + buf * BUF;
-    float* sb = sa + SK * TM;
-    float* sb2 = sb + SK * TN;
-    la.store(sa);
-    lb.store(sb);
-    if (DUAL) lb2.store(sb2);
-    __syncthreads();
-    if (k0 + SK < Kd) fetch(k0 + SK);
+  for (int k0 = 0, buf = 0; k0 < Kd; k0 += SPAN) {
+#pragma unroll
+    for (int h = 0; h < SPAN / SK; ++h, buf ^= 1) {
+      const int kt = k0 + h * SK;
+      if (kt >= Kd) break;
+      float* sa = smem + buf * BUF;
+      float* sb = sa + SK * TM;
+      float* sb2 = sb + SK * TN;
+      la.store(sa);
+      lb.store(sb);
+      if (DUAL) lb2.store(sb2);
+      __syncthreads();
+      if (kt + SK < Kd) fetch(kt + SK);
+#pragma unroll
+      for (int q = 0; q < PARTS; ++q) {
+        float(&acc)[4][4] = sum[h * PARTS + q];
+        float(&acc2)[4][4] = sum2[DUAL ? h * PARTS + q : 0];
 #pragma unroll 8  // a kernel this short is bound by instruction fetch if the body is longer
-    for (int kk = 0; kk < SK / G; ++kk) {
-      const int k = grp_k * (SK / G) + kk;
-      const float4 av = *reinterpret_cast<const float4*>(&sa[tile_at<TM>(k, 4 * ty)]);
-      const float4 bv = *reinterpret_cast<const float4*>(&sb[tile_at<TN>(k, 4 * tx)]);
-      const float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
+        for (int kk = 0; kk < PART; ++kk) {
+          const int k = (grp_k * PARTS + q) * PART + kk;
+          const float4 av = *reinterpret_cast<const float4*>(&sa[tile_at<TM>(k, 4 * ty)]);
+          const float4 bv = *reinterpret_cast<const float4*>(&sb[tile_at<TN>(k, 4 * tx)]);
+          const float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
-      if (DUAL) {
-        const float4 cv = *reinterpret_cast<const float4*>(&sb2[tile_at<TN>(k, 4 * tx)]);
-        const float cr[4] = {cv.x, cv.y, cv.z, cv.w};
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
+          if (DUAL) {
+            const float4 cv = *reinterpret_cast<const float4*>(&sb2[tile_at<TN>(k, 4 * tx)]);
+            const float cr[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc2[DUAL ? i : 0][j] = fmaf(ar[i], cr[j], acc2[DUAL ? i : 0][j]);
+              for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(ar[i], cr[j], acc2[i][j]);
+          }
+        }
       }
     }
   }
   // this thread's outputs: rows m_of(i), columns nc .. nc + 3
   const int nc = n0 + 4 * (G == 1 ? tx : tid % (TN / 4));
   auto m_of = [&](int i) { return G == 1 ? 4 * ty + i : tid / (TN / 4) + i * (SIMT_THREADS / (TN / 4)); };
-  if (G > 1) {  // add the groups' partial sums, in group order
-    constexpr int P = TN + 4;
+  float(&acc)[4][4] = sum[0];
+  float(&acc2)[4][4] = sum2[0];
+  // the parts added in part order: a thread's own, or all groups' through shared memory
+  constexpr int P = TN + 4;
+  if (G > 1) {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       *reinterpret_cast<float4*>(&smem[(grp_k * TM + 4 * ty + i) * P + 4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
       if (DUAL)
         *reinterpret_cast<float4*>(&smem[((G + grp_k) * TM + 4 * ty + i) * P + 4 * tx]) =
-            make_float4(acc2[DUAL ? i : 0][0], acc2[DUAL ? i : 0][1], acc2[DUAL ? i : 0][2], acc2[DUAL ? i : 0][3]);
+            make_float4(acc2[i][0], acc2[i][1], acc2[i][2], acc2[i][3]);
     }
     __syncthreads();
+  }
+  if (S > 1) {
 #pragma unroll
     for (int i = 0; i < MR; ++i) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         float v = 0.f, v2 = 0.f;
 #pragma unroll
-        for (int q = 0; q < G; ++q) {
-          v += smem[(q * TM + m_of(i)) * P + nc - n0 + j];
+        for (int q = 0; q < S; ++q) {
+          v += G == 1 ? sum[q < O ? q : 0][i][j] : smem[(q * TM + m_of(i)) * P + nc - n0 + j];
           if (DUAL) v2 += smem[((G + q) * TM + m_of(i)) * P + nc - n0 + j];
         }
         acc[i][j] = v;
-        if (DUAL) acc2[DUAL ? i : 0][j] = v2;
+        if (DUAL) acc2[i][j] = v2;
       }
     }
   }
@@ -278,7 +301,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
         // v = A[r,n], acc2 = B[r,n]: H = silu(A) * B; the backward pass needs only the two local
         // derivatives dH/dA = B silu'(A) and dH/dB = silu(A), which are what is kept (packed columns)
         const int pg = pack_col(n, g.I), pu = pg + pack_width(n, g.I);
-        const float b = acc2[DUAL ? i : 0][j];
+        const float b = acc2[i][j];
         const float sg = 1.0f / (1.0f + expf(-v));
         const float as = v * sg;
         if (g.C != nullptr) {  // inference: nothing is kept for a backward pass
@@ -317,9 +340,9 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   }
 }
 
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int SIMT_THREADS = 256>
+template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int S, int SIMT_THREADS = 256>
 static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
-  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s, g));
+  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, S, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s, g));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -343,14 +366,14 @@ int simt_launch(SimtGemm g, int n_groups, int64_t max_m, cudaStream_t s) {
   // SIMT_ROWS: whole tiles of all groups, and one more per group for its remainder
   auto m_tiles = [&](int tm) { return (int)((max_m + tm - 1) / tm) + (rows ? n_groups : 0); };
   const int64_t blocks64 = (int64_t)((max_m + 63) / 64) * ((g.Ndim + 63) / 64) * z;
-  const bool dual = g.epi == SIMT_EPI_SWIGLU_FWD;
-  if (blocks64 >= 2 * 148)
-    return dual ? simt_launch_tile<T, TC, 64, 64, 16, true>(g, m_tiles(64), z, s)
-                : simt_launch_tile<T, TC, 64, 64, 16, false>(g, m_tiles(64), z, s);
-  if (dual) return simt_launch_tile<T, TC, 32, 32, 32, true>(g, m_tiles(32), z, s);
-  // the backward's partial row dots cover 64 columns each
-  return g.epi == SIMT_EPI_SWIGLU_BWD ? simt_launch_tile<T, TC, 32, 64, 32, false>(g, m_tiles(32), z, s)
-                                      : simt_launch_tile<T, TC, 32, 32, 32, false>(g, m_tiles(32), z, s);
+  const bool large = blocks64 >= 2 * 148;
+  // four partial sums; two in the backward of SwiGLU, whose partial row dots cover 64 columns each
+  if (g.epi == SIMT_EPI_SWIGLU_FWD) return simt_launch_tile<T, TC, 32, 32, 32, true, 4>(g, m_tiles(32), z, s);
+  if (g.epi == SIMT_EPI_SWIGLU_BWD)
+    return large ? simt_launch_tile<T, TC, 64, 64, 16, false, 2>(g, m_tiles(64), z, s)
+                 : simt_launch_tile<T, TC, 32, 64, 32, false, 2>(g, m_tiles(32), z, s);
+  return large ? simt_launch_tile<T, TC, 64, 64, 16, false, 4>(g, m_tiles(64), z, s)
+               : simt_launch_tile<T, TC, 32, 32, 32, false, 4>(g, m_tiles(32), z, s);
 }
 
 // Gate logits (Eq. 1) in fp32 arithmetic: L = X Wg^T and, as one more row of the other operand, z = X wsg.
@@ -364,7 +387,7 @@ int simt_gate_logits(const c2r_config* cfg, const void* X, const void* Wg, const
   // a tile without thread groups: one chain of products in k order, whatever the batch (near-ties must not move with it)
   g.n_groups = 1;
   g.vec = simt_vec<T>(g);
-  return simt_launch_tile<T, float, 32, 32, 32, false, 64>(g, (cfg->N + 31) / 32, 1, s);
+  return simt_launch_tile<T, float, 32, 32, 32, false, 1, 64>(g, (cfg->N + 31) / 32, 1, s);
 }
 template int simt_gate_logits<float>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);
 template int simt_gate_logits<__nv_bfloat16>(const c2r_config*, const void*, const void*, const void*, float*, float*, cudaStream_t);

@@ -58,3 +58,30 @@ def test_gate_logits_of_unaligned_arrays(offset):
         cfg = B.make_config(N, d, E, 16, 2, 3, 1, 0, B.BF16 if bf16 else B.F32, 1)
         B.gate_logits(cfg, flat[offset:offset + N * d].view(N, d), dev(Wg, dt), None, L, None)
         assert_close_abs(host(L), O.gate_logits(X, Wg), 1e-4, "L")
+
+
+# a batch that takes 32-wide tiles inside one that takes the large tiles in every product; contractions that end inside a part
+@pytest.mark.parametrize("n,N,d,E,I,K,I_s,bf16", [(37, 4096, 200, 5, 336, 2, 0, False), (300, 4100, 264, 4, 528, 3, 400, False),
+                                                  (37, 6000, 200, 5, 336, 2, 272, True)])
+def test_results_of_a_token_do_not_depend_on_the_batch(n, N, d, E, I, K, I_s, bf16):
+    """The CUDA-core kernels (fp32, and bf16 with d no multiple of 16), forward and backward, bit for bit."""
+    from paper_2504_01337_b200.layer import C2RLayer
+    wl = G.Workload("batch", N=N, d=d, E=E, I=I, K=K, T=E - 1, P=2, I_s=I_s, bf16=bf16, seed=8)
+    X, dY = G.hidden(wl), G.grad_out(wl)
+    Wg, wsg = G.gate_weights(wl)
+    W1, W3, W2 = G.expert_weights(wl)
+    sh = G.shared_weights(wl) if I_s else None
+    got = []
+    for m in (n, N):
+        lay = C2RLayer(m, d, E, I, K, E - 1, 2, I_s, bf16, row_align=1, backward=True)
+        lay.set_params(Wg, W1, W3, W2, wsg, sh)
+        lay.set_routing()
+        lay.set_input(X[:m], dY[:m])
+        lay.forward()
+        lay.backward()
+        rows = lay.t["row_of_slot"].long()[:n * K]
+        t = {x: lay.t[x][:n] for x in ("L", "idx", "w", "Y", "dl", "dX") + (("Ys", "dXs", "dz") if I_s else ())}
+        t.update({x: lay.t[x][rows] for x in ("H", "AB", "Yp", "dAB", "dXp")})
+        got.append(t)
+    for x in got[0]:
+        assert torch.equal(got[0][x], got[1][x]), x
