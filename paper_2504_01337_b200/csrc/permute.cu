@@ -286,8 +286,9 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
 // 16-byte chunk per lane, and no more, so that the combine's blocks (four to an SM) start together (1021 tokens of d = 4096: 5 parts
 // 22.8 us, 4 parts 15.8).  With a warp per token, 1021 tokens of d = 4096 left most of the chip idle (combine 38 us, row
 // gather 20 us) and a single token took 23 us in the combine, 16 loads one after another.
+constexpr int ROW_WARPS = 148 * 32;
 inline int row_parts(long long tokens, int chunks_per_warp) {
-  const long long want = 148 * 32 / (tokens > 0 ? tokens : 1);
+  const long long want = ROW_WARPS / (tokens > 0 ? tokens : 1);
   return (int)(want < 1 ? 1 : want > chunks_per_warp ? chunks_per_warp : want);
 }
 
@@ -380,9 +381,10 @@ __device__ __forceinline__ void load_as_float(const S* p, float* f) {
 //          + ecoef(t) * extra[t,:]                           (ecoef = sigmoid(z[t]) if z else 1)
 //          + sum_k dl[t,k] * Wg[idx[t,k],:] + dz[t] * wsg[:] (gate terms, optional)
 //          + out[t,:] if accumulate.
-// src == NULL: no such term (the producer already added its rows into extra).  src / extra are the fp32 partial results of the expert GEMMs; out has the storage type.
-// `parts` warps per token, fp32 accumulation in k order.  Serves the combine and the gradient un-permute.
-template <typename T>
+// src == NULL: no such term (the producer already added its rows into extra).  src / extra are the fp32 partial results of the
+// expert GEMMs; out has the storage type.  fp32 accumulation in k order.  Serves the combine and the gradient un-permute.
+// SPLIT: `parts` warps per token, else one.
+template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(256) gather_sum_kernel(const float* __restrict__ src, const int32_t* __restrict__ rows_g,
                                                          const float* __restrict__ coef, const float* __restrict__ extra,
                                                          const float* __restrict__ z, const int32_t* __restrict__ idx,
@@ -392,6 +394,7 @@ __global__ void __launch_bounds__(256) gather_sum_kernel(const float* __restrict
   chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
+  if (!SPLIT) parts = 1;
   const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int t = (int)(wid / parts), part = (int)(wid - (long long)t * parts);
   if (t >= N) return;  // warp-uniform
@@ -832,6 +835,10 @@ extern "C" int c2r_permute_rows(const c2r_config* cfg, const void* X, const int3
   return permute_rows_launch(cfg, (const float*)X, row_of_slot, counts, offsets, (float*)Xp, as_stream(stream));
 }
 
+// In bf16 the form that takes `parts` at run time holds more loads in flight, in 56 registers and four blocks per SM; with one
+// warp per token known it takes 34 registers and seven blocks.  The first is the better one while its blocks start in one
+// wave or nearly fill two, the second beyond (us, combine, top-4: 4096 tokens of 2048 32.5 / 34, 6000 52 / 42, 8192 57 / 62,
+// 16384 109 / 102, 65536 386 / 364, 300000 of 256 266 / 219).  In fp32 both take 40.
 template <typename T>
 static int gather_sum_launch(const c2r_config* cfg, const void* src, const int32_t* rows, const float* coef,
                              const void* extra, const float* z, const int32_t* idx, const float* dl, const void* Wg,
@@ -839,9 +846,10 @@ static int gather_sum_launch(const c2r_config* cfg, const void* src, const int32
   if (cfg->N == 0) return C2R_OK;
   const int parts = row_parts(cfg->N, (cfg->d / Vec16<T>::N + 31) / 32);
   const long long warps = (long long)cfg->N * parts;
-  C2R_CUDA(launch_chained(gather_sum_kernel<T>, (unsigned)((warps + 7) / 8), 256, 0, s, (const float*)src, rows, coef, (const float*)extra, z, idx, dl,
-                          (const T*)Wg, dz, (const T*)wsg, (T*)out, accumulate, cfg->N,
-                          cfg->d, cfg->K, parts));
+  const bool split = parts > 1 || (sizeof(T) == 2 && (warps <= ROW_WARPS || (2 * warps > 3 * ROW_WARPS && warps <= 2 * ROW_WARPS)));
+  C2R_CUDA(launch_chained(split ? gather_sum_kernel<T, true> : gather_sum_kernel<T, false>, (unsigned)((warps + 7) / 8), 256, 0, s,
+                          (const float*)src, rows, coef, (const float*)extra, z, idx, dl, (const T*)Wg, dz, (const T*)wsg,
+                          (T*)out, accumulate, cfg->N, cfg->d, cfg->K, parts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
