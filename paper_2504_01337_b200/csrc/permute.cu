@@ -1117,15 +1117,18 @@ __global__ void __launch_bounds__(PERM_THREADS) dedup_hist_kernel(const int32_t*
 
 // The rows of both stages: `parts` warps per token read its row once and write it to the receive row of every partition
 // that needs it and to its K rows of the per-expert layout, which are what replication from the receive buffer would give.
-// Blocks past the token blocks zero the rows of that layout that hold no slot.  Bound by the bytes (16384 tokens of 2048, top-4,
-// 4 partitions: 507 MB; two kernels, of which the second read the receive buffer again, took 110 us, this one 95).
+// Blocks past the token blocks zero the rows of that layout that hold no slot: PAD_BLOCKS per expert for the rows that close
+// its segment, the rest for the rows past the last segment.  (Blocks that looked for them in slot_of_row, one load after
+// another, outlasted the token blocks where rows are short: whole dispatch of 300000 tokens of 256, top-4, 590 us, so 324;
+// 65536 of 2048 421 / 378.)  Bound by the bytes (16384 tokens of 2048, top-4, 4 partitions: 507 MB; two kernels, of which the
+// second read the receive buffer again, took 110 us, this one 95).
 template <typename T>
 __global__ void __launch_bounds__(256) dedup_rows_kernel(const T* __restrict__ X, const int32_t* __restrict__ key,
                                                          const int32_t* __restrict__ recv_row_of_slot,
                                                          const int32_t* __restrict__ row_of_slot,
-                                                         const int32_t* __restrict__ slot_of_row, T* __restrict__ Xr,
-                                                         T* __restrict__ Xp, int N, int d, int K, long long R, int token_blocks,
-                                                         int parts) {
+                                                         const int32_t* __restrict__ counts, const int32_t* __restrict__ offsets,
+                                                         T* __restrict__ Xr, T* __restrict__ Xp, int N, int d, int E, int K,
+                                                         long long R, int row_align, int token_blocks, int pad_blocks, int parts) {
   chain_begin();
   using V = Vec16<T>;
   const int lane = threadIdx.x & 31;
@@ -1134,11 +1137,19 @@ __global__ void __launch_bounds__(256) dedup_rows_kernel(const T* __restrict__ X
     V zero;
     float zf[V::N] = {};
     zero.from_float(zf);
-    const long long step = (long long)(gridDim.x - token_blocks) * (blockDim.x >> 5);
-    for (long long r = (long long)(blockIdx.x - token_blocks) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += step) {
-      if (slot_of_row[r] >= 0) continue;
-      for (int c = lane; c < chunks; c += 32) zero.store(Xp + (size_t)r * d + (size_t)c * V::N);
+    int b = blockIdx.x - token_blocks, blocks = PAD_BLOCKS;
+    long long r = offsets[E], end = R;
+    if (b < pad_blocks) {
+      const int e = b / PAD_BLOCKS, n = counts[e];
+      r = offsets[e] + n;
+      end = offsets[e] + (n + row_align - 1) / row_align * row_align;
+      b %= PAD_BLOCKS;
+    } else {
+      b -= pad_blocks;
+      blocks = gridDim.x - token_blocks - pad_blocks;
     }
+    for (r += b * (blockDim.x >> 5) + (threadIdx.x >> 5); r < end; r += (long long)blocks * (blockDim.x >> 5))
+      for (int c = lane; c < chunks; c += 32) zero.store(Xp + (size_t)r * d + (size_t)c * V::N);
     return;
   }
   const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1240,10 +1251,12 @@ static int dispatch_dedup_impl(const c2r_config* cfg, const int32_t* idx, const 
   if (X != nullptr && R > 0) {
     const int parts = row_parts(N, (cfg->d / Vec16<T>::N + 31) / 32);
     const int token_blocks = (int)(((long long)N * parts + 7) / 8);
-    const int pad_blocks = R > NK ? (int)(R - NK + 7 < 8 * 296 ? (R - NK + 7) / 8 : 296) : 0;
+    const int pad_blocks = R > NK ? E * PAD_BLOCKS : 0;
+    const int tail_blocks = (int)(R - NK + 7 < 8 * 296 ? (R - NK + 7) / 8 : 296);
     if (token_blocks + pad_blocks > 0) {
-      C2R_CUDA(launch_chained(dedup_rows_kernel<T>, token_blocks + pad_blocks, 256, 0, s, X, key, recv_row_of_slot, row_of_slot,
-                              slot_of_row, Xr, Xp, N, cfg->d, K, R, token_blocks, parts));
+      C2R_CUDA(launch_chained(dedup_rows_kernel<T>, token_blocks + pad_blocks + tail_blocks, 256, 0, s, X, key, recv_row_of_slot,
+                              row_of_slot, counts, offsets, Xr, Xp, N, cfg->d, E, K, R, cfg->row_align, token_blocks, pad_blocks,
+                              parts));
       C2R_LAUNCH_CHECK();
     }
   }

@@ -48,3 +48,30 @@ def test_combine_and_unpermute(N, d, K, bf16):
     e = host(idx)
     check(sum(Yp[r[:, k]].astype(np.float64) for k in range(K)) + Ys + dz[:, None].astype(np.float64) * wsg
           + sum(w[:, k:k + 1].astype(np.float64) * Wg[e[:, k]] for k in range(K)))
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("N,K,d,align,used", [(2, 2, 16, 128, 2), (1, 1, 8, 128, 9), (300, 2, 264, 128, 3), (700, 8, 1032, 5, 9), (9000, 3, 64, 96, 4)])
+def test_rows_without_a_slot_of_the_two_stage_dispatch_are_zero(N, K, d, align, used, bf16):
+    """The rows that close each segment and the rows past the last one, with experts nobody chose: bit for bit the plain
+    gather's rows, and zeros everywhere else."""
+    from paper_2504_01337_b200 import binding as B
+    E, P = 9, 4
+    dt = torch.bfloat16 if bf16 else torch.float32
+    rng = np.random.default_rng(N + K)
+    pool = np.arange(max(used, K), dtype=np.int32)
+    idx = dev(rng.permuted(np.tile(pool, (N, 1)), axis=1)[:, :K].copy().reshape(N, K))
+    cfg = B.make_config(N, d, E, 16, K, 0, P, 0, B.BF16 if bf16 else B.F32, align)
+    R, cap = B.permuted_rows(cfg), N * min(K, P)
+    t = [torch.full((n,), -7, dtype=torch.int32, device="cuda") for n in (E, E + 1, N * K, R, P, P + 1, N * K, cap)]
+    X = dev(rng.standard_normal((N, d)).astype(np.float32).reshape(N, d), dt)
+    Xr, Xp = torch.full((cap, d), 7.0, dtype=dt, device="cuda"), torch.full((R, d), 7.0, dtype=dt, device="cuda")
+    ws = torch.empty(B.workspace_bytes(cfg, B.WS_DISPATCH_DEDUP), dtype=torch.uint8, device="cuda")
+    rank = dev(rng.permutation(E).astype(np.int32))
+    B.dispatch_dedup(cfg, idx, dev((np.arange(E) % P).astype(np.int32)), rank, X, *t, Xr, Xp, torch.zeros(1, dtype=torch.int32, device="cuda"), ws)
+    slot = host(t[3])
+    ref = torch.zeros((R, d), dtype=dt, device="cuda")
+    live = np.nonzero(slot >= 0)[0]
+    assert live.size == N * K
+    ref[dev(live)] = X[dev(slot[live] // K)]
+    assert torch.equal(Xp, ref)
