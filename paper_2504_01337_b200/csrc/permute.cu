@@ -292,10 +292,13 @@ inline int row_parts(long long tokens, int chunks_per_warp) {
   return (int)(want < 1 ? 1 : want > chunks_per_warp ? chunks_per_warp : want);
 }
 
-// Row gather: a token's row is read once and written to its K rows by `parts` warps.  Blocks past the token blocks zero the
+// Row gather: a token's row is read once and written to its K rows by `parts` warps, U chunks per lane at a time: 1 where a lane
+// has no more (16384 tokens of 256, top-4, 8.4 us with 4 at a time, 7.9 so), else 4, for which the token and part come from
+// 32-bit arithmetic -- with a 64-bit division the compiler kept fewer loads in flight (16384 tokens of 4096, top-8,
+// 222 us / 207).  Blocks past the token blocks zero the
 // padding rows that close each expert's aligned segment (PAD_BLOCKS blocks per expert).
 constexpr int PAD_BLOCKS = 8;
-template <typename T>
+template <typename T, int U>
 __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__ X,
                                                            const int32_t* __restrict__ row_of_slot, T* __restrict__ Xp,
                                                            int N, int d, int K, const int32_t* __restrict__ counts,
@@ -315,8 +318,8 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__
       for (int c = lane; c < d / V::N; c += 32) zero.store(Xp + (size_t)r * d + (size_t)c * V::N);
     return;
   }
-  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int t = (int)(wid / parts), part = (int)(wid - (long long)t * parts);
+  const int wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  // below 2^31: several parts only where tokens are few
+  const int t = parts == 1 ? wid : wid / parts, part = wid - t * parts;
   if (t >= N) return;  // warp-uniform
   const int my_row = (lane < K) ? row_of_slot[(size_t)t * K + lane] : 0;
   int rows[8];
@@ -325,17 +328,17 @@ __global__ void __launch_bounds__(256) permute_rows_kernel(const T* __restrict__
   const int chunks = d / V::N;
   const T* src = X + (size_t)t * d;
   const int step = 32 * parts;  // the part's chunks: every parts-th group of 32
-  for (int c0 = 32 * part + lane; c0 < chunks; c0 += step * 4) {
-    V v[4];
+  for (int c0 = 32 * part + lane; c0 < chunks; c0 += step * U) {
+    V v[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < U; ++u)
       if (c0 + step * u < chunks) v[u].load(src + (size_t)(c0 + step * u) * V::N);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (k >= K) break;
       T* dst = Xp + (size_t)rows[k] * d;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < U; ++u)
         if (c0 + step * u < chunks) v[u].store(dst + (size_t)(c0 + step * u) * V::N);
     }
   }
@@ -751,8 +754,9 @@ static int permute_rows_launch(const c2r_config* cfg, const T* X, const int32_t*
   const int token_blocks = (int)(((long long)cfg->N * parts + 7) / 8);
   const int pad_blocks = cfg->row_align > 1 ? cfg->E * PAD_BLOCKS : 0;
   if (token_blocks + pad_blocks == 0) return C2R_OK;
-  C2R_CUDA(launch_chained(permute_rows_kernel<T>, token_blocks + pad_blocks, 256, 0, s, X, row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts, offsets,
-                          token_blocks, cfg->row_align, parts));
+  const bool deep = cfg->d / Vec16<T>::N > 32 * parts;
+  C2R_CUDA(launch_chained(deep ? permute_rows_kernel<T, 4> : permute_rows_kernel<T, 1>, token_blocks + pad_blocks, 256, 0, s, X,
+                          row_of_slot, Xp, cfg->N, cfg->d, cfg->K, counts, offsets, token_blocks, cfg->row_align, parts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

@@ -75,3 +75,24 @@ def test_rows_without_a_slot_of_the_two_stage_dispatch_are_zero(N, K, d, align, 
     assert live.size == N * K
     ref[dev(live)] = X[dev(slot[live] // K)]
     assert torch.equal(Xp, ref)
+
+
+# a row within one group of 32 16-byte chunks per lane, exactly one, one more, and several per warp; several warps per token
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("N,K,d", [(1, 8, 2056), (40, 3, 264), (3000, 2, 128), (3000, 1, 256), (3000, 5, 264), (5000, 8, 1032), (5001, 4, 24)])
+def test_row_gather(N, K, d, bf16):
+    from paper_2504_01337_b200 import binding as B
+    E = 9
+    dt = torch.bfloat16 if bf16 else torch.float32
+    rng = np.random.default_rng(N + d)
+    idx = dev(rng.permuted(np.tile(np.arange(E, dtype=np.int32), (N, 1)), axis=1)[:, :K].copy())
+    cfg = B.make_config(N, d, E, 16, K, 0, 1, 0, B.BF16 if bf16 else B.F32, 32)
+    (counts, offsets, rows, slot), R = _index(B, cfg, idx)
+    X = dev(rng.standard_normal((N, d)).astype(np.float32), dt)
+    Xp = torch.full((R, d), 7.0, dtype=dt, device="cuda")
+    B.permute_rows(cfg, X, rows, counts, offsets, Xp)
+    end, s = int(offsets[E]), slot.long()
+    ref = torch.full((R, d), 7.0, dtype=dt, device="cuda")  # rows past the layout are left alone
+    ref[:end] = 0
+    ref[s >= 0] = X[s[s >= 0] // K]
+    assert torch.equal(Xp, ref)
