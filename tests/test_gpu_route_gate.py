@@ -108,3 +108,24 @@ def test_two_stage_dispatch_against_numpy(N, K, P):
     rrs = got["recv_row_of_slot"]
     assert np.array_equal(got["token_of_recv_row"][rrs], np.repeat(np.arange(N), K))
     assert ((rrs[:, None] >= got["recv_offsets"][None, :-1]) & (rrs[:, None] < got["recv_offsets"][None, 1:])).argmax(1).tolist() == q.reshape(-1).tolist()
+
+
+# full softmax by warps: every K at its block size, one token, a batch of one block, two warps' worth of experts; N on both
+# sides of the line on blocks (592 blocks of 64 tokens) and of a small batch (128 tokens)
+@pytest.mark.parametrize("K,E,N", [(1, 33, 128), (1, 33, 129), (2, 64, 1), (3, 60, 127), (4, 33, 130), (5, 60, 97), (6, 64, 161), (7, 33, 65),
+                                   (8, 60, 1), (8, 34, 592 * 64), (8, 34, 592 * 64 + 1)])
+@pytest.mark.parametrize("renorm", [0, 1])
+def test_full_softmax_of_small_batches(K, E, N, renorm):
+    from paper_2504_01337_b200 import binding as B
+    rng = np.random.default_rng(K * 100 + E + N)
+    L = (2 * rng.standard_normal((N, E))).astype(np.float32)
+    L[rng.random((N, E)) < 0.05] = -np.inf
+    L[:, E - 1] = np.maximum(L[:, E - 1], -8.0)  # a finite logit in every row
+    cfg = B.make_config(N, 8, E, 16, K, K, 1, 0, B.F32, 1, renorm)
+    idx, w, p = torch.zeros((N, K), dtype=torch.int32, device="cuda"), torch.zeros((N, K), device="cuda"), torch.zeros((N, E), device="cuda")
+    B.route(cfg, dev(L), None, idx, w, p)
+    ridx, rw = O.topk_route(L, K, bool(renorm))
+    assert np.array_equal(host(idx), ridx)
+    # expf and a division: a few units in the last place of values up to 1
+    assert_close_abs(host(w), rw, 1e-6, "w")
+    assert_close_abs(host(p), O.softmax_rows(L), 1e-6, "p")
