@@ -61,7 +61,8 @@ def test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared):
     assert torch.equal(big[:N], L) and torch.equal(zb[:N], z)
 
 
-@pytest.mark.parametrize("N,K,P", [(1, 3, 4), (150, 7, 2), (1700, 6, 5), (40000, 4, 3), (525000, 1, 3)])
+@pytest.mark.parametrize("N,K,P", [(1, 3, 4), (150, 7, 2), (1700, 6, 5), (40000, 4, 3), (525000, 1, 3), (263000, 2, 1),
+                                   (176000, 3, 2)])
 def test_two_stage_dispatch_against_numpy(N, K, P):
     """Both index paths (up to and beyond 1024 blocks of the counting sort), tokens that meet a partition several times; the
     receive side is a stable sort of the first slots by partition, so numpy gives it directly."""
@@ -95,7 +96,7 @@ def test_two_stage_dispatch_against_numpy(N, K, P):
     assert np.array_equal(got["row_of_slot"], row_of_slot)
     # receive side
     q = part[idx]
-    first = np.array([[all(q[t, j] != q[t, k] for j in range(k)) for k in range(K)] for t in range(N)]) if N < 50000 else np.ones((N, K), bool)
+    first = np.stack([(q[:, :k] != q[:, k:k + 1]).all(1) for k in range(K)], axis=1)
     slots = np.nonzero(first.reshape(-1))[0]
     qs = q.reshape(-1)[slots]
     recv = slots[np.argsort(qs, kind="stable")]
