@@ -291,7 +291,9 @@ def dispatch_report(L, mask, Cm_host, E, K, T, partitions=(2, 4, 8)):
 def dedup_dispatch_timing(lay, reps=5):
     """The zero-redundancy two-stage dispatch (Sec. 3.4) on the bench batch, timed beside the plain
     dispatch it replaces: stage 1 writes one row per (token, partition) -- the rows an all-to-all
-    would carry -- and stage 2 replicates inside the partition."""
+    would carry -- and stage 2 replicates inside the partition.  On one device the library writes the
+    contents of both in one pass over the hidden states, so this is the cost of having both buffers, not
+    of a stage 2 that reads the receive buffer."""
     import torch
     from paper_2504_01337_b200 import binding as B
     c, t = lay.cfg, lay.t

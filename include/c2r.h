@@ -162,9 +162,11 @@ int c2r_permute_rows(const c2r_config* cfg, const void* X, const int32_t* row_of
  * experts.  Partition q receives recv_counts[q] rows, in token order, at rows
  * [recv_offsets[q], recv_offsets[q+1]) of Xr; recv_offsets[P] is the number of rows an all-to-all
  * would carry (the `dedup` total of c2r_dispatch_volume, against N*K for the plain dispatch).
- * Stage 2, local to a partition: the per-expert layout of c2r_permute is filled from the receive
- * buffer, Xp[r,:] = Xr[recv_row_of_slot[slot_of_row[r]],:].  With a partition-major expert_rank a
- * partition's rows of Xp read only that partition's segment of Xr.
+ * Stage 2, local to a partition: the per-expert layout of c2r_permute holds the rows replicated out of
+ * the receive buffer, Xp[r,:] = Xr[recv_row_of_slot[slot_of_row[r]],:]; with a partition-major expert_rank
+ * a partition's rows of Xp come from that partition's segment of Xr alone.  On one device both buffers
+ * are written in one pass that reads each row of X once: the call gives the contents of both stages, and
+ * its time is not that of a second stage which reads Xr.
  * part [E] int32 (expert -> partition, cfg->P partitions); the other inputs as c2r_permute.
  * out: counts, offsets, row_of_slot, slot_of_row, Xp exactly as c2r_permute writes them (bit-exact);
  *      recv_counts [P], recv_offsets [P+1] int32; recv_row_of_slot [N*K] int32; token_of_recv_row
@@ -249,7 +251,8 @@ typedef struct c2r_expert_opts {
  * R = rows of the buffers.  Padding rows of Xp must be zero.  n_experts = 1 with counts = {R},
  * offsets = {0,R} evaluates the dense shared expert.
  * bf16 runs on the tensor cores (tcgen05) when d % 16 == 0 and, for n_experts > 1, row_align is a
- * multiple of 128; other shapes and fp32 use a CUDA-core kernel.  status (one int32, may be NULL)
+ * multiple of 128; other shapes and fp32 use a CUDA-core kernel.  A row's results do not depend on how
+ * many other rows the call has (sums over channels are added in one order for all batch sizes).  status (one int32, may be NULL)
  * receives C2R_STATUS_WAIT_TIMEOUT if a bounded wait inside the kernel gave up (results invalid). */
 int c2r_grouped_swiglu_fwd(const c2r_config* cfg, int n_experts, int I, int64_t R, const void* Xp,
                            const int32_t* counts, const int32_t* offsets, const void* W13p, const void* W2,

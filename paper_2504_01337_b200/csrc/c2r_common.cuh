@@ -64,10 +64,10 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // Every kernel of the library is launched so that its blocks may start while the last blocks of the kernel before it on the
 // stream still run (programmatic dependent launch), and begins with chain_begin(): let the next kernel do the same, then
 // wait until the kernel before has completed and its writes are visible.  What overlaps is launch latency, block start-up,
-// barrier and tensor-memory set-up -- a layer is 7 to 30 launches, most of them a few microseconds long
-// (us without / with: forward pass of 1 token 90 / 79,
-// of 1021 tokens of the LLaMA shape 180 / 164, fp32 training step of 1500 tokens 200 / 188, two-stage dispatch 184 / 162).  No kernel may return before the wait: the next one relies on
-// this one's completion to imply that of all earlier ones.
+// barrier and tensor-memory set-up -- a layer is 7 to 30 launches, most of them a few microseconds long (us without / with:
+// forward pass of 1 token 88 / 74, of 64 tokens 233 / 221, fp32 training step of 1500 tokens 206 / 193; calibration, two-stage
+// dispatch and passes past 0.5 ms move by no more than their spread).  No kernel may return, or touch what an earlier one
+// reads or writes, before the wait: the next one relies on this one's completion to imply that of all earlier ones.
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t c = {};

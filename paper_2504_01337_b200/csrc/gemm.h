@@ -90,6 +90,9 @@ int tc_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
 // this: 237 / 183 at 4 rows, 238 / 202 at 34, 238 / 226 at 68; LLaMA-MoE shape 105 / 95 at 32, 105 / 107 at 64; 12 experts of
 // 512: 36 / 34 at 43, 36 / 44 at 85).  A dense group that rides along with the routed ones may have 128 rows: the
 // launches it saves and the SMs it fills are worth more than its own loss (Qwen shape, 128 tokens, whole forward 382 / 319).
+// The host knows the mean only.  Where routing is skewed so far that most rows meet in a few experts, their token chunks
+// read the weights again and pair tiles would be the faster ones from 64 tokens on (Qwen shape, whole pass call by call,
+// pair tiles / this: 108 / 79 at 16 tokens, 120 / 122 at 64, 137 / 165 at 256, 174 / 224 at 720).
 constexpr int SKINNY_ROWS = 48, SKINNY_ROWS_PAIRED = 128;
 bool skinny_supported(const c2r_config* cfg, const SwigluCall& a, int max_rows);
 // One or two such calls in one launch per product (the routed experts and the shared expert).

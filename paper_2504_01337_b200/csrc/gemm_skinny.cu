@@ -16,7 +16,7 @@
 // launches, not four.
 //
 // Measured, Qwen shape, both products of the routed experts after an L2 flush: 64 tokens 237 -> 183 us (1.04 GB, 5.7 TB/s),
-// 1 token 52 -> 36 us; a whole forward pass of 64 tokens 368 -> 286 us, of one token 170 -> 112 us.
+// 1 token 52 -> 36 us; a whole forward pass of 64 tokens, with the other kernels as they are now, 366 -> 221 us, of one token 172 -> 75 us.
 //
 // Warp roles (192 threads): warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2..5 epilogue (TMEM -> shared
 // memory -> coalesced stores).  Waits are bounded like in the other tensor-core kernels.

@@ -13,8 +13,9 @@
 // (TMEM -> registers -> a per-warp staging tile in shared memory -> global, row-contiguously; fused
 // SwiGLU forms; two warps per TMEM lane quarter).
 // The producer and the issuer keep their whole warp converged and elect the issuing thread per stage: from one divergent
-// lane every descriptor and coordinate had to be moved into uniform registers one at a time (routed forward and backward
-// at N = 16384, Qwen shape: step 6797 -> 6555 us; forward alone 2101 -> 2002 us).
+// lane every descriptor and coordinate had to be moved into uniform registers one at a time (Qwen shape, the change alone:
+// forward of 16384 tokens with skewed routing 2104 -> 2019 us, of 4096 tokens 739 -> 709; training steps of 8192 tokens of
+// the LLaMA shape 2191 -> 2161, of 16384 of the Qwen shape 1 to 3 % in the power cap's spread, of 65536 none).
 // Pipelines: 5 shared-memory stages (full barrier in the even CTA counts both CTAs' bytes; the
 // MMA's commit frees the stage in both CTAs) and two TMEM accumulators of 256 columns, so the
 // epilogue of tile i overlaps the MMAs of tile i+1.  Every wait is bounded: on expiry the kernel

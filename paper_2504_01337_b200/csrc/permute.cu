@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const T* __restrict__ 
 
 // dWg[e, cols] = sum over expert e's rows r of dl[slot_of_row[r]] * Xp[r, cols].
 // grid (d / (32*VEC), E); the warps split the rows, four in flight each, partial sums merged in warp order.  Bound by the
-// latency of its loads: 8 warps with one row at a time took 33 us for 375 rows per expert 11.7 now.
+// latency of its loads (fp32, d = 256, 8 experts of 375 rows: 33 us with 8 warps of one row at a time, 11.7 so).
 constexpr int GW_WARPS = 32;
 template <typename T>
 __global__ void __launch_bounds__(GW_WARPS * 32) gate_wgrad_kernel(const T* __restrict__ Xp, const int32_t* __restrict__ counts,

@@ -1,4 +1,5 @@
-// Gate logits, C2R / Top-K routing, collaboration matrix, Top-T sets and dispatch volume.
+// C2R / Top-K routing, collaboration matrix, Top-T sets and dispatch volume; entry point of the gate logits, whose kernels are
+// in gate_tc.cu and gemm_simt.cu.
 // Integer outputs are exact and independent of scheduling (integer atomics only where the
 // result does not depend on their order).
 #include "c2r_common.cuh"
