@@ -73,3 +73,23 @@ def test_uneven_counts_take_the_same_kernel(counts):
         assert_close_rms(host(Yp)[rows], (s * Yref)[rows], 3e-2, "Yp", out_bf16=False)
     other = np.setdiff1d(np.arange(R), rows)  # rows that belong to no expert are left alone
     assert (host(Yp)[other] == 7.0).all() and (host(H)[other] == 7.0).all()
+
+
+@pytest.mark.parametrize("n", [1, 17, 100, 129])
+def test_a_token_gets_the_same_bits_from_either_kernel(n):
+    """Batches on both sides of the rule, alone and with the shared expert in the launch, against a large batch's first tokens."""
+    from paper_2504_01337_b200.layer import C2RLayer
+    wl = G.Workload("either", N=1500, d=336, E=8, I=400, K=3, T=4, P=2, I_s=528, bf16=True, seed=11)
+    X = G.hidden(wl)
+    Wg, wsg = G.gate_weights(wl)
+    W, sh, sets = G.expert_weights(wl), G.shared_weights(wl), random_sets(wl.E, wl.T, seed=5)
+    got = []
+    for m in (n, wl.N):
+        lay = C2RLayer(m, wl.d, wl.E, wl.I, wl.K, wl.T, wl.P, wl.I_s, True, backward=False)
+        lay.set_params(Wg, *W, wsg, sh)
+        lay.set_routing(mask=mask_of(sets, wl.E))
+        lay.set_input(X[:m])
+        lay.forward()
+        rows = lay.t["row_of_slot"].long()[:n * wl.K]
+        got.append([lay.t[x][:n] for x in ("L", "idx", "Ys", "Hs", "Y")] + [lay.t[x][rows] for x in ("H", "Yp")])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
