@@ -87,20 +87,20 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
 // chained kernel become resident as the SMs of the kernel before it fall free, and the first SMs to do so take as many as fit:
 // seven routing blocks on one SM, bound by its issue slots, while most of the chip waits (4096 tokens behind a pair GEMM: 24 us where
 // the kernel alone takes 9).  A block counts with what it asks for, so it asks for its share of an SM.
-constexpr int SPREAD_SMS = 148, SPREAD_SMEM = 226 * 1024;
+constexpr int SPREAD_SMS = 148, SPREAD_SMEM = 120 * 1024;
 inline int spread_smem(int64_t blocks, int need) {
   const int64_t per_sm = (blocks + SPREAD_SMS - 1) / SPREAD_SMS;
-  const int64_t share = per_sm > 0 && per_sm <= 16 ? SPREAD_SMEM / per_sm / 1024 * 1024 - 2048 : 0;
-  return share > need ? (int)share : need;
+  const int share = per_sm > 0 && per_sm <= 8 ? 227 * 1024 / ((int)per_sm + 1) + 1024 : 0;  // one more does not fit
+  return share > need ? share : need;
 }
-// Raises a kernel's limit of dynamic shared memory to what spread_smem may return, once per device (`done`: one flag each).
+// Raises a kernel's limit of dynamic shared memory, once per device (`done`: a flag each).
 template <typename... P>
-inline int allow_smem(void (*kernel)(P...), int (&done)[64]) {
+inline int allow_smem(void (*kernel)(P...), int (&done)[64], int bytes = SPREAD_SMEM) {
   int dev = 0;
   C2R_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return C2R_ERR_UNSUPPORTED_SHAPE;
   if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
-    C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_SMEM - 2048));
+    C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
   }
   return C2R_OK;

@@ -11,13 +11,13 @@ thread_local int g_last_cuda_error = 0;
 unsigned long long g_launch_count = 0;
 
 // ---------------------------------------------------------------------------------------------
-// Routing (Sec. 3.3 step 2).  A thread per token over logits staged in shared memory as order-preserving integer keys: K
-// scans, each for the best remaining candidate under the total order (value desc, index asc); after the first the candidates
-// are those in the top-1 expert's collaborator mask.  The kernel is bound by the instructions of the blocks it has -- their number is
-// fixed by the dispatch's blocking -- and a scan costs an instruction or two per logit for 32 tokens at once; a warp per token with
-// a warp-wide arg-max per round took several times as many
-// (16384 tokens, 60 experts, top-4: 13.5 us with a shuffle arg-max, 10.6 with an integer one, 8.8 here; 512 tokens, 8 experts,
-// top-2: 17.4, 13.2, 4.4).
+// Routing (Sec. 3.3 step 2).  LANES threads per token hold its logits in registers, eight each, as order-preserving integer
+// keys; K rounds, each a maximum and then the lowest index that has it under the total order (value desc, index asc), after
+// the first among the experts of the top-1 expert's collaborator mask.  The number of blocks is fixed by the dispatch's blocking,
+// at most one per SM up to 148 blocks, so a block's latency is what the kernel takes: a thread per token over keys staged in
+// shared memory waits for 60 dependent selects a round, here it is eight and three shuffles.  us a call, that way / this: 16384 tokens
+// of 60 experts, top-8 13.9 / 6.8, 24000 tokens, top-4 11.0 / 8.1, 40000 13.8 / 10.9, 65536 12.9 / 14.1 (bound by instructions, of which
+// this has some more); with p, 24000 tokens, top-2 26.6 / 10.5.  Behind a pair GEMM (4096 tokens) 24 / 6, as its blocks spread.
 // ---------------------------------------------------------------------------------------------
 // Order-preserving map of a logit to an unsigned key above 0 (-0 and +0 share one, as they compare equal); 0 marks an
 // expert that is not a candidate.
@@ -27,195 +27,152 @@ __device__ __forceinline__ uint32_t logit_key(float v) {
 }
 __device__ __forceinline__ float key_logit(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k); }
 
-// Keys per token in shared memory: whole groups of four, and odd, so that the threads of a warp read one expert's keys
-// without bank conflicts.
-__host__ __device__ inline int route_pitch(int E) { return (E + 3) / 4 * 4 + 1; }
-
-// The largest key among the candidates (bits of avail), lowest index first; key 0 and index -1 if there are none.  Four
-// interleaved chains of compare-and-select.
-__device__ __forceinline__ void best_candidate(const uint32_t* row, uint64_t avail, int E, uint32_t& key, int& sel) {
-  uint32_t b[4] = {0u, 0u, 0u, 0u};
-  int at[4] = {64, 64, 64, 64};
-  uint32_t bits = (uint32_t)avail;
-#pragma unroll 2
-  for (int e0 = 0; e0 < E; e0 += 4, bits >>= 4) {
-    if (e0 == 32) bits = (uint32_t)(avail >> 32);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t k = row[e0 + q] & (uint32_t)((int32_t)(bits << (31 - q)) >> 31);
-      at[q] = k > b[q] ? e0 + q : at[q];
-      b[q] = max(k, b[q]);
-    }
-  }
-  key = b[0]; sel = at[0];
-#pragma unroll
-  for (int q = 1; q < 4; ++q)
-    if (b[q] > key || (b[q] == key && at[q] < sel)) { key = b[q]; sel = at[q]; }
-  if (key == 0u) sel = -1;
-}
-
 // A block owns tokens_per_block consecutive tokens (the blocking of the dispatch's counting sort).  block_counts (optional):
 // [blocks][E] experts' slot counts of the block's tokens -- the histogram the dispatch starts from, so it need not read
 // idx again to build it.
 //
-// WARP_SOFTMAX: the full softmax by a warp per token, four tokens at a time, instead of a thread per token.
-template <int K, bool WARP_SOFTMAX>
-__global__ void __launch_bounds__(512) route_kernel(const float* __restrict__ L, const uint64_t* __restrict__ mask,
-                                                    int32_t* __restrict__ idx, float* __restrict__ w, float* __restrict__ p,
-                                                    int32_t* __restrict__ status, int N, int E, int renorm, int tokens_per_block,
-                                                    int32_t* __restrict__ block_counts) {
+// Lane l of a token's LANES holds experts 4 l .. 4 l + 3 and as many from 4 LANES on: E <= 8 LANES.  FULL: the softmax over all
+// experts is wanted, for p or for weights that are not renormalised.
+template <int K, int LANES, bool FULL>
+__global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* __restrict__ L, const uint64_t* __restrict__ mask,
+                                                     int32_t* __restrict__ idx, float* __restrict__ w, float* __restrict__ p,
+                                                     int32_t* __restrict__ status, int N, int E, int renorm, int tokens_per_block,
+                                                     int32_t* __restrict__ block_counts) {
   chain_begin();
-  extern __shared__ uint32_t s_key[];  // [tokens][route_pitch(E)]
   __shared__ uint64_t s_mask[64];
   __shared__ int s_cnt[64];
-  __shared__ float s_soft[WARP_SOFTMAX ? 128 : 1];  // a token's largest logit, then its denominator
-  const int tid = threadIdx.x;
+  constexpr int OWN = (K + LANES - 1) / LANES;  // selections a lane keeps: j = sub, sub + LANES, ..
+  const int tid = threadIdx.x, sub = tid & (LANES - 1);
   const int t_begin = blockIdx.x * tokens_per_block, tokens = min(N - t_begin, tokens_per_block);
-  const int pitch = route_pitch(E);
+  const bool vec = (E & 3) == 0 && ((uintptr_t)L & 15u) == 0;
+  int flags = 0;
+  auto expert = [&](int i) { return 4 * sub + (i & 3) + (i >> 2) * 4 * LANES; };
+  auto load = [&](int t, float (&v)[8]) {
+    const float* row = L + (size_t)(t_begin + min(t, tokens - 1)) * E;
+    if (vec) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (expert(4 * h) < E) x = *reinterpret_cast<const float4*>(row + expert(4 * h));
+        v[4 * h] = x.x; v[4 * h + 1] = x.y; v[4 * h + 2] = x.z; v[4 * h + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = expert(i) < E ? row[expert(i)] : 0.f;
+    }
+  };
+  const int per_pass = blockDim.x / LANES, t_warp = tid / 32 * (32 / LANES), t_lane = (tid & 31) / LANES;
+  float next[8];
+  load(t_warp + t_lane, next);
   if (tid < 64) {
     s_cnt[tid] = 0;
     s_mask[tid] = (tid < E && mask != nullptr) ? mask[tid] : ~0ull;
   }
-  int flags = 0;
-  {
-    // eight loads in flight per thread (clamped, not predicated: a load under a condition waits for the one before it)
-    const float* src = L + (size_t)t_begin * E;
-    auto put = [&](int at, float v) {
-      if (v != v) { v = -INFINITY; flags |= C2R_STATUS_NAN_LOGIT; }
-      s_key[at] = logit_key(v);
-    };
-    if ((E & 3) == 0 && ((uintptr_t)L & 15u) == 0) {
-      const int per = E >> 2, n = tokens * per;
-      for (int i0 = tid; i0 < n; i0 += 8 * blockDim.x) {
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = reinterpret_cast<const float4*>(src)[min(i0 + u * (int)blockDim.x, n - 1)];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int i = i0 + u * blockDim.x, at = 4 * i + i / per;  // pitch E + 1
-          if (i < n) { put(at, v[u].x); put(at + 1, v[u].y); put(at + 2, v[u].z); put(at + 3, v[u].w); }
-        }
-      }
-    } else {
-      const int n = tokens * E;
-      for (int i0 = tid; i0 < n; i0 += 8 * blockDim.x) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = src[min(i0 + u * (int)blockDim.x, n - 1)];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int i = i0 + u * blockDim.x;
-          if (i < n) put(i / E * pitch + i % E, v[u]);
-        }
-      }
-    }
-  }
   __syncthreads();
-  const size_t o = (size_t)(t_begin + tid) * K;
-  float lg[K];
-  if (tid < tokens) {
-    uint32_t* row = s_key + tid * pitch;
-    uint32_t key[K];
-    int sel[K];
-    uint64_t avail = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
+  for (int t0 = t_warp; t0 < tokens; t0 += per_pass) {  // warp-uniform
+    const int t = t0 + t_lane;
+    const bool live = t < tokens;
+    uint32_t key[8];
 #pragma unroll
-    for (int j = 0; j < K; ++j) {
-      best_candidate(row, avail, E, key[j], sel[j]);
-      if (sel[j] >= 0) avail &= ~(1ull << sel[j]);
-      if (j == 0) avail &= s_mask[sel[0]];
+    for (int i = 0; i < 8; ++i) {
+      float v = next[i];
+      if (v != v) { v = -INFINITY; if (live) flags |= C2R_STATUS_NAN_LOGIT; }
+      key[i] = expert(i) < E ? logit_key(v) : 0u;
     }
-    // Eq. 1 weights.  The round-0 logit is the row maximum, so it is the softmax shift for both forms.
-    float ek[8];
-#pragma unroll
-    for (int j = 0; j < K; ++j) lg[j] = sel[j] >= 0 ? key_logit(key[j]) : -INFINITY;
+    if (t0 + per_pass < tokens) load(t + per_pass, next);
+    float ex[FULL ? 8 : 1], top = 0.f, lg[OWN];
+    int own[OWN];
     uint64_t chosen = 0;
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-      if (sel[j] < 0) {  // candidate set exhausted: fall back to the lowest unselected expert
-        flags |= C2R_STATUS_SET_TOO_SMALL;
+      uint32_t m = max(max(max(key[0], key[1]), max(key[2], key[3])), max(max(key[4], key[5]), max(key[6], key[7])));
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      int sel = 64;
+#pragma unroll
+      for (int i = 7; i >= 0; --i) sel = key[i] == m ? expert(i) : sel;
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) sel = min(sel, __shfl_xor_sync(0xffffffffu, sel, o));
+      if (j == 0) {
+        top = key_logit(m);
+        if (FULL) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) ex[FULL ? i : 0] = expert(i) < E ? expf(key_logit(key[i]) - top) : 0.f;
+        }
+        const uint64_t set = s_mask[sel];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t bits = (uint32_t)(set >> ((4 * sub + h * 4 * LANES) & 63));
+#pragma unroll
+          for (int i = 0; i < 4; ++i) key[4 * h + i] = (bits >> i & 1u) ? key[4 * h + i] : 0u;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) key[i] = expert(i) == sel ? 0u : key[i];
+      if (m == 0u) {  // candidate set exhausted: fall back to the lowest unselected expert
+        if (live) flags |= C2R_STATUS_SET_TOO_SMALL;
         const uint64_t valid = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
-        sel[j] = __ffsll((long long)(valid & ~chosen)) - 1;
+        sel = __ffsll((long long)(valid & ~chosen)) - 1;
       }
-      chosen |= 1ull << sel[j];
+      chosen |= 1ull << sel;
+      if ((j & (LANES - 1)) == sub) { own[j / LANES] = sel; lg[j / LANES] = m != 0u ? key_logit(m) : -INFINITY; }
     }
-    const float top = lg[0];
+    // Eq. 1 weights.  The round-0 logit is the row maximum, so it is the softmax shift for both forms.  Sums are binary trees:
+    // over the slot (distances 4, 2, 1), over the expert index (32, 16, 8, 4, 2, 1).
+    float denom = 0.f;
     if (renorm) {
+      float part[8 / LANES > 0 ? 8 / LANES : 1];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) ek[j] = j < K ? expf(lg[j < K ? j : 0] - top) : 0.f;
-      const float denom = ((ek[0] + ek[4]) + (ek[2] + ek[6])) + ((ek[1] + ek[5]) + (ek[3] + ek[7]));
+      for (int q = 0; q < 8 / LANES; ++q) part[q] = q < OWN && sub + q * LANES < K ? expf(lg[q < OWN ? q : 0] - top) : 0.f;
 #pragma unroll
-      for (int j = 0; j < K; ++j) w[o + j] = ek[j] / denom;
+      for (int h = 4 / LANES; h > 0; h >>= 1)
+#pragma unroll
+        for (int q = 0; q < h; ++q) part[q] += part[q + h];
+      denom = part[0];
+#pragma unroll
+      for (int o = LANES / 2; o > 0; o >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, o);
     }
-    if (WARP_SOFTMAX) {
-      s_soft[tid] = top;
-    } else if (!renorm || p != nullptr) {  // the full softmax, summed as a binary tree over the expert index
-      float s16[16];
+    if (FULL) {
+      float u[4];
 #pragma unroll
-      for (int x = 0; x < 16; ++x) {
-        float v[4];
+      for (int i = 0; i < 4; ++i) {
+        u[i] = ex[FULL ? i : 0] + ex[FULL ? 4 + i : 0];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = x + 16 * q < E ? expf(key_logit(row[x + 16 * q]) - top) : 0.f;
-        s16[x] = (v[0] + v[2]) + (v[1] + v[3]);
+        for (int o = LANES / 2; o > 0; o >>= 1) u[i] += __shfl_xor_sync(0xffffffffu, u[i], o);
       }
-#pragma unroll
-      for (int h = 8; h > 0; h >>= 1)
-#pragma unroll
-        for (int x = 0; x < 8; ++x)
-          if (x < h) s16[x] += s16[x + h];
-      if (p != nullptr)
-        for (int e = 0; e < E; ++e) row[e] = __float_as_uint(expf(key_logit(row[e]) - top) / s16[0]);
-      if (!renorm) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) w[o + j] = expf(lg[j] - top) / s16[0];
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      idx[o + j] = sel[j];
-      if (block_counts != nullptr) atomicAdd(&s_cnt[sel[j]], 1);  // integer counts: the order does not matter
-    }
-  }
-  if (WARP_SOFTMAX) {  // the same tree of additions over lanes
-    __syncthreads();
-    constexpr int U = 4;
-    const int lane = tid & 31, warps = blockDim.x >> 5;
-    for (int t0 = tid >> 5; t0 < tokens; t0 += U * warps) {
-      float e0[U], e1[U], s[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int t = t0 + u * warps < tokens ? t0 + u * warps : t0;
-        const uint32_t* row = s_key + t * pitch;
-        e0[u] = lane < E ? expf(key_logit(row[lane]) - s_soft[t]) : 0.f;
-        e1[u] = lane + 32 < E ? expf(key_logit(row[lane + 32]) - s_soft[t]) : 0.f;
-        s[u] = e0[u] + e1[u];
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int u = 0; u < U; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], off);
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int t = t0 + u * warps;
-        if (t >= tokens) break;
+      const float sum = (u[0] + u[2]) + (u[1] + u[3]);
+      if (!renorm) denom = sum;
+      if (p != nullptr && live) {
         float* out = p + (size_t)(t_begin + t) * E;
-        if (lane < E) out[lane] = e0[u] / s[u];
-        if (lane + 32 < E) out[lane + 32] = e1[u] / s[u];
-        if (lane == 0) s_soft[t] = s[u];
+        if (vec && ((uintptr_t)p & 15u) == 0) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (expert(4 * h) < E)
+              *reinterpret_cast<float4*>(out + expert(4 * h)) =
+                  make_float4(ex[FULL ? 4 * h : 0] / sum, ex[FULL ? 4 * h + 1 : 0] / sum, ex[FULL ? 4 * h + 2 : 0] / sum, ex[FULL ? 4 * h + 3 : 0] / sum);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (expert(i) < E) out[expert(i)] = ex[FULL ? i : 0] / sum;
+        }
       }
     }
-    if (!renorm) {
-      __syncthreads();
-      if (tid < tokens) {
+    if (live) {
+      const size_t o = (size_t)(t_begin + t) * K;
 #pragma unroll
-        for (int j = 0; j < K; ++j) w[o + j] = expf(lg[j] - lg[0]) / s_soft[tid];
+      for (int q = 0; q < OWN; ++q) {
+        const int j = sub + q * LANES;
+        if (j < K) {
+          idx[o + j] = own[q];
+          w[o + j] = expf(lg[q] - top) / denom;
+          if (block_counts != nullptr) atomicAdd(&s_cnt[own[q]], 1);  // integer counts: the order does not matter
+        }
       }
     }
   }
-  if (block_counts != nullptr || (p != nullptr && !WARP_SOFTMAX)) {
+  if (block_counts != nullptr) {
     __syncthreads();
-    if (block_counts != nullptr && tid < E) block_counts[(size_t)blockIdx.x * E + tid] = s_cnt[tid];
-    if (p != nullptr && !WARP_SOFTMAX)
-      for (int i = tid; i < tokens * E; i += blockDim.x) p[(size_t)t_begin * E + i] = __uint_as_float(s_key[i / E * pitch + i % E]);
+    if (tid < E) block_counts[(size_t)blockIdx.x * E + tid] = s_cnt[tid];
   }
   if (status != nullptr) {
     flags = __reduce_or_sync(0xffffffffu, flags);
@@ -223,36 +180,34 @@ __global__ void __launch_bounds__(512) route_kernel(const float* __restrict__ L,
   }
 }
 
-// Blocks of few tokens (at most 128: K >= 4, or a batch that small) over many experts leave a thread 2 E exponentials one
-// after another, and the block four warps to hide them with: there the full softmax takes warps, and the block 512 threads
-// (us with p, 60 experts, thread / warp: 1000 tokens top-4 18.5 / 8.5, top-8 18.3 / 9.8, 100 tokens top-1 12.3 / 5.7).  Few
-// experts leave its lanes idle (1000 tokens, 8 experts, top-4: 6.2 / 10.4), and many blocks fill the chip with either: up to
-// four blocks per SM (512 blocks 29.3 / 20.1, 1024 blocks 25.6 / 31.5, 33 experts).
-template <int K, bool WARP_SOFTMAX = false>
+template <int K, int LANES, bool FULL>
 static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
                         int32_t* status, int32_t* block_counts, cudaStream_t s) {
-  const int tpb = perm_tokens_per_block(K);
-  if constexpr (!WARP_SOFTMAX)
-    if (p != nullptr && cfg->E > 32 && (cfg->N < tpb ? cfg->N : tpb) <= 128 && cfg->N <= (int64_t)4 * 148 * tpb)
-      return route_launch<K, true>(cfg, L, mask, idx, w, p, status, block_counts, s);
-  const int threads = WARP_SOFTMAX ? 512 : tpb < 128 ? 128 : (tpb + 31) / 32 * 32;
-  const int smem = tpb * route_pitch(cfg->E) * (int)sizeof(uint32_t);
-  if (smem > 48 * 1024) {
-    constexpr int MAX_DEV = 64;
-    static int done[MAX_DEV] = {};  // the kernel's shared-memory limit is set on this device
-    int dev = 0;
-    C2R_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= MAX_DEV) return C2R_ERR_UNSUPPORTED_SHAPE;
-    if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
-      C2R_CUDA(cudaFuncSetAttribute(route_kernel<K, WARP_SOFTMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    perm_tokens_per_block(K) * route_pitch(64) * (int)sizeof(uint32_t)));
-      __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
-    }
-  }
-  C2R_CUDA(launch_chained(route_kernel<K, WARP_SOFTMAX>, (cfg->N + tpb - 1) / tpb, threads, smem, s, L, mask, idx, w, p, status, cfg->N, cfg->E, cfg->renorm, tpb,
-                          block_counts));
+  const int tpb = perm_tokens_per_block(K), most = (cfg->N < tpb ? cfg->N : tpb) * LANES;
+  const int blocks = (cfg->N + tpb - 1) / tpb;
+  // one block per SM with all its tokens at once; beyond, blocks that fit an SM together
+  const int limit = (FULL ? 512 : 1024) >> (blocks > SPREAD_SMS);
+  const int threads = most > limit ? limit : most < 64 ? 64 : (most + 31) / 32 * 32;  // at least the 64 that handle the mask and the counts
+  static int done[64] = {};
+  const int rc = allow_smem(route_kernel<K, LANES, FULL>, done);
+  if (rc) return rc;
+  C2R_CUDA(launch_chained(route_kernel<K, LANES, FULL>, blocks, threads, spread_smem(blocks, 0), s, L, mask, idx, w, p, status, cfg->N, cfg->E,
+                          cfg->renorm, tpb, block_counts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
+}
+template <int K, bool FULL>
+static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
+                        int32_t* status, int32_t* block_counts, cudaStream_t s) {
+  return cfg->E <= 16   ? route_launch<K, 2, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s)
+         : cfg->E <= 32 ? route_launch<K, 4, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s)
+                        : route_launch<K, 8, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s);
+}
+template <int K>
+static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
+                        int32_t* status, int32_t* block_counts, cudaStream_t s) {
+  return p != nullptr || !cfg->renorm ? route_launch<K, true>(cfg, L, mask, idx, w, p, status, block_counts, s)
+                                      : route_launch<K, false>(cfg, L, mask, idx, w, p, status, block_counts, s);
 }
 
 __global__ void route_bwd_kernel(const float* __restrict__ w, const float* __restrict__ dw, float* __restrict__ dl,
