@@ -16,12 +16,15 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// Expert key of slot s (clamped into [0,E); -1 = the slot takes no part: past the end, or a negative key when
+// Whether this thread's slot of the block exists.
+__device__ __forceinline__ bool slot_live(long long NK, int slots_per_block) {
+  return (int)(threadIdx.x & ~31u) < slots_per_block && (long long)blockIdx.x * slots_per_block + threadIdx.x < NK;
+}
+
+// Expert key of a slot that holds e (clamped into [0,E); -1 = the slot takes no part: it does not exist, or a negative key when
 // skip_negative is set, which the de-duplicated dispatch uses).
-__device__ __forceinline__ int slot_key(const int32_t* __restrict__ idx, long long s, long long NK, int E, int skip_negative,
-                                        int& flags) {
-  if (s >= NK) return -1;
-  int e = idx[s];
+__device__ __forceinline__ int slot_key(int e, bool live, int E, int skip_negative, int& flags) {
+  if (!live) return -1;
   if (e < 0 || e >= E) {
     if (skip_negative && e < 0) return -1;
     flags |= C2R_STATUS_BAD_INDEX;
@@ -32,27 +35,26 @@ __device__ __forceinline__ int slot_key(const int32_t* __restrict__ idx, long lo
 
 // Per-group, per-expert counts of this block's slots: inside a 32-slot group, lanes with equal expert form a
 // peer set (match.any) whose lowest lane records the set size -- no atomics, and the order of slots is kept.
-// grp_cnt must be zero on entry.  Returns this thread's key.
-__device__ __forceinline__ int group_count(const int32_t* __restrict__ idx, long long NK, int E, int slots_per_block,
-                                           int (*grp_cnt)[64], int& flags, int skip_negative) {
+// grp_cnt must be zero on entry.  raw: what the thread's slot holds, if it is live.  Returns this thread's key.
+__device__ __forceinline__ int group_count(int raw, bool live, int E, int (*grp_cnt)[64], int& flags, int skip_negative) {
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-  int e = -1;
-  if (32 * g < slots_per_block)
-    e = slot_key(idx, (long long)blockIdx.x * slots_per_block + threadIdx.x, NK, E, skip_negative, flags);
+  const int e = slot_key(raw, live, E, skip_negative, flags);
   const uint32_t peers = __match_any_sync(0xffffffffu, e);
   if (e >= 0 && lane == __ffs(peers) - 1) grp_cnt[g][e] = __popc(peers);
   return e;
 }
 
-// Layout position -> expert from expert_rank (NULL = identity).  A table that is not a permutation of
-// [0,E) (an entry out of range, a duplicate, hence a hole) is replaced by the identity order and reported.
-// All threads of the block must call; needs E <= 64 <= blockDim.x.  Ends with a barrier.
-__device__ __forceinline__ void layout_order(const int32_t* __restrict__ expert_rank, int E, int* s_by_rank, int* s_bad) {
+// Layout position -> expert from the experts' ranks: thread e < E passes its expert's, from expert_rank (NULL = identity).  A
+// table that is not a permutation of [0,E) (an entry out of range, a duplicate, hence a hole) is replaced by the identity
+// order and reported.  All threads of the block must call; needs E <= 64 <= blockDim.x.  Ends with a barrier.
+__device__ __forceinline__ int rank_of_thread(const int32_t* __restrict__ expert_rank, int E) {
+  return expert_rank != nullptr && (int)threadIdx.x < E ? expert_rank[threadIdx.x] : (int)threadIdx.x;
+}
+__device__ __forceinline__ void layout_order(int r, int E, int* s_by_rank, int* s_bad) {
   if (threadIdx.x < 64) s_by_rank[threadIdx.x] = -1;
   if (threadIdx.x == 0) *s_bad = 0;
   __syncthreads();
   if ((int)threadIdx.x < E) {
-    const int r = expert_rank ? expert_rank[threadIdx.x] : (int)threadIdx.x;
     if (r < 0 || r >= E) *s_bad = 1;
     else s_by_rank[r] = threadIdx.x;  // duplicates: one writer wins and some other position stays -1
   }
@@ -88,9 +90,11 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_hist_kernel(const int32_t* 
   chain_begin();
   __shared__ int grp_cnt[PERM_GROUPS][64];
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) (&grp_cnt[0][0])[i] = 0;
+  const bool live = slot_live(NK, slots_per_block);
+  const int raw = live ? idx[(long long)blockIdx.x * slots_per_block + threadIdx.x] : 0;
   __syncthreads();
   int flags = 0;
-  group_count(idx, NK, E, slots_per_block, grp_cnt, flags, skip_negative);
+  group_count(raw, live, E, grp_cnt, flags, skip_negative);
   __syncthreads();
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
     int s = 0;
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ b
     }
     if (lane == 0) s_counts[e] = running;
   }
-  layout_order(expert_rank, E, s_by_rank, &s_bad);
+  layout_order(rank_of_thread(expert_rank, E), E, s_by_rank, &s_bad);
   segment_offsets(s_by_rank, s_counts, E, row_align, offsets);
   if (threadIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
   if (threadIdx.x < E) counts[threadIdx.x] = s_counts[threadIdx.x];
@@ -136,11 +140,10 @@ __global__ void __launch_bounds__(1024) perm_scan_kernel(int32_t* __restrict__ b
 
 // Stable rank of a block's slots once grp_cnt holds the per-group counts and s_start[e] the row at which the
 // block's first slot of expert e lands: rows of earlier groups of the block, then lower lanes of the group.
-// w (optional): w_row[row] = w[slot], the routing weight of the slot that owns the row.  slot_of_row gets slot / slot_div.
-__device__ __forceinline__ void rank_and_write(int e, long long NK, int E, int slots_per_block, int (*grp_cnt)[64],
+// w_row (optional): w_row[row] = weight, the routing weight of the slot that owns the row.  slot_of_row gets slot / slot_div.
+__device__ __forceinline__ void rank_and_write(int e, int E, int slots_per_block, int (*grp_cnt)[64],
                                                const int* s_start, int32_t* __restrict__ row_of_slot,
-                                               int32_t* __restrict__ slot_of_row, const float* __restrict__ w,
-                                               float* __restrict__ w_row, int slot_div = 1, int* my_row = nullptr) {
+                                               int32_t* __restrict__ slot_of_row, float weight, float* __restrict__ w_row, int slot_div = 1, int* my_row = nullptr) {
   for (int x = threadIdx.x; x < E; x += blockDim.x) {
     int run = s_start[x];
 #pragma unroll
@@ -158,7 +161,7 @@ __device__ __forceinline__ void rank_and_write(int e, long long NK, int E, int s
     const int row = grp_cnt[g][e] + __popc(peers & lanemask_lt());
     row_of_slot[s] = row;
     slot_of_row[row] = slot_div == 1 ? (int32_t)s : (int32_t)(s / slot_div);
-    if (w_row != nullptr) w_row[row] = w[s];
+    if (w_row != nullptr) w_row[row] = weight;
     if (my_row != nullptr) *my_row = row;
   }
 }
@@ -175,11 +178,15 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_kernel(const int32_t* 
   __shared__ int s_start[64];
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) (&grp_cnt[0][0])[i] = 0;
   for (int e = threadIdx.x; e < E; e += blockDim.x) s_start[e] = offsets[e] + block_base[(size_t)blockIdx.x * E + e];
+  const bool live = slot_live(NK, slots_per_block);
+  const long long slot = (long long)blockIdx.x * slots_per_block + threadIdx.x;
+  const int raw = live ? idx[slot] : 0;
+  const float weight = live && w_row != nullptr ? w[slot] : 0.f;
   __syncthreads();
   int flags = 0;
-  const int e = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, skip_negative);
+  const int e = group_count(raw, live, E, grp_cnt, flags, skip_negative);
   __syncthreads();
-  rank_and_write(e, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, w, w_row);
+  rank_and_write(e, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, weight, w_row);
 }
 
 // The scan folded into the rank pass (for batches of at most PERM_FUSED_MAX_BLOCKS blocks): every block
@@ -194,21 +201,29 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_kernel(const int32_t* 
 // and slot_of_row holds tokens (slot / K).
 constexpr int PERM_FUSED_MAX_BLOCKS = 1024;
 constexpr int PERM_MARK_BLOCKS = 16;
+struct RankArgs {
+  const int32_t* idx;
+  const int32_t* block_counts;
+  const int32_t* expert_rank;
+  int32_t *counts, *offsets, *row_of_slot, *slot_of_row;
+  const float* w;
+  float* w_row;
+  int32_t* status;
+  long long R;
+  int E, row_align;
+};
 template <bool DEDUP>
-__global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int32_t* __restrict__ idx, long long NK, int E,
-                                                                       int slots_per_block,
-                                                                       const int32_t* __restrict__ block_counts,
-                                                                       int n_blocks,
-                                                                       const int32_t* __restrict__ expert_rank,
-                                                                       int row_align, long long R,
-                                                                       int32_t* __restrict__ counts,
-                                                                       int32_t* __restrict__ offsets,
-                                                                       int32_t* __restrict__ row_of_slot,
-                                                                       int32_t* __restrict__ slot_of_row,
-                                                                       const float* __restrict__ w,
-                                                                       float* __restrict__ w_row,
-                                                                       int32_t* __restrict__ status, int K) {
-  chain_begin();
+__device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int slots_per_block, int n_blocks, int K) {
+  const int E = a.E, row_align = a.row_align;
+  int32_t* __restrict__ slot_of_row = a.slot_of_row;
+  int32_t* __restrict__ row_of_slot = a.row_of_slot;
+  float* __restrict__ w_row = a.w_row;
+  // everything the block reads from global memory is asked for before the first barrier
+  const long long slot = (long long)blockIdx.x * slots_per_block + threadIdx.x;
+  const bool live = slot_live(NK, slots_per_block);
+  const int raw = live ? a.idx[slot] : 0;
+  const float weight = live && w_row != nullptr ? a.w[slot] : 0.f;
+  const int rank_mine = rank_of_thread(a.expert_rank, E);
   constexpr int PARTS = PERM_THREADS / 64;
   __shared__ int grp_cnt[PERM_GROUPS][64];
   __shared__ int s_start[64], s_total[64], s_by_rank[64], s_off[65];
@@ -221,7 +236,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
     if (e < E) {
 #pragma unroll 8
       for (int b = part; b < n_blocks; b += PARTS) {
-        const int v = block_counts[(size_t)b * E + e];
+        const int v = a.block_counts[(size_t)b * E + e];
         total += v;
         before += (b < (int)blockIdx.x) ? v : 0;
       }
@@ -229,7 +244,7 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
     s_part[0][part][e] = before;
     s_part[1][part][e] = total;
   }
-  layout_order(expert_rank, E, s_by_rank, &s_bad);  // (its barriers also publish s_part and the zeroed grp_cnt)
+  layout_order(rank_mine, E, s_by_rank, &s_bad);  // (its barriers also publish s_part and the zeroed grp_cnt)
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
     int before = 0, total = 0;
 #pragma unroll
@@ -239,14 +254,14 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
   }
   __syncthreads();
   segment_offsets(s_by_rank, s_total, E, row_align, s_off);
-  if (threadIdx.x == 0 && blockIdx.x == 0 && s_bad && status != nullptr) atomicOr(status, C2R_STATUS_BAD_INDEX);
+  if (threadIdx.x == 0 && blockIdx.x == 0 && s_bad && a.status != nullptr) atomicOr(a.status, C2R_STATUS_BAD_INDEX);
   int flags = 0;
-  const int e_mine = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, DEDUP);
+  const int e_mine = group_count(raw, live, E, grp_cnt, flags, DEDUP);
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int e = threadIdx.x; e <= E; e += blockDim.x) {
-      offsets[e] = s_off[e];
-      if (e < E) counts[e] = s_total[e];
+      a.offsets[e] = s_off[e];
+      if (e < E) a.counts[e] = s_total[e];
     }
   }
   // rows without a slot: the padding that closes each segment and the rows past the layout, all blocks together
@@ -258,28 +273,46 @@ __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const int
       if (w_row != nullptr) w_row[r] = 0.f;
     }
   }
-  for (long long r = s_off[E] + first; r < R; r += stride) {
+  for (long long r = s_off[E] + first; r < a.R; r += stride) {
     slot_of_row[r] = -1;
     if (w_row != nullptr) w_row[r] = 0.f;
   }
   for (int e = threadIdx.x; e < E; e += blockDim.x) s_start[e] += s_off[e];
   __syncthreads();
   if constexpr (!DEDUP) {
-    rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, w, w_row);
+    rank_and_write(e_mine, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, weight, w_row);
   } else {
     __shared__ int s_row[PERM_THREADS], s_q[PERM_THREADS];
     int row = -1;
-    rank_and_write(e_mine, NK, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, nullptr, nullptr, K, &row);
+    rank_and_write(e_mine, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, 0.f, nullptr, K, &row);
     s_row[threadIdx.x] = row;
     s_q[threadIdx.x] = e_mine;
     __syncthreads();
-    const long long slot = (long long)blockIdx.x * slots_per_block + threadIdx.x;
-    if ((int)threadIdx.x < slots_per_block && slot < NK && e_mine < 0) {  // a block owns whole tokens
-      const int q = -2 - idx[slot];
+    if (live && e_mine < 0) {  // a block owns whole tokens
+      const int q = -2 - raw;
       for (int j = threadIdx.x / K * K; j < (int)threadIdx.x; ++j)
         if (s_q[j] == q) { row_of_slot[slot] = s_row[j]; break; }
     }
   }
+}
+
+// Blocks y = 0: `a`.  y = 1 (the two-stage dispatch): the receive side's `b`, which only needs the same histogram launch.
+template <bool TWO>
+__global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const RankArgs a, const RankArgs b, long long NK, int slots_per_block,
+                                                                       int n_blocks, int K) {
+  chain_begin();
+  if (TWO && blockIdx.y == 1) rank_block<true>(b, NK, slots_per_block, n_blocks, K);
+  else rank_block<false>(a, NK, slots_per_block, n_blocks, K);
+}
+template <bool TWO>
+static int rank_launch(const RankArgs& a, const RankArgs& b, long long NK, int slots_per_block, int n_blocks, int grid, int K, cudaStream_t s) {
+  static int done[64] = {};
+  const int rc = allow_smem(perm_rank_fused_kernel<TWO>, done);
+  if (rc) return rc;
+  C2R_CUDA(launch_chained(perm_rank_fused_kernel<TWO>, dim3(grid, TWO ? 2 : 1), PERM_THREADS, spread_smem((TWO ? 2 : 1) * grid, 0), s, a, b, NK,
+                          slots_per_block, n_blocks, K));
+  C2R_LAUNCH_CHECK();
+  return C2R_OK;
 }
 
 // Warps over which a token's row is spread where there are few tokens: enough for 32 warps per SM, each with at least one
@@ -780,9 +813,9 @@ int permute_impl(const c2r_config* cfg, const int32_t* idx, const int32_t* exper
   if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
     // a batch of few blocks still has up to row_align - 1 padding rows per expert to mark: blocks without slots help with them
     const int grid = nb < PERM_MARK_BLOCKS && cfg->row_align > 1 ? PERM_MARK_BLOCKS : nb;
-    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, grid, PERM_THREADS, 0, s, idx, NK, cfg->E, spb, block_counts, nb, expert_rank, cfg->row_align,
-                          R, counts, offsets, row_of_slot, slot_of_row, w, w_row, status, (int)cfg->K));
-    C2R_LAUNCH_CHECK();
+    const RankArgs a = {idx, block_counts, expert_rank, counts, offsets, row_of_slot, slot_of_row, w, w_row, status, R, cfg->E, cfg->row_align};
+    const int rc = rank_launch<false>(a, a, NK, spb, nb, grid, cfg->K, s);
+    if (rc) return rc;
   } else {
     C2R_CUDA(cudaMemsetAsync(slot_of_row, 0xFF, sizeof(int32_t) * R, s));
     if (w_row != nullptr) C2R_CUDA(cudaMemsetAsync(w_row, 0, sizeof(float) * R, s));
@@ -1089,11 +1122,15 @@ __global__ void __launch_bounds__(PERM_THREADS) dedup_hist_kernel(const int32_t*
   chain_begin();
   __shared__ int grp_cnt[PERM_GROUPS][64], grp_cnt_p[PERM_GROUPS][64];
   __shared__ int s_q[PERM_THREADS];
+  __shared__ int s_part[64];
+  const bool live = slot_live(NK, slots_per_block);
+  const int raw = live ? idx[(long long)blockIdx.x * slots_per_block + threadIdx.x] : 0;
+  if ((int)threadIdx.x < E) s_part[threadIdx.x] = min(max(part[threadIdx.x], 0), P - 1);
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) { (&grp_cnt[0][0])[i] = 0; (&grp_cnt_p[0][0])[i] = 0; }
   __syncthreads();
   int flags = 0;
-  const int e = group_count(idx, NK, E, slots_per_block, grp_cnt, flags, 0);
-  const int q = e >= 0 ? min(max(part[e], 0), P - 1) : -1;
+  const int e = group_count(raw, live, E, grp_cnt, flags, 0);
+  const int q = e >= 0 ? s_part[e] : -1;
   s_q[threadIdx.x] = q;
   __syncthreads();
   int first = q;
@@ -1216,17 +1253,17 @@ static int dispatch_dedup_impl(const c2r_config* cfg, const int32_t* idx, const 
   const int nb = perm_blocks(cfg);
   const int spb = perm_tokens_per_block(K) * K;
   if (nb > 0 && nb <= PERM_FUSED_MAX_BLOCKS) {
-    // Three launches for both indices (eleven took 39 us of 16384 tokens' dispatch).  scratch: [nb][P] block counts, which fit:
+    // Two launches for both indices (eleven took 39 us of 16384 tokens' dispatch, three 17, these 9).  scratch: [nb][P] block counts, which fit:
     // a block but the last owns at least 448 slots and P is at most 64, and the area is a whole number of 256 bytes.
-    C2R_CUDA(launch_chained(dedup_hist_kernel, nb, PERM_THREADS, 0, s, idx, part, NK, E, K, P, spb, block_counts, scratch, key,
+    static int done[64] = {};
+    if (const int rc = allow_smem(dedup_hist_kernel, done)) return rc;
+    C2R_CUDA(launch_chained(dedup_hist_kernel, nb, PERM_THREADS, spread_smem(nb, 0), s, idx, part, NK, E, K, P, spb, block_counts, scratch, key,
                             status));
     C2R_LAUNCH_CHECK();
-    C2R_CUDA(launch_chained(perm_rank_fused_kernel<false>, nb, PERM_THREADS, 0, s, idx, NK, E, spb, block_counts, nb, expert_rank,
-                            cfg->row_align, R, counts, offsets, row_of_slot, slot_of_row, nullptr, nullptr, status, K));
-    C2R_LAUNCH_CHECK();
-    C2R_CUDA(launch_chained(perm_rank_fused_kernel<true>, nb, PERM_THREADS, 0, s, key, NK, P, spb, scratch, nb, nullptr, 1, cap,
-                            recv_counts, recv_offsets, recv_row_of_slot, token_of_recv_row, nullptr, nullptr, nullptr, K));
-    C2R_LAUNCH_CHECK();
+    const RankArgs a = {idx, block_counts, expert_rank, counts, offsets, row_of_slot, slot_of_row, nullptr, nullptr, status, R, E, cfg->row_align};
+    const RankArgs b = {key, scratch, nullptr, recv_counts, recv_offsets, recv_row_of_slot, token_of_recv_row, nullptr, nullptr, nullptr, cap, P, 1};
+    const int rc = rank_launch<true>(a, b, NK, spb, nb, nb, K, s);
+    if (rc) return rc;
   } else {
     // the per-expert layout itself (counts, offsets, both row maps) is the plain dispatch's
     int rc = permute_impl<T>(cfg, idx, expert_rank, nullptr, counts, offsets, row_of_slot, slot_of_row, nullptr, status, ws, s,
