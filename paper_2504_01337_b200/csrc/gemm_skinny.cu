@@ -91,18 +91,6 @@ __device__ __forceinline__ bool skinny_unit(const SkinnyParams& p, const int (*s
   return true;
 }
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z, int w) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
-      : "memory");
-}
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 // Barrier of the epilogue warps that also agrees on whether all of them may go on.
 __device__ __forceinline__ bool epilogue_all(bool ok) {
@@ -340,22 +328,6 @@ bool skinny_supported(const c2r_config* cfg, const SwigluCall& a, int max_rows) 
   const uintptr_t bits = (uintptr_t)a.Xp | (uintptr_t)a.W13p | (uintptr_t)a.W2 | (uintptr_t)a.H | (uintptr_t)a.Yp;
   return a.AB == nullptr && a.X == nullptr && a.token_acc == nullptr && a.Xp != nullptr && a.Yp != nullptr &&
          (bits & 15u) == 0 && expected_rows(cfg, a) <= max_rows;
-}
-
-// bf16 rows of length K viewed as [groups][k-block][row][64] for boxes of ks k-blocks x `rows` rows: a stage's k-blocks come
-// with one TMA instruction and lie in shared memory the way the MMA descriptors walk them.
-static int slab_map(CUtensorMap* m, const void* base, int64_t K, int64_t n_rows, int64_t kfull, int64_t groups, int rows, int ks) {
-  EncodeTiledFn enc = get_encode();
-  if (!enc) return C2R_ERR_CUDA;
-  cuuint64_t dims[4] = {BK, (cuuint64_t)n_rows, (cuuint64_t)kfull, (cuuint64_t)groups};
-  cuuint64_t strides[3] = {(cuuint64_t)K * 2, BK * 2, (cuuint64_t)(K * n_rows) * 2};
-  cuuint32_t box[4] = {BK, (cuuint32_t)rows, (cuuint32_t)ks, 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { g_last_cuda_error = (int)cudaErrorInvalidValue; return C2R_ERR_CUDA; }
-  return C2R_OK;
 }
 
 static int skinny_launch(const c2r_config* cfg, const SwigluCall* calls, int n, bool up, cudaStream_t s) {

@@ -61,6 +61,12 @@ def test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared):
     assert torch.equal(big[:N], L) and torch.equal(zb[:N], z)
 
 
+# experts in tiles of 16 and of 32, a last one that is not full, whole, or alone; contractions shorter and longer than the ring
+@pytest.mark.parametrize("N,d,E,shared", [(64, 4096, 63, True), (1184, 328, 64, False), (1600, 1040, 50, True), (1600, 64, 33, False), (2300, 528, 17, True)])
+def test_gate_logits_do_not_depend_on_the_expert_tile(N, d, E, shared):
+    test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared)
+
+
 @pytest.mark.parametrize("N,K,P", [(1, 3, 4), (150, 7, 2), (1700, 6, 5), (40000, 4, 3), (525000, 1, 3), (263000, 2, 1),
                                    (176000, 3, 2)])
 def test_two_stage_dispatch_against_numpy(N, K, P):
