@@ -43,81 +43,69 @@ __global__ void pack_kernel(const T* __restrict__ W1, const T* __restrict__ W3, 
 }
 
 
-// Four consecutive elements as floats; `vec`: base pointers and strides are known to be aligned for one vector load.
-__device__ __forceinline__ float4 load4(const float* p, bool vec) {
-  if (vec) return *reinterpret_cast<const float4*>(p);
-  return make_float4(p[0], p[1], p[2], p[3]);
-}
-__device__ __forceinline__ float4 load4(const __nv_bfloat16* p, bool vec) {
-  if (vec) {
-    const uint2 u = *reinterpret_cast<const uint2*>(p);
-    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
-                       __uint_as_float(u.y & 0xFFFF0000u));
-  }
-  return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+// Four consecutive elements of a shared-memory tile as floats.
+__device__ __forceinline__ float4 tile4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 tile4(const __nv_bfloat16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xFFFF0000u));
 }
 
-// Operand tiles are [SK][W] floats.  The 4-wide column groups of row k are permuted by ^ ((k >> 2) & 7): a thread that
-// loaded four consecutive k of one row stores them down a column without bank conflicts, and four consecutive columns
-// still lie in 16 aligned bytes.
-template <int W>
-__device__ __forceinline__ int tile_at(int k, int m) {
-  return k * W + ((((m >> 2) ^ ((k >> 2) & 7)) & (W / 4 - 1)) << 2) + (m & 3);
-}
+constexpr int SPAN = 32;  // k-elements of a tile
 
-// A W x SK operand tile on its way from global memory to shared memory, held in registers while the previous tile is used.
-// Addresses are worked out once and advanced by a k-tile: the small problems are bound by instructions as much as by latency.
-template <typename T, int W, int SK, int SIMT_THREADS>
+// A tile of W rows (columns of the output) x SPAN k of one operand on its way to shared memory by cp.async, in the order in which
+// it lies in global memory: KM (k contiguous) as [W][SPAN] with rows padded against bank conflicts, else as [SPAN][W].
+// Addresses are worked out once and advanced: the small problems are bound by instructions as much as by latency.
+template <typename T, int W, bool KM, int THREADS>
 struct TileLoad {
-  static constexpr int PER = W * SK / 4 / SIMT_THREADS;  // four-element pieces per thread
-  static_assert(W * SK / 4 % SIMT_THREADS == 0, "every thread loads the same number of pieces");
-  float4 v[PER];
+  static constexpr int EPC = 16 / sizeof(T);                                    // elements per 16-byte piece
+  static constexpr int PITCH = KM ? SPAN + EPC : W;                             // elements per row of the tile
+  static constexpr int ELEMS = KM ? W * PITCH : SPAN * W;
+  static constexpr int PIECES = W * SPAN / EPC, PER = (PIECES + THREADS - 1) / THREADS;
   const T* src[PER];   // next piece; NULL where the tile has no such row
   int k_of[PER], at[PER];
   long long step;
-  int lane_step;       // distance of a piece's elements in the shared tile
-  // row(m): address of element (m, 0); element (m, k) lies k * sk further, and for sk != 1 rows lie next to each other
+  // row(m): address of element (m, 0); element (m, k) lies k * sk further, and without KM rows lie next to each other
   template <typename Row>
   __device__ __forceinline__ void init(Row row, long long sk, int m_left) {
-    step = SK * sk;
-    lane_step = sk == 1 ? W : 1;
+    step = SPAN * sk;
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-      const int x = threadIdx.x + i * SIMT_THREADS;
-      const int k = sk == 1 ? 4 * (x % (SK / 4)) : x / (W / 4), m = sk == 1 ? x / (SK / 4) : 4 * (x % (W / 4));
+      const int x = threadIdx.x + i * THREADS;
+      const int k = KM ? EPC * (x % (SPAN / EPC)) : x / (W / EPC), m = KM ? x / (SPAN / EPC) : EPC * (x % (W / EPC));
       k_of[i] = k;
-      at[i] = tile_at<W>(k, m);
-      src[i] = m < m_left ? row(m) + k * sk : nullptr;
+      at[i] = KM ? m * PITCH + k : k * W + m;
+      src[i] = (PIECES % THREADS == 0 || x < PIECES) && m < m_left ? row(m) + k * sk : nullptr;
     }
   }
-  __device__ __forceinline__ void load(int k_left, bool vec) {
-    if (vec) {
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (src[i] != nullptr && k_of[i] < k_left) v[i] = load4(src[i], true);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (src[i] != nullptr && k_of[i] < k_left) v[i] = load4(src[i], false);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-      if (src[i] != nullptr) src[i] += step;
-  }
-  __device__ __forceinline__ void store(float* tile) const {
+  // any: an aligned address that may be named where nothing is read
+  __device__ __forceinline__ void fetch(T* tile, int k_left, bool vec, const T* any) {
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-      if (lane_step == 1) {
-        *reinterpret_cast<float4*>(&tile[at[i]]) = v[i];
-      } else {  // the four k of a piece share a column group: W floats apart
-        tile[at[i]] = v[i].x;
-        tile[at[i] + W] = v[i].y;
-        tile[at[i] + 2 * W] = v[i].z;
-        tile[at[i] + 3 * W] = v[i].w;
+      if (PIECES % THREADS != 0 && (int)threadIdx.x + i * THREADS >= PIECES) continue;
+      const bool live = src[i] != nullptr && k_of[i] < k_left;
+      if (vec) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(tile + at[i])),
+                     "l"(live ? src[i] : any), "r"(live ? 16 : 0)
+                     : "memory");
+      } else {
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) tile[at[i] + j] = live ? src[i][j] : from_f32<T>(0.f);
+      }
+      if (src[i] != nullptr) src[i] += step;
+    }
+  }
+  // The four rows (columns of the output) that thread t of W / 4 has, and their elements k .. k + 3: v[row][k].
+  static __device__ __forceinline__ int row_of(int t, int i) { return KM ? t + (W / 4) * i : 4 * t + i; }
+  static __device__ __forceinline__ void read(const T* tile, int t, int k, float (&v)[4][4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 x = tile4(KM ? tile + row_of(t, i) * PITCH + k : tile + (k + i) * W + 4 * t);
+      const float e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (KM) v[i][j] = e[j];
+        else v[j][i] = e[j];
       }
     }
   }
@@ -128,26 +116,30 @@ struct TileLoad {
 // A block computes TM x TN outputs; (TM / 4)(TN / 4) threads hold a 4 x 4 share each.  A sum over k is kept as S partial sums,
 // part j over the j-th of S equal pieces of every SPAN consecutive k, added in part order at the end.  Groups of threads keep
 // a part each, or a thread keeps all: a result does not depend on the tile its batch was given, and is nearer to the
-// exact sum than one chain is.  The next k-tile is loaded into registers while the current one is used (two shared-memory
-// buffers, one barrier per tile).  The small configurations this serves are bound by latency: a chain of 16-deep tiles, each
-// waiting for its own loads, took 80 us for K = 256 where this takes 16.5 (1024 rows, 128 dual columns; weight gradients of
-// 375 rows 158 -> 28; whole fp32 training step of 1500 tokens 500 -> 190).  64 x 64 tiles where they fill the chip, else
-// 32-wide ones; the two SwiGLU products always take 32 x 32, since at 64 x 64 their parts are 128 registers of a thread and
-// one block per SM (forward of 4096 tokens of 512, top-4 of 8 experts of 512: 861 us with one chain per sum, 1018 with the
-// parts at 64 x 64, 980 so; 1250 before there were parts and prefetched tiles).
+// exact sum than one chain is.  STAGES - 1 tiles of both operands are on their way (cp.async) while one is used.  The small
+// configurations this serves are bound by latency and by the operands' way from shared memory (two 16-byte reads per 16 products;
+// 8 x 8 outputs per thread halve those, but leave too few warps: training step of 1500 tokens 159 us, so 222).  Tiles that went
+// through registers, one ahead, transposed on their way, took, in us before / after for whole passes: fp32 forward of 4096 tokens of 512,
+// top-4 of 8 x 512, 982 / 920, training step 2956 / 2716; bf16 off the tensor-core shapes (8192 tokens of 264) 419 / 316 and 1443 / 1091;
+// the expert calls of 512 tokens alone 21.5 / 22.1 and 46.7 / 49.1.
+// 64 x 64 tiles where they fill the chip, else 32-wide ones; the two SwiGLU products always take 32 x 32, since at 64 x 64 their
+// parts are 128 registers of a thread and one block per SM.
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
-constexpr int SPAN = 32;
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int S, int SIMT_THREADS>
+template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int STAGES, int SIMT_THREADS>
 __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   chain_begin();
+  using LA = TileLoad<T, TM, AK, SIMT_THREADS>;
+  using LB = TileLoad<T, TN, BN, SIMT_THREADS>;
   constexpr int GROUP = (TM / 4) * (TN / 4), G = SIMT_THREADS / GROUP;  // threads per group, groups
-  constexpr int PART = SPAN / S, PARTS = SK / PART / G, O = S / G;      // length of a part; a thread's parts per k-tile, in all
+  constexpr int PART = SPAN / S, O = S / G;                             // length of a part; a thread's parts per tile
   static_assert(!DUAL || G > 1, "two products keep their parts in groups");
-  static_assert(SPAN % SK == 0 && PARTS * PART * G == SK && (G == 1 || O == 1), "a group of threads keeps one part, or a thread all of them");
+  static_assert(PART % 4 == 0 && (G == 1 || O == 1), "a group of threads keeps one part, or a thread all of them");
   constexpr int MR = G == 1 ? 4 : TM * TN / (4 * SIMT_THREADS);         // output rows a thread finishes, four columns each
-  constexpr int TILES = 2 * SK * (TM + TN * (DUAL ? 2 : 1)), RED = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4);
-  __shared__ __align__(16) float smem[TILES > RED ? TILES : RED];
+  constexpr int STAGE = LA::ELEMS + (DUAL ? 2 : 1) * LB::ELEMS;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  T* const tiles = reinterpret_cast<T*>(smem_raw);
+  float* const smem = reinterpret_cast<float*>(smem_raw);
   __shared__ float sred[TM][TN / 4 + 1];  // per-row partial dots of the SwiGLU backward, one column per thread column
   const int tid = threadIdx.x, lane = tid & 31;
   int grp, m0, M, Kd;
@@ -194,72 +186,79 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   const int grp_k = tid / GROUP, tg = tid % GROUP;
   const int tx = tg % (TN / 4), ty = tg / (TN / 4);
   float sum[O][4][4] = {}, sum2[DUAL ? O : 1][4][4] = {};
-  TileLoad<T, TM, SK, SIMT_THREADS> la;
-  TileLoad<T, TN, SK, SIMT_THREADS> lb, lb2;
+  LA la;
+  LB lb, lb2;
   la.init(rowA, g.sak, M - m0);
   lb.init(rowB, g.sbk, g.Ndim - n0);
   if (DUAL) lb2.init(rowB2, g.sbk, g.Ndim - n0);
-  auto fetch = [&](int k0) {
-    la.load(Kd - k0, vec);
-    lb.load(Kd - k0, vec);
-    if (DUAL) lb2.load(Kd - k0, vec);
+  const int n_tiles = (Kd + SPAN - 1) / SPAN;
+  auto fetch = [&](int t) {
+    if (t < n_tiles) {
+      T* sa = tiles + t % STAGES * STAGE;
+      la.fetch(sa, Kd - t * SPAN, vec, (const T*)g.A);
+      lb.fetch(sa + LA::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
+      if (DUAL) lb2.fetch(sa + LA::ELEMS + LB::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  constexpr int BUF = SK * (TM + TN * (DUAL ? 2 : 1));
-  fetch(0);
-  for (int k0 = 0, buf = 0; k0 < Kd; k0 += SPAN) {
 #pragma unroll
-    for (int h = 0; h < SPAN / SK; ++h, buf ^= 1) {
-      const int kt = k0 + h * SK;
-      if (kt >= Kd) break;
-      float* sa = smem + buf * BUF;
-      float* sb = sa + SK * TM;
-      float* sb2 = sb + SK * TN;
-      la.store(sa);
-      lb.store(sb);
-      if (DUAL) lb2.store(sb2);
-      __syncthreads();
-      if (kt + SK < Kd) fetch(kt + SK);
+  for (int t = 0; t < STAGES - 1; ++t) fetch(t);
+  for (int t = 0; t < n_tiles; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();  // tile t is there, and the one before it is no longer read
+    fetch(t + STAGES - 1);
+    const T* sa = tiles + t % STAGES * STAGE;
+    const T* sb = sa + LA::ELEMS;
+    const T* sb2 = sb + LB::ELEMS;
 #pragma unroll
-      for (int q = 0; q < PARTS; ++q) {
-        float(&acc)[4][4] = sum[h * PARTS + q];
-        float(&acc2)[4][4] = sum2[DUAL ? h * PARTS + q : 0];
-#pragma unroll 8  // a kernel this short is bound by instruction fetch if the body is longer
-        for (int kk = 0; kk < PART; ++kk) {
-          const int k = (grp_k * PARTS + q) * PART + kk;
-          const float4 av = *reinterpret_cast<const float4*>(&sa[tile_at<TM>(k, 4 * ty)]);
-          const float4 bv = *reinterpret_cast<const float4*>(&sb[tile_at<TN>(k, 4 * tx)]);
-          const float ar[4] = {av.x, av.y, av.z, av.w}, br[4] = {bv.x, bv.y, bv.z, bv.w};
+    for (int q = 0; q < O; ++q) {
+#pragma unroll 4
+      for (int k4 = 0; k4 < PART; k4 += 4) {
+        const int k = (G == 1 ? q : grp_k) * PART + k4;
+        float av[4][4], bv[4][4];
+        LA::read(sa, ty, k, av);
+        LB::read(sb, tx, k, bv);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
-          if (DUAL) {
-            const float4 cv = *reinterpret_cast<const float4*>(&sb2[tile_at<TN>(k, 4 * tx)]);
-            const float cr[4] = {cv.x, cv.y, cv.z, cv.w};
+            for (int j = 0; j < 4; ++j) sum[q][i][j] = fmaf(av[i][kk], bv[j][kk], sum[q][i][j]);
+        if (DUAL) {
+          LB::read(sb2, tx, k, bv);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(ar[i], cr[j], acc2[i][j]);
-          }
+              for (int j = 0; j < 4; ++j) sum2[DUAL ? q : 0][i][j] = fmaf(av[i][kk], bv[j][kk], sum2[DUAL ? q : 0][i][j]);
         }
       }
     }
   }
-  // this thread's outputs: rows m_of(i), columns nc .. nc + 3
-  const int nc = n0 + 4 * (G == 1 ? tx : tid % (TN / 4));
-  auto m_of = [&](int i) { return G == 1 ? 4 * ty + i : tid / (TN / 4) + i * (SIMT_THREADS / (TN / 4)); };
+  // this thread's outputs: rows m_of(i), columns n_of(j) of the tile
+  auto m_of = [&](int i) { return G == 1 ? LA::row_of(ty, i) : tid / (TN / 4) + i * (SIMT_THREADS / (TN / 4)); };
+  auto n_of = [&](int j) { return G == 1 ? LB::row_of(tx, j) : 4 * (tid % (TN / 4)) + j; };
   float(&acc)[4][4] = sum[0];
   float(&acc2)[4][4] = sum2[0];
   // the parts added in part order: a thread's own, or all groups' through shared memory
   constexpr int P = TN + 4;
   if (G > 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      *reinterpret_cast<float4*>(&smem[(grp_k * TM + 4 * ty + i) * P + 4 * tx]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      if (DUAL)
-        *reinterpret_cast<float4*>(&smem[((G + grp_k) * TM + 4 * ty + i) * P + 4 * tx]) =
-            make_float4(acc2[i][0], acc2[i][1], acc2[i][2], acc2[i][3]);
+      float* row = &smem[(grp_k * TM + LA::row_of(ty, i)) * P];
+      if constexpr (BN) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) row[LB::row_of(tx, j)] = acc[i][j];
+      } else {  // four columns in a row
+        *reinterpret_cast<float4*>(row + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      }
+      if (DUAL) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) row[G * TM * P + LB::row_of(tx, j)] = acc2[i][j];
+      }
     }
     __syncthreads();
   }
@@ -271,8 +270,8 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
         float v = 0.f, v2 = 0.f;
 #pragma unroll
         for (int q = 0; q < S; ++q) {
-          v += G == 1 ? sum[q < O ? q : 0][i][j] : smem[(q * TM + m_of(i)) * P + nc - n0 + j];
-          if (DUAL) v2 += smem[((G + q) * TM + m_of(i)) * P + nc - n0 + j];
+          v += G == 1 ? sum[q < O ? q : 0][i][j] : smem[(q * TM + m_of(i)) * P + n_of(j)];
+          if (DUAL) v2 += smem[((G + q) * TM + m_of(i)) * P + n_of(j)];
         }
         acc[i][j] = v;
         if (DUAL) acc2[i][j] = v2;
@@ -285,7 +284,8 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   for (int i = 0; i < MR; ++i) {
     const int lm = m_of(i), m = m0 + lm;
     float qrow = 0.f;
-    if (want_q) sred[lm][(nc - n0) / 4] = 0.f;
+    const int col4 = G == 1 ? tx : tid % (TN / 4);
+    if (want_q) sred[lm][col4] = 0.f;
     if (m >= M) continue;
     float sc = 1.f;  // per-row scale of H (SwiGLU forms)
     if (g.scale_kind != 0 && g.row_scale != nullptr) {
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = nc + j;
+      const int n = n0 + n_of(j);
       if (n >= g.Ndim) continue;
       float v = acc[i][j];
       if (DUAL) {
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
         if (want_q) qrow = fmaf(v, to_f32(((const T*)g.aux2)[(long long)(r0 + m) * g.I + n]), qrow);
       }
     }
-    if (want_q) sred[lm][(nc - n0) / 4] = qrow;
+    if (want_q) sred[lm][col4] = qrow;
   }
   if (want_q) {  // (uniform across the block) row dots <dH_r, H_r> over this block's 64 columns, in column order
     __syncthreads();
@@ -340,23 +340,29 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   }
 }
 
-template <typename T, typename TC, int TM, int TN, int SK, bool DUAL, int S, int SIMT_THREADS = 256>
+template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int SIMT_THREADS = 256>
 static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
-  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, SK, DUAL, S, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z), SIMT_THREADS, 0, s, g));
+  constexpr int STAGES = 4, G = SIMT_THREADS / ((TM / 4) * (TN / 4));
+  constexpr int tiles = STAGES * (int)sizeof(T) * (TileLoad<T, TM, AK, SIMT_THREADS>::ELEMS + (DUAL ? 2 : 1) * TileLoad<T, TN, BN, SIMT_THREADS>::ELEMS);
+  constexpr int red = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4) * 4, smem = tiles > red ? tiles : red;
+  static int done[64] = {};
+  if (const int rc = allow_smem(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, SIMT_THREADS>, done, smem)) return rc;
+  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z),
+                          SIMT_THREADS, smem, s, g));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
 
-// Whether every group of four elements the kernel loads lies on a four-element boundary.
+// Whether every 16-byte piece the kernel loads lies on a 16-byte boundary.
 template <typename T>
 static int simt_vec(const SimtGemm& g) {
+  constexpr int EPC = 16 / sizeof(T);
   const uintptr_t bits = (uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last;
-  return (bits & (4 * sizeof(T) - 1)) == 0 && (g.sak == 1 ? g.sam : g.sak) % 4 == 0 &&
-         (g.sbk == 1 ? g.sbn : g.sbk) % 4 == 0 && g.sB % 4 == 0;
+  return (bits & 15u) == 0 && (g.sak == 1 ? g.sam : g.sak) % EPC == 0 && (g.sbk == 1 ? g.sbn : g.sbk) % EPC == 0 && g.sB % EPC == 0;
 }
 
-// max_m: rows (SIMT_ROWS: of all groups together) or Mdim.
-template <typename T, typename TC = T>
+// max_m: rows (SIMT_ROWS: of all groups together) or Mdim.  AK / BN: the contraction index is the contiguous one of A / of B.
+template <bool AK, bool BN, typename T, typename TC = T>
 int simt_launch(SimtGemm g, int n_groups, int64_t max_m, cudaStream_t s) {
   if (n_groups == 0 || max_m == 0 || g.Ndim == 0) return C2R_OK;
   g.n_groups = n_groups;
@@ -368,12 +374,16 @@ int simt_launch(SimtGemm g, int n_groups, int64_t max_m, cudaStream_t s) {
   const int64_t blocks64 = (int64_t)((max_m + 63) / 64) * ((g.Ndim + 63) / 64) * z;
   const bool large = blocks64 >= 2 * 148;
   // four partial sums; two in the backward of SwiGLU, whose partial row dots cover 64 columns each
-  if (g.epi == SIMT_EPI_SWIGLU_FWD) return simt_launch_tile<T, TC, 32, 32, 32, true, 4>(g, m_tiles(32), z, s);
-  if (g.epi == SIMT_EPI_SWIGLU_BWD)
-    return large ? simt_launch_tile<T, TC, 64, 64, 16, false, 2>(g, m_tiles(64), z, s)
-                 : simt_launch_tile<T, TC, 32, 64, 32, false, 2>(g, m_tiles(32), z, s);
-  return large ? simt_launch_tile<T, TC, 64, 64, 16, false, 4>(g, m_tiles(64), z, s)
-               : simt_launch_tile<T, TC, 32, 32, 32, false, 4>(g, m_tiles(32), z, s);
+  if constexpr (AK && BN) {
+    if (g.epi == SIMT_EPI_SWIGLU_FWD) return simt_launch_tile<T, TC, 32, 32, true, 4, AK, BN>(g, m_tiles(32), z, s);
+  }
+  if constexpr (AK && !BN) {
+    if (g.epi == SIMT_EPI_SWIGLU_BWD)
+      return large ? simt_launch_tile<T, TC, 64, 64, false, 2, AK, BN>(g, m_tiles(64), z, s)
+                   : simt_launch_tile<T, TC, 32, 64, false, 2, AK, BN>(g, m_tiles(32), z, s);
+  }
+  return large ? simt_launch_tile<T, TC, 64, 64, false, 4, AK, BN>(g, m_tiles(64), z, s)
+               : simt_launch_tile<T, TC, 32, 32, false, 4, AK, BN>(g, m_tiles(32), z, s);
 }
 
 // Gate logits (Eq. 1) of fp32 layers: L = X Wg^T and, as one more row of the other operand, z = X wsg.  Every logit is one chain of
@@ -487,7 +497,7 @@ static int gate_simt_launch(const c2r_config* cfg, const __nv_bfloat16* X, const
   g.Mdim = cfg->N; g.Ndim = cfg->E + (wsg ? 1 : 0); g.Kdim = cfg->d;
   g.n_groups = 1;
   g.vec = simt_vec<__nv_bfloat16>(g);
-  return simt_launch_tile<__nv_bfloat16, float, 32, 32, 32, false, 1, 64>(g, (cfg->N + 31) / 32, 1, s);
+  return simt_launch_tile<__nv_bfloat16, float, 32, 32, false, 1, true, true, 64>(g, (cfg->N + 31) / 32, 1, s);
 }
 
 template <typename T>
@@ -508,14 +518,14 @@ int simt_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) 
   g.row_scale = a.row_scale; g.scale_kind = a.row_scale ? a.scale_kind : 0;
   g.A = a.Xp; g.sam = d; g.sak = 1; g.B = a.W13p; g.sbn = d; g.sbk = 1; g.sB = (long long)2 * I * d;
   g.C = a.AB; g.ldc = 2 * I; g.Ndim = I; g.Kdim = d;
-  int rc = simt_launch<T>(g, a.nE, max_m, s);
+  int rc = simt_launch<true, true, T>(g, a.nE, max_m, s);
   if (rc) return rc;
   g.epi = SIMT_EPI_STORE; g.aux_out = nullptr; g.row_scale = nullptr; g.scale_kind = 0;
   // Yp = H W2^T  (fp32 partial result)
   g.A = a.H; g.sam = I; g.sak = 1; g.B = a.W2; g.sbn = I; g.sbk = 1; g.sB = (long long)d * I;
   g.C = a.Yp; g.ldc = d; g.Ndim = d; g.Kdim = I;
   g.token_acc = a.token_acc; g.slot_of_row = a.slot_of_row; g.slots_per_token = cfg->K;
-  return simt_launch<T, float>(g, a.nE, max_m, s);
+  return simt_launch<true, true, T, float>(g, a.nE, max_m, s);
 }
 
 template <typename T>
@@ -529,26 +539,26 @@ int simt_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) 
   g.row_scale = a.row_scale; g.scale_kind = a.row_scale ? a.scale_kind : 0;
   g.A = a.dYp; g.sam = d; g.sak = 1; g.B = a.W2; g.sbn = 1; g.sbk = I; g.sB = (long long)d * I;
   g.C = a.dAB; g.ldc = 2 * I; g.Ndim = I; g.Kdim = d;
-  int rc = simt_launch<T>(g, nE, max_m, s);
+  int rc = simt_launch<true, false, T>(g, nE, max_m, s);
   if (rc) return rc;
   // dXp = dAB W13p  (fp32 partial result)
   g.epi = SIMT_EPI_STORE; g.aux = nullptr; g.aux2 = nullptr; g.qpart = nullptr; g.row_scale = nullptr; g.scale_kind = 0;
   g.A = a.dAB; g.sam = 2 * I; g.sak = 1; g.B = a.W13p; g.sbn = 1; g.sbk = d; g.sB = (long long)2 * I * d;
   g.C = a.dXp; g.ldc = d; g.Ndim = d; g.Kdim = 2 * I;
   g.token_acc = a.token_acc; g.slot_of_row = a.slot_of_row; g.slots_per_token = cfg->K;
-  rc = simt_launch<T, float>(g, nE, max_m, s);
+  rc = simt_launch<true, false, T, float>(g, nE, max_m, s);
   if (rc) return rc;
   g.token_acc = nullptr;
   // dW2_e = dYp_e^T H_e   [d, I]
   g.mode = SIMT_WGRAD; g.accumulate = a.accumulate;
   g.A = a.dYp; g.sam = 1; g.sak = d; g.B = a.H; g.sbn = 1; g.sbk = I;
   g.C = a.dW2; g.ldc = I; g.sC = (long long)d * I; g.Mdim = d; g.Ndim = I;
-  rc = simt_launch<T>(g, nE, d, s);
+  rc = simt_launch<false, false, T>(g, nE, d, s);
   if (rc) return rc;
   // dW13p_e = dAB_e^T Xp_e   [2I, d]
   g.A = a.dAB; g.sam = 1; g.sak = 2 * I; g.B = a.Xp; g.sbn = 1; g.sbk = d;
   g.C = a.dW13p; g.ldc = d; g.sC = (long long)2 * I * d; g.Mdim = 2 * I; g.Ndim = d;
-  return simt_launch<T>(g, nE, 2 * I, s);
+  return simt_launch<false, false, T>(g, nE, 2 * I, s);
 }
 
 template int simt_swiglu_fwd<float>(const c2r_config*, const SwigluCall&, cudaStream_t);

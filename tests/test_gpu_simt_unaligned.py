@@ -1,0 +1,35 @@
+"""CUDA-core expert GEMMs on arrays that start off a 16-byte boundary (element-wise loads): the same bits as on aligned ones."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+# contractions with a remainder beyond a 32-wide tile and shorter than one; tiles of 32 and (last case) of 64; an empty expert
+@pytest.mark.parametrize("bf16,offset", [(False, 1), (False, 2), (True, 1), (True, 4)])
+@pytest.mark.parametrize("counts,d,I", [([37, 0, 5, 64], 40, 48), ([1, 2], 8, 16), ([700, 650, 800], 520, 144)])
+def test_unaligned_arrays(counts, d, I, bf16, offset):
+    from paper_2504_01337_b200 import binding as B
+    E, R = len(counts), sum(counts)
+    dt = torch.bfloat16 if bf16 else torch.float32
+    cfg = B.make_config(R, d, E, I, 1, 0, 1, 0, B.BF16 if bf16 else B.F32, 1)  # several experts, rows not aligned to 128: off the tensor cores
+    g = torch.Generator(device="cuda").manual_seed(d)
+    cnt = torch.tensor(counts, dtype=torch.int32, device="cuda")
+    off = torch.tensor([sum(counts[:i]) for i in range(E + 1)], dtype=torch.int32, device="cuda")
+    shapes = dict(X=(R, d), W13=(E, 2 * I, d), W2=(E, d, I), dY=(R, d))
+    flat = {k: torch.empty(torch.Size(s).numel(), dtype=dt, device="cuda").normal_(0, 0.3, generator=g) for k, s in shapes.items()}
+
+    def run(shift):
+        t = {}
+        for k, s in shapes.items():
+            a = torch.zeros(flat[k].numel() + 16, dtype=dt, device="cuda")
+            a[shift:shift + flat[k].numel()] = flat[k]
+            t[k] = a[shift:shift + flat[k].numel()].view(s)
+        AB, H, Yp = torch.empty((R, 2 * I), dtype=dt, device="cuda"), torch.empty((R, I), dtype=dt, device="cuda"), torch.empty((R, d), device="cuda")
+        dAB, dXp, dW13, dW2 = torch.empty_like(AB), torch.empty_like(Yp), torch.empty_like(t["W13"]), torch.empty_like(t["W2"])
+        B.grouped_swiglu_fwd(cfg, E, I, R, t["X"], cnt, off, t["W13"], t["W2"], AB, H, Yp)
+        B.grouped_swiglu_bwd(cfg, E, I, R, t["X"], cnt, off, t["W13"], t["W2"], AB, H, t["dY"], dAB, dXp, dW13, dW2)
+        torch.cuda.synchronize()
+        return AB, H, Yp, dAB, dXp, dW13, dW2
+
+    assert all(torch.isfinite(a).all() and torch.equal(a, b) for a, b in zip(run(0), run(offset)))
