@@ -91,9 +91,7 @@ static int swiglu_fwd_dispatch(const c2r_config* cfg, const SwigluCall& a, cudaS
   if (a.R == 0) return C2R_OK;
   if (cfg->dtype == C2R_F32) return simt_swiglu_fwd<float>(cfg, a, s);
   if (tc_supported(cfg, a.nE, a.I, a.R))
-    return a.nE > 1 && skinny_supported(cfg, a, SKINNY_ROWS) ? skinny_swiglu_fwd(cfg, &a, 1, s)
-           : ragged_supported(cfg, a)                        ? ragged_swiglu_fwd(cfg, a, s)
-                                                             : tc_swiglu_fwd(cfg, a, s);
+    return skinny_supported(cfg, a, SKINNY_ROWS) ? skinny_swiglu_fwd(cfg, &a, 1, s) : tc_swiglu_fwd(cfg, a, s);
   return simt_swiglu_fwd<__nv_bfloat16>(cfg, a, s);
 }
 

@@ -85,28 +85,18 @@ enum { TC_EPI_SWIGLU_FWD = 0, TC_EPI_F32 = 1, TC_EPI_SWIGLU_BWD = 2, TC_EPI_WGRA
 bool tc_supported(const c2r_config* cfg, int nE, int I, int64_t R);
 int tc_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
 int tc_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
-// Forward calls that keep nothing for a backward pass (bf16) choose among three kernels by the rows the host can expect: the slots
-// spread evenly over the experts, or all rows of a single group.  us per call of both products:
-//  - weight streaming (128 weight rows of one SM against 16 or 32 tokens) up to 20 rows per expert.  Streaming / tokens as N of
-//    pair MMAs: 60 experts of 1408, d 2048: 169 / 175 at 16 rows, 199 / 173 at 24; 16 of 688, d 4096: 68.6 / 65.1 at 16,
-//    78.8 / 66.2 at 24; 8 of 512, d 1024: 13.5 / 15.8 at 8, 15.7 / 16.0 at 20, 17.8 / 16.2 at 24; 33 of 1024, d 1024: 47.2 / 49.1 at
-//    20, 52.2 / 47.7 at 24.  A single group is always worse off (d 2048, 4 rows: 22.0 / 16.5 at I = 256, 47.7 / 33.7 at 5632), but
-//    may ride along with the routed experts, where it costs no launch of its own, with up to 128 rows;
-//  - tokens as N of pair MMAs up to 768 rows per expert and 1024 of a single group.  Pair tiles of 256 tokens / this: 60 experts of
-//    1408, d 2048: 281 / 244 at 150 rows, 405 / 313 at 273, 641 / 595 at 600, 1020 / 970 at 1092 with other shapes losing 5 %
-//    (16 of 688, d 4096: 195 / 182 at 512, 240 / 237 at 700, 338 / 350 at 1024; 24 of 400, d 768: 76 / 78 at 1000); single group,
-//    d 2048: I = 5632 60 / 49 at 512 rows, 75 / 70 at 1024, 114 / 116 at 2048; I = 1024 30 / 35 at 2048.  It takes skewed counts well
-//    (4 experts of 300 rows and 20 of one: streaming 136, pair tiles 88 by the mean, this 83);
-//  - pair tiles of 256 tokens beyond.
-constexpr int SKINNY_ROWS = 20, SKINNY_ROWS_PAIRED = 128, RAGGED_ROWS = 768, RAGGED_ROWS_SINGLE = 1024;
-// Rows an expert is expected to have, as far as the host knows: all of R for a single group, else the batch's slots
-// spread evenly.  Only a hint: the kernels take any counts.
-int64_t expected_rows(const c2r_config* cfg, const SwigluCall& a);
+// Weight-streaming forward for a handful of rows per expert (bf16, nothing kept for a backward pass).
+// The line: with the routed experts' rows spread evenly, up to 48 rows per expert (Qwen-MoE shape, us, pair tiles against
+// this: 237 / 183 at 4 rows, 238 / 202 at 34, 238 / 226 at 68; LLaMA-MoE shape 105 / 95 at 32, 105 / 107 at 64; 12 experts of
+// 512: 36 / 34 at 43, 36 / 44 at 85).  A dense group that rides along with the routed ones may have 128 rows: the
+// launches it saves and the SMs it fills are worth more than its own loss (Qwen shape, 128 tokens, whole forward 382 / 319).
+// The host knows the mean only.  Where routing is skewed so far that most rows meet in a few experts, their token chunks
+// read the weights again and pair tiles would be the faster ones from 64 tokens on (Qwen shape, whole pass call by call,
+// pair tiles / this: 108 / 79 at 16 tokens, 120 / 122 at 64, 137 / 165 at 256, 174 / 224 at 720).
+constexpr int SKINNY_ROWS = 48, SKINNY_ROWS_PAIRED = 128;
 bool skinny_supported(const c2r_config* cfg, const SwigluCall& a, int max_rows);
-// The routed experts alone or, in the same two launches, with the shared expert.
+// One or two such calls in one launch per product (the routed experts and the shared expert).
 int skinny_swiglu_fwd(const c2r_config* cfg, const SwigluCall* calls, int n, cudaStream_t s);
-bool ragged_supported(const c2r_config* cfg, const SwigluCall& a);
-int ragged_swiglu_fwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s);
 // Rows of the partial-dot buffer the backward call writes for this shape (depends on which kernel serves it).
 int swiglu_qparts(const c2r_config* cfg, int nE, int I, int64_t R);
 

@@ -3,7 +3,7 @@
 // With few rows the product is bound by reading every weight once: 138 MB for one token of the Qwen-MoE-shaped layer
 // (d 2048, 60 experts of 1408, top-4, shared 5632), 1.1 GB for 64.  The 256 x 256 pair tiles of tc_gemm_kernel are the
 // wrong shape for that: one token's output is 8 to 44 such tiles, so most SMs stay idle.  Here the weights are the M
-// operand (128 accumulator lanes) and the tokens its N of 16 or 32 columns.  A unit of work is a slice of an expert's
+// operand (128 accumulator lanes) and the tokens its N of 16..128 columns.  A unit of work is a slice of an expert's
 // weight rows (CH gate and CH up rows, or 2 CH output channels) against one chunk of the expert's tokens over the
 // whole contraction; CTAs are persistent and walk the units, the TMA ring (about 190 KB) runs across unit boundaries, so
 // an SM always has its whole ring of weight bytes in flight.  A stage is several k-blocks that one TMA instruction
@@ -320,7 +320,9 @@ skinny_kernel(const __grid_constant__ SkinnyMaps maps0, const __grid_constant__ 
   }
 }
 
-int64_t expected_rows(const c2r_config* cfg, const SwigluCall& a) {
+// Rows an expert is expected to have, as far as the host knows: all of R for a single group, else the batch's slots
+// spread evenly.  Only a hint: the kernel takes any counts.
+static int64_t expected_rows(const c2r_config* cfg, const SwigluCall& a) {
   return a.nE == 1 ? a.R : ((int64_t)cfg->N * cfg->K + a.nE - 1) / a.nE;
 }
 
@@ -356,11 +358,12 @@ static int skinny_launch(const c2r_config* cfg, const SwigluCall* calls, int n, 
   const int wr = up ? p.ch : 2 * p.ch, parts = up ? 2 : 1;
   int nb_max = 16;
   for (int i = 0; i < n; ++i) {
-    // Chunks of half as many tokens again as expected: most experts fit one, and few columns are empty.  All stages have the
-    // size of the larger problem's, so the shared expert's tokens come in chunks of 32 at most, whose weights the later
-    // chunks find in the L2 (64 tokens of the Qwen shape 235 us with one chunk of 64, 219 with two of 32; 128 tokens 263 / 247).
+    // Chunks of half as many tokens again as expected: most experts fit one, and few columns are empty.  In a shared launch
+    // all stages have the size of the larger problem's, so the shared expert's tokens come in chunks of 32 at most, whose weights
+    // the later chunks find in the L2 (64 tokens of the Qwen shape 235 us with one chunk of 64, 219 with two of 32; 128
+    // tokens 263 / 247).
     const int64_t rows = expected_rows(cfg, calls[i]), want = calls[i].nE == 1 ? rows : rows + rows / 2;
-    for (p.pr[i].nb = 16; p.pr[i].nb < want && p.pr[i].nb < 32; p.pr[i].nb <<= 1) {}
+    for (p.pr[i].nb = 16; p.pr[i].nb < want && p.pr[i].nb < (n > 1 ? 32 : 128); p.pr[i].nb <<= 1) {}
     if (p.pr[i].nb > nb_max) nb_max = p.pr[i].nb;
   }
   const int kb_bytes = (parts * wr + nb_max) * BK * 2;
