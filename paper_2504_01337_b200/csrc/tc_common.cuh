@@ -11,7 +11,11 @@ namespace c2r {
 constexpr int BM = 128;
 constexpr int BK = 64;          // 64 bf16 = one 128-byte swizzle row
 constexpr int UMMA_K = 16;
-constexpr uint32_t WAIT_LIMIT = 1u << 24;         // try_wait polls before a wait gives up
+// try_wait polls before a wait gives up.  A poll of a barrier that is not ready comes back after 4.06 us (16 polls 63.7 us), so
+// this is about a second: a thousand times the longest wait of a working kernel (a contraction of a few thousand k-blocks),
+// and little enough that a stuck launch is reported and not taken for a hang (2^24 polls were 68 s).
+constexpr uint32_t WAIT_LIMIT = 1u << 18;
+static_assert(WAIT_LIMIT * 4.06e-6 < 2.0, "a wait that gives up does so within two seconds");
 
 // ---- PTX wrappers ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
