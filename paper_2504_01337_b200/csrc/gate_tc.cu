@@ -10,11 +10,14 @@
 //
 // Few tokens are few tiles, and a CTA that streams 128 tokens alone is slow: a tile then has 64 or 32 tokens (the MMA still
 // computes 128 rows, the rest is whatever the stage holds and is not stored), and where SMs are left over the experts are
-// split into tiles of 32 or 16: a stage is then as small as 8 KB and nearly a whole contraction of 2048 is in flight at once.  A split
+// split into tiles of 32 or 16: a k-block is then as small as 6 KB, and a whole contraction of 2048 is in flight at once.  A split
 // of the contraction over a cluster would add a token's products in another order, and logits that differ in their last bits
 // route near-ties to other experts; every logit here is the same sum, bit for bit, in whatever tile.
-// Where a stage is small it holds up to four k-blocks, brought by one instruction per operand (a k-block at a time took 175 ns of the
+// Where a k-block is small a stage holds up to four, brought by one instruction per operand (a k-block at a time took 175 ns of the
 // issuing thread, however many were in flight).
+// Whole tiles (128 tokens, all experts: more than 64 tokens for every SM) are bound by the memory and by the two issuing threads, so
+// they have instances with everything known at compile time and plain maps (us a call, in the general form / so: 19000 tokens of 4096
+// and 24 experts 40.0 / 37.0, 20000 of 2048 and 60 23.3 / 21.8, 25000 of 1024 and 48 15.0 / 13.8, 65536 of 512 and 12 15.5 / 14.1).
 // (us by events after an L2 flush, all experts in a tile and a k-block per stage / this: 14.3 / 11.3 for 1 to 64 tokens of d = 2048 and
 // 60 experts, 19.5 / 17.4 for 1021 and 24.6 / 23.4 for 8192 of d = 4096 and 16; 16384 and more take 128-token tiles as before.)
 #include "gemm.h"
@@ -22,7 +25,7 @@
 
 namespace c2r {
 
-constexpr int GT_RING = 208 * 1024;        // bytes of operands in flight: 8 stages of a full tile, 26 of the smallest
+constexpr int GT_RING = 208 * 1024;        // bytes of operands in flight: 8 to 11 stages of a whole tile; 4 to 8 of four k-blocks, or more of fewer, else
 constexpr int GT_MAX_STAGES = 32;
 constexpr int GT_S_BYTES = 16 * BK * 2;    // the shared gate's block, 2 KB
 constexpr int GT_THREADS = 192;
@@ -33,9 +36,14 @@ struct GateMaps {
   CUtensorMap x, w, s, x_tail, w_tail, s_tail;
 };
 
+// TW > 0 (whole tiles): 128 tokens x all E <= TW experts, a k-block per stage, plain maps (the *_tail ones); tm, tw, ks are not read.
+// S: with the shared gate's block in every stage.  TW = 0: everything as the arguments say.
+template <int TW, bool S>
 __global__ void __launch_bounds__(GT_THREADS, 1)
 gate_tc_kernel(const __grid_constant__ GateMaps maps, float* __restrict__ L, float* __restrict__ z, int N, int d,
-               int E, int has_shared, int tm, int tw, int ks, int32_t* __restrict__ status) {
+               int E, int has_shared, int tm_, int tw_, int ks_, int32_t* __restrict__ status) {
+  constexpr bool WHOLE = TW > 0;
+  const int tm = WHOLE ? BM : tm_, tw = WHOLE ? TW : tw_, ks = WHOLE ? 1 : ks_;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ uint64_t bars[2 * GT_MAX_STAGES + 4];
@@ -66,9 +74,9 @@ gate_tc_kernel(const __grid_constant__ GateMaps maps, float* __restrict__ L, flo
   volatile int* abort_flag = &s_abort;
 
   // tiles of tm tokens x tw experts; the shared gate rides along with all experts, or is a tile of its own where they are split
-  const bool with_s = has_shared && E <= tw;
-  const int e_parts = (E + tw - 1) / tw, parts = e_parts + (has_shared && !with_s), tiles = (N + tm - 1) / tm * parts;
-  const int kfull = d / BK, slabs = (kfull + ks - 1) / ks, steps = slabs + (d % BK != 0);
+  const bool with_s = WHOLE ? S : has_shared && E <= tw;
+  const int e_parts = WHOLE ? 1 : (E + tw - 1) / tw, parts = WHOLE ? 1 : e_parts + (has_shared && !with_s), tiles = (N + tm - 1) / tm * parts;
+  const int kfull = d / BK, slabs = WHOLE ? (d + BK - 1) / BK : (kfull + ks - 1) / ks, steps = WHOLE ? slabs : slabs + (d % BK != 0);
   // a stage holds ks k-blocks of X, then ks of Wg, each followed by wsg's if that rides along
   const uint32_t x_kb = tm * BK * 2, w_kb = tw * BK * 2 + (with_s ? GT_S_BYTES : 0), stage_bytes = ks * (x_kb + w_kb);
   const int stages = min(GT_MAX_STAGES, (int)(GT_RING / stage_bytes));
@@ -85,7 +93,12 @@ gate_tc_kernel(const __grid_constant__ GateMaps maps, float* __restrict__ L, flo
         const uint32_t fb = full0 + 8 * stage;
         const uint32_t sx = smem_base + stage * stage_bytes, sw = sx + ks * x_kb;
         if (elect_one()) {
-          if (j < slabs) {
+          if (WHOLE) {
+            mbar_expect_tx(fb, stage_bytes);
+            tma_load_2d(sx, &maps.x_tail, fb, j * BK, row0);
+            tma_load_2d(sw, &maps.w_tail, fb, j * BK, 0);
+            if (S) tma_load_2d(sw + tw * BK * 2, &maps.s_tail, fb, j * BK, 0);
+          } else if (j < slabs) {
             mbar_expect_tx(fb, stage_bytes);
             tma_load_4d(sx, &maps.x, fb, 0, row0, j * ks, 0);
             if (with_s) {
@@ -123,7 +136,7 @@ gate_tc_kernel(const __grid_constant__ GateMaps maps, float* __restrict__ L, flo
         if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * stage, phase, abort_flag))) { ok = false; break; }
         tc_fence_after();
         uint32_t sx = smem_base + stage * stage_bytes, sw = sx + ks * x_kb;
-        const int nk = j < slabs ? min(ks, kfull - j * ks) : 1;
+        const int nk = WHOLE ? 1 : j < slabs ? min(ks, kfull - j * ks) : 1;
         if (elect_one()) {
           for (int i = 0; i < nk; ++i, sx += x_kb, sw += w_kb) {
 #pragma unroll
@@ -205,7 +218,19 @@ bool gate_tc_supported(const c2r_config* cfg) {
 
 constexpr int GT_SMEM = GT_RING + BM * BK * 2 + 1024;  // + what the last stage's MMA reads past its rows
 
-// SM count of the current device (a negative error code if that fails); the first call per device also sets the kernel's
+using GateKernel = void (*)(GateMaps, float*, float*, int, int, int, int, int, int, int, int32_t*);
+// The kernel for whole tiles of tw experts, or (0) the general one.
+static GateKernel gate_kernel(int tw, bool s) {
+  switch (tw) {
+    case 16: return s ? gate_tc_kernel<16, true> : gate_tc_kernel<16, false>;
+    case 32: return s ? gate_tc_kernel<32, true> : gate_tc_kernel<32, false>;
+    case 48: return s ? gate_tc_kernel<48, true> : gate_tc_kernel<48, false>;
+    case 64: return s ? gate_tc_kernel<64, true> : gate_tc_kernel<64, false>;
+    default: return gate_tc_kernel<0, false>;
+  }
+}
+
+// SM count of the current device (a negative error code if that fails); the first call per device also sets the kernels'
 // shared-memory limit.
 static int gate_sms() {
   constexpr int MAX_DEV = 64;
@@ -215,7 +240,8 @@ static int gate_sms() {
   if (dev < 0 || dev >= MAX_DEV) return C2R_ERR_UNSUPPORTED_SHAPE;
   int sms = __atomic_load_n(&sms_of_device[dev], __ATOMIC_ACQUIRE);
   if (sms == 0) {
-    C2R_CUDA(cudaFuncSetAttribute(gate_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GT_SMEM));
+    for (int tw = 0; tw <= 64; tw += 16)
+      for (int sh = 0; sh < 2; ++sh) C2R_CUDA(cudaFuncSetAttribute(gate_kernel(tw, sh), cudaFuncAttributeMaxDynamicSharedMemorySize, GT_SMEM));
     C2R_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     __atomic_store_n(&sms_of_device[dev], sms, __ATOMIC_RELEASE);
   }
@@ -252,7 +278,8 @@ int gate_tc_launch(const c2r_config* cfg, const void* X, const void* Wg, const v
   }
   if (!with_s && wsg && (rc = make_map(&m.s_tail, wsg, d, 1, 0, BK, tw))) return rc;
   const int grid = (int)(tiles_of(tw) < sms ? tiles_of(tw) : sms);
-  C2R_CUDA(launch_chained(gate_tc_kernel, grid, GT_THREADS, GT_SMEM, s, m, L, z, N, d, E, wsg != nullptr, tm, tw, ks, status));
+  const bool whole = tm == BM && E <= tw;
+  C2R_CUDA(launch_chained(gate_kernel(whole ? tw : 0, wsg != nullptr), grid, GT_THREADS, GT_SMEM, s, m, L, z, N, d, E, wsg != nullptr, tm, tw, ks, status));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }

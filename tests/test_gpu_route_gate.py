@@ -67,6 +67,14 @@ def test_gate_logits_do_not_depend_on_the_expert_tile(N, d, E, shared):
     test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared)
 
 
+# whole tiles of 16, 32, 48 and 64 experts, with and without the shared gate, against the general form (a batch below 64 tokens per
+# SM): contractions of one k-block, with a partial last one and longer than the ring; the first E of each tile's range and the last
+@pytest.mark.parametrize("N,d,E,shared", [(77, 64, 2, True), (77, 1096, 16, False), (300, 72, 17, False), (300, 712, 32, True), (1000, 136, 33, True),
+                                          (1000, 704, 48, True), (9472, 200, 49, False), (9472, 72, 63, True)])
+def test_gate_logits_of_whole_tiles(N, d, E, shared):
+    test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared)
+
+
 @pytest.mark.parametrize("N,K,P", [(1, 3, 4), (150, 7, 2), (1700, 6, 5), (40000, 4, 3), (525000, 1, 3), (263000, 2, 1),
                                    (176000, 3, 2)])
 def test_two_stage_dispatch_against_numpy(N, K, P):
