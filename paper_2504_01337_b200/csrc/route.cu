@@ -11,13 +11,16 @@ thread_local int g_last_cuda_error = 0;
 unsigned long long g_launch_count = 0;
 
 // ---------------------------------------------------------------------------------------------
-// Routing (Sec. 3.3 step 2).  LANES threads per token hold its logits in registers, eight each, as order-preserving integer
+// Routing (Sec. 3.3 step 2).  LANES threads per token hold its logits in registers, PER each, as order-preserving integer
 // keys; K rounds, each a maximum and then the lowest index that has it under the total order (value desc, index asc), after
 // the first among the experts of the top-1 expert's collaborator mask.  The number of blocks is fixed by the dispatch's blocking,
-// at most one per SM up to 148 blocks, so a block's latency is what the kernel takes: a thread per token over keys staged in
-// shared memory waits for 60 dependent selects a round, here it is eight and three shuffles.  us a call, that way / this: 16384 tokens
-// of 60 experts, top-8 13.9 / 6.8, 24000 tokens, top-4 11.0 / 8.1, 40000 13.8 / 10.9, 65536 12.9 / 14.1 (bound by instructions, of which
-// this has some more); with p, 24000 tokens, top-2 26.6 / 10.5.  Behind a pair GEMM (4096 tokens) 24 / 6, as its blocks spread.
+// at most one per SM up to 148 blocks, so up to there a block's latency is what the kernel takes: a thread per token over keys staged
+// in shared memory waits for 60 dependent selects a round, here it is PER and two reductions of log2(LANES) shuffles.  With more
+// blocks the kernel is bound by instructions, of which few threads with many experts each, and PER cut to E, need the fewest.
+// us a call, a thread per token / always eight experts a thread / this: 16384 tokens of 60 experts, top-8 12.5 / 6.8 / 6.9; 40000, top-4
+// 13.5 / 11.0 / 10.3; 65536 12.9 / 14.2 / 13.5; 262144 39.1 / 46.7 / 41.2; 48 experts, top-4, 131072 19.5 / 23.8 / 16.4; 24 experts
+// 11.3 / 12.9 / 9.1; with p, 24000 tokens of 60, top-4 11.7 / 12.6 / 10.6, 131072 47 / 36 / 35.  Behind a pair GEMM (4096 tokens) 24 / 6, as its
+// blocks spread.
 // ---------------------------------------------------------------------------------------------
 // Order-preserving map of a logit to an unsigned key above 0 (-0 and +0 share one, as they compare equal); 0 marks an
 // expert that is not a candidate.
@@ -31,9 +34,11 @@ __device__ __forceinline__ float key_logit(uint32_t k) { return __uint_as_float(
 // [blocks][E] experts' slot counts of the block's tokens -- the histogram the dispatch starts from, so it need not read
 // idx again to build it.
 //
-// Lane l of a token's LANES holds experts 4 l .. 4 l + 3 and as many from 4 LANES on: E <= 8 LANES.  FULL: the softmax over all
-// experts is wanted, for p or for weights that are not renormalised.
-template <int K, int LANES, bool FULL>
+// Lane l of a token's LANES holds experts 4 l .. 4 l + 3, as many from 4 LANES on, and so forth, PER in all: E <= PER LANES.  BITS:
+// those that may not be chosen again are taken out by a bit each, ahead of the next round's maximum, and not by a compare of each with
+// the choice (compares / bits, 262144 tokens: 60 experts, top-8 65.7 / 63.9, 24 experts 31.6 / 27.6; with eight a thread 16 experts
+// 21.7 / 20.9 at top-8 but 16.1 / 17.1 at top-6).  FULL: the softmax over all experts is wanted, for p or for weights that are not renormalised.
+template <int K, int LANES, int PER, bool FULL>
 __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* __restrict__ L, const uint64_t* __restrict__ mask,
                                                      int32_t* __restrict__ idx, float* __restrict__ w, float* __restrict__ p,
                                                      int32_t* __restrict__ status, int N, int E, int renorm, int tokens_per_block,
@@ -41,28 +46,29 @@ __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* _
   chain_begin();
   __shared__ uint64_t s_mask[64];
   __shared__ int s_cnt[64];
+  constexpr bool BITS = PER > 8;
   constexpr int OWN = (K + LANES - 1) / LANES;  // selections a lane keeps: j = sub, sub + LANES, ..
   const int tid = threadIdx.x, sub = tid & (LANES - 1);
   const int t_begin = blockIdx.x * tokens_per_block, tokens = min(N - t_begin, tokens_per_block);
   const bool vec = (E & 3) == 0 && ((uintptr_t)L & 15u) == 0;
   int flags = 0;
   auto expert = [&](int i) { return 4 * sub + (i & 3) + (i >> 2) * 4 * LANES; };
-  auto load = [&](int t, float (&v)[8]) {
+  auto load = [&](int t, float (&v)[PER]) {
     const float* row = L + (size_t)(t_begin + min(t, tokens - 1)) * E;
     if (vec) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < PER / 4; ++h) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (expert(4 * h) < E) x = *reinterpret_cast<const float4*>(row + expert(4 * h));
         v[4 * h] = x.x; v[4 * h + 1] = x.y; v[4 * h + 2] = x.z; v[4 * h + 3] = x.w;
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = expert(i) < E ? row[expert(i)] : 0.f;
+      for (int i = 0; i < PER; ++i) v[i] = expert(i) < E ? row[expert(i)] : 0.f;
     }
   };
   const int per_pass = blockDim.x / LANES, t_warp = tid / 32 * (32 / LANES), t_lane = (tid & 31) / LANES;
-  float next[8];
+  float next[PER];
   load(t_warp + t_lane, next);
   if (tid < 64) {
     s_cnt[tid] = 0;
@@ -72,43 +78,56 @@ __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* _
   for (int t0 = t_warp; t0 < tokens; t0 += per_pass) {  // warp-uniform
     const int t = t0 + t_lane;
     const bool live = t < tokens;
-    uint32_t key[8];
+    uint32_t key[PER], avail = ~0u;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < PER; ++i) {
       float v = next[i];
       if (v != v) { v = -INFINITY; if (live) flags |= C2R_STATUS_NAN_LOGIT; }
       key[i] = expert(i) < E ? logit_key(v) : 0u;
     }
     if (t0 + per_pass < tokens) load(t + per_pass, next);
-    float ex[FULL ? 8 : 1], top = 0.f, lg[OWN];
+    float ex[FULL ? PER : 1], top = 0.f, lg[OWN];
     int own[OWN];
     uint64_t chosen = 0;
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-      uint32_t m = max(max(max(key[0], key[1]), max(key[2], key[3])), max(max(key[4], key[5]), max(key[6], key[7])));
+      uint32_t best[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if (BITS && j > 0) key[i] = (avail >> i & 1u) ? key[i] : 0u;
+        best[i & 3] = max(best[i & 3], key[i]);
+      }
+      uint32_t m = max(max(best[0], best[1]), max(best[2], best[3]));
 #pragma unroll
       for (int o = LANES / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
       int sel = 64;
 #pragma unroll
-      for (int i = 7; i >= 0; --i) sel = key[i] == m ? expert(i) : sel;
+      for (int i = PER - 1; i >= 0; --i) sel = key[i] == m ? expert(i) : sel;
 #pragma unroll
       for (int o = LANES / 2; o > 0; o >>= 1) sel = min(sel, __shfl_xor_sync(0xffffffffu, sel, o));
       if (j == 0) {
         top = key_logit(m);
         if (FULL) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) ex[FULL ? i : 0] = expert(i) < E ? expf(key_logit(key[i]) - top) : 0.f;
+          for (int i = 0; i < PER; ++i) ex[FULL ? i : 0] = expert(i) < E ? expf(key_logit(key[i]) - top) : 0.f;
         }
         const uint64_t set = s_mask[sel];
+        avail = 0u;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < PER / 4; ++h) {
           const uint32_t bits = (uint32_t)(set >> ((4 * sub + h * 4 * LANES) & 63));
+          if (BITS) avail |= (bits & 15u) << (4 * h);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) key[4 * h + i] = (bits >> i & 1u) ? key[4 * h + i] : 0u;
+          for (int i = 0; i < 4; ++i)
+            if (!BITS) key[4 * h + i] = (bits >> i & 1u) ? key[4 * h + i] : 0u;
         }
       }
+      if (BITS) {
+        if ((sel >> 2 & (LANES - 1)) == sub) avail &= ~(1u << ((sel & 3) + 4 * (sel / (4 * LANES))));
+      } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) key[i] = expert(i) == sel ? 0u : key[i];
+        for (int i = 0; i < PER; ++i) key[i] = expert(i) == sel ? 0u : key[i];
+      }
       if (m == 0u) {  // candidate set exhausted: fall back to the lowest unselected expert
         if (live) flags |= C2R_STATUS_SET_TOO_SMALL;
         const uint64_t valid = (E == 64) ? ~0ull : ((1ull << E) - 1ull);
@@ -133,10 +152,19 @@ __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* _
       for (int o = LANES / 2; o > 0; o >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, o);
     }
     if (FULL) {
+      constexpr int PARTS = PER <= 4 ? 1 : PER <= 8 ? 2 : 4;
+      static_assert(!FULL || PER <= 16, "the sum's tree over a lane's groups of four");
       float u[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        u[i] = ex[FULL ? i : 0] + ex[FULL ? 4 + i : 0];
+        float part[PARTS];
+#pragma unroll
+        for (int h = 0; h < PARTS; ++h) part[h] = 4 * h < PER ? ex[FULL && 4 * h < PER ? 4 * h + i : 0] : 0.f;
+#pragma unroll
+        for (int x = PARTS / 2; x > 0; x >>= 1)
+#pragma unroll
+          for (int h = 0; h < x; ++h) part[h] += part[h + x];
+        u[i] = part[0];
 #pragma unroll
         for (int o = LANES / 2; o > 0; o >>= 1) u[i] += __shfl_xor_sync(0xffffffffu, u[i], o);
       }
@@ -146,13 +174,13 @@ __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* _
         float* out = p + (size_t)(t_begin + t) * E;
         if (vec && ((uintptr_t)p & 15u) == 0) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
+          for (int h = 0; h < PER / 4; ++h)
             if (expert(4 * h) < E)
               *reinterpret_cast<float4*>(out + expert(4 * h)) =
                   make_float4(ex[FULL ? 4 * h : 0] / sum, ex[FULL ? 4 * h + 1 : 0] / sum, ex[FULL ? 4 * h + 2 : 0] / sum, ex[FULL ? 4 * h + 3 : 0] / sum);
         } else {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
+          for (int i = 0; i < PER; ++i)
             if (expert(i) < E) out[expert(i)] = ex[FULL ? i : 0] / sum;
         }
       }
@@ -180,28 +208,45 @@ __global__ void __launch_bounds__(FULL ? 512 : 1024) route_kernel(const float* _
   }
 }
 
-template <int K, int LANES, bool FULL>
+template <int K, int LANES, int PER, bool FULL>
 static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
                         int32_t* status, int32_t* block_counts, cudaStream_t s) {
   const int tpb = perm_tokens_per_block(K), most = (cfg->N < tpb ? cfg->N : tpb) * LANES;
   const int blocks = (cfg->N + tpb - 1) / tpb;
-  // one block per SM with all its tokens at once; beyond, blocks that fit an SM together
-  const int limit = (FULL ? 512 : 1024) >> (blocks > SPREAD_SMS);
+  // One block per SM with all its tokens at once; beyond, blocks that fit an SM together; far beyond, blocks that load their next
+  // tokens while they rank these (60 experts, top-4, 512 / 256 threads: 65536 tokens 13.5 / 13.8, 90000 16.7 / 16.2, 262144 45.1 / 41.2;
+  // with K > 4 a block has 320 threads or 256 anyway, and 320 are the better).
+  const int limit = blocks <= SPREAD_SMS ? (FULL ? 512 : 1024) : FULL ? 256 : blocks > 4 * SPREAD_SMS && most > 384 ? 256 : 512;
   const int threads = most > limit ? limit : most < 64 ? 64 : (most + 31) / 32 * 32;  // at least the 64 that handle the mask and the counts
   static int done[64] = {};
-  const int rc = allow_smem(route_kernel<K, LANES, FULL>, done);
+  const int rc = allow_smem(route_kernel<K, LANES, PER, FULL>, done);
   if (rc) return rc;
-  C2R_CUDA(launch_chained(route_kernel<K, LANES, FULL>, blocks, threads, spread_smem(blocks, 0), s, L, mask, idx, w, p, status, cfg->N, cfg->E,
+  C2R_CUDA(launch_chained(route_kernel<K, LANES, PER, FULL>, blocks, threads, spread_smem(blocks, 0), s, L, mask, idx, w, p, status, cfg->N, cfg->E,
                           cfg->renorm, tpb, block_counts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
+// Threads per token and experts per thread.  Where all of a block's tokens are ranked at once and no SM has a second block, latency
+// counts: eight experts a thread (decode of one token 67.9 / 68.7 with sixteen).  Else two threads up to 24 experts and four beyond,
+// with as few places as hold E (a place costs as much as an expert: 33 experts in 64 places 46.9 us, in 48 places 31.1, 262144
+// tokens, top-4).  25 to 32 experts take four threads until instructions are all that counts (32 experts, four / two: top-4
+// 65536 tokens 8.2 / 8.4, 90000 10.1 / 9.4, 262144 27.9 / 22.2, but top-2 131072 9.9 / 10.5; the full softmax is always better off
+// with four, top-4 131072 tokens 19.0 / 20.5).
 template <int K, bool FULL>
 static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,
                         int32_t* status, int32_t* block_counts, cudaStream_t s) {
-  return cfg->E <= 16   ? route_launch<K, 2, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s)
-         : cfg->E <= 32 ? route_launch<K, 4, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s)
-                        : route_launch<K, 8, FULL>(cfg, L, mask, idx, w, p, status, block_counts, s);
+  const int tpb = perm_tokens_per_block(K), blocks = (cfg->N + tpb - 1) / tpb;
+  const bool many = !FULL && cfg->N > 512 * SPREAD_SMS && blocks > 4 * SPREAD_SMS;
+  auto at_once = [&](int lanes) { return blocks <= SPREAD_SMS && (cfg->N < tpb ? cfg->N : tpb) * lanes <= (FULL ? 512 : 1024); };
+  const auto launch = cfg->E <= 8                   ? route_launch<K, 2, 4, FULL>
+                      : cfg->E <= 16                ? route_launch<K, 2, 8, FULL>
+                      : cfg->E <= 24 && !at_once(4) ? route_launch<K, 2, 12, FULL>
+                      : cfg->E <= 32 && many        ? route_launch<K, 2, 16, FULL>
+                      : cfg->E <= 32                ? route_launch<K, 4, 8, FULL>
+                      : at_once(8)                  ? route_launch<K, 8, 8, FULL>
+                      : cfg->E <= 48                ? route_launch<K, 4, 12, FULL>
+                                                    : route_launch<K, 4, 16, FULL>;
+  return launch(cfg, L, mask, idx, w, p, status, block_counts, s);
 }
 template <int K>
 static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* mask, int32_t* idx, float* w, float* p,

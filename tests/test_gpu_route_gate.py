@@ -67,6 +67,41 @@ def test_gate_logits_do_not_depend_on_the_expert_tile(N, d, E, shared):
     test_gate_logits_do_not_depend_on_the_token_tile(N, d, E, shared)
 
 
+# expert counts at both ends of what a token's threads hold together (8, 16, 24, 32, 48, 64), a thread with fewer selections than
+# rounds and with more; enough tokens for every number of threads per block, and for two threads per token of 25 to 32 experts
+@pytest.mark.parametrize("E,K,N", [(2, 1, 37), (8, 8, 700), (9, 5, 700), (16, 3, 700), (17, 8, 700), (24, 2, 700), (25, 3, 700), (32, 8, 700), (33, 5, 700),
+                                   (48, 8, 700), (49, 3, 700), (64, 2, 700), (17, 4, 19000), (24, 8, 9500), (33, 8, 9500), (48, 4, 19000), (49, 4, 19000), (25, 8, 76000), (32, 4, 76000), (31, 5, 76000), (60, 4, 76000), (64, 8, 38000)])
+def test_route_at_the_edges_of_a_thread(E, K, N):
+    from paper_2504_01337_b200 import binding as B
+    rng = np.random.default_rng(E + K)
+    L = (rng.integers(-6, 7, (N, E)) / 4).astype(np.float32)  # many ties
+    L[rng.random((N, E)) < 0.02] = -np.inf
+    nan = rng.random(N) < 0.1
+    L[nan, rng.integers(0, E, N)[nan]] = np.nan
+    T = max(K - 1, 1)
+    sets = random_sets(E, T, seed=E) if T <= E - 1 else None
+    ref = np.where(np.isnan(L), -np.inf, L)
+    ref[np.isinf(ref).all(1), 0] = 0.0  # (a row of -inf alone has no weights)
+    Lin = np.where(np.isinf(np.where(np.isnan(L), -np.inf, L)).all(1)[:, None], ref, L)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    for masked in ((False, True) if sets is not None else (False,)):
+        for want_p in (False, True):
+            cfg = B.make_config(N, 64, E, 16, K, T, 1, 0, B.F32, 1)
+            idx, w, status = torch.zeros((N, K), **i32), torch.zeros((N, K), device="cuda"), torch.zeros(1, **i32)
+            p = torch.zeros((N, E), device="cuda") if want_p else None
+            ws = torch.zeros(B.workspace_bytes(cfg, B.WS_PERMUTE), dtype=torch.uint8, device="cuda")
+            B.route(cfg, dev(Lin), dev(mask_of(sets, E).view(np.int64)) if masked else None, idx, w, p, status, ws)
+            ridx, rw = O.c2r_route(ref, sets, K) if masked else O.topk_route(ref, K)
+            assert np.array_equal(host(idx), ridx)
+            assert_close_abs(host(w), rw, 1e-6, "w")
+            if want_p:
+                e = np.exp(ref.astype(np.float64) - ref.max(1, keepdims=True))
+                assert_close_abs(host(p), e / e.sum(1, keepdims=True), 1e-6, "p")
+            assert int(status.item()) == 1  # NaN logits, and nothing else
+            counts = host(ws.view(torch.int32))[:ws.numel() // 4 // E * E].reshape(-1, E).sum(0)
+            assert np.array_equal(counts, np.bincount(ridx.ravel(), minlength=E))
+
+
 # whole tiles of 16, 32, 48 and 64 experts, with and without the shared gate, against the general form (a batch below 64 tokens per
 # SM): contractions of one k-block, with a partial last one and longer than the ring; the first E of each tile's range and the last
 @pytest.mark.parametrize("N,d,E,shared", [(77, 64, 2, True), (77, 1096, 16, False), (300, 72, 17, False), (300, 712, 32, True), (1000, 136, 33, True),
