@@ -78,21 +78,40 @@ struct TileLoad {
       src[i] = (PIECES % THREADS == 0 || x < PIECES) && m < m_left ? row(m) + k * sk : nullptr;
     }
   }
-  // any: an aligned address that may be named where nothing is read
-  __device__ __forceinline__ void fetch(T* tile, int k_left, bool vec, const T* any) {
+  // any: an aligned address that may be named where nothing is read.  V16: pieces are aligned; else vec (simt_vec) says how far.
+  template <bool V16>
+  __device__ __forceinline__ void fetch(T* tile, int k_left, int vec, const T* any) {
+    T plain[PER][EPC];
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
       if (PIECES % THREADS != 0 && (int)threadIdx.x + i * THREADS >= PIECES) continue;
       const bool live = src[i] != nullptr && k_of[i] < k_left;
-      if (vec) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(tile + at[i])),
-                     "l"(live ? src[i] : any), "r"(live ? 16 : 0)
-                     : "memory");
-      } else {
+      const T* from = live ? src[i] : any;
+      const uint32_t to = (uint32_t)__cvta_generic_to_shared(tile + at[i]);
+      const int n = live ? 16 : 0;
+      if (V16) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(n) : "memory");
+      } else if (vec == 8) {
 #pragma unroll
-        for (int j = 0; j < EPC; ++j) tile[at[i] + j] = live ? src[i][j] : from_f32<T>(0.f);
+        for (int j = 0; j < 16; j += 8)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(to + j), "l"((const char*)from + (live ? j : 0)), "r"(n >> 1) : "memory");
+      } else if (vec == 4) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 4)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to + j), "l"((const char*)from + (live ? j : 0)), "r"(n >> 2) : "memory");
+      } else if (sizeof(T) == 2) {
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) plain[i][j] = live ? src[i][j] : from_f32<T>(0.f);
       }
       if (src[i] != nullptr) src[i] += step;
+    }
+    if (!V16 && sizeof(T) == 2 && vec == 0) {
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if (PIECES % THREADS != 0 && (int)threadIdx.x + i * THREADS >= PIECES) continue;
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) tile[at[i] + j] = plain[i][j];
+      }
     }
   }
   // The four rows (columns of the output) that thread t of W / 4 has, and their elements k .. k + 3: v[row][k].
@@ -126,7 +145,7 @@ struct TileLoad {
 // parts are 128 registers of a thread and one block per SM.
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
-template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int STAGES, int SIMT_THREADS>
+template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int STAGES, bool V16, int SIMT_THREADS>
 __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   chain_begin();
   using LA = TileLoad<T, TM, AK, SIMT_THREADS>;
@@ -175,7 +194,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   if (m0 >= M || n0 >= g.Ndim) return;
   const T* A = (const T*)g.A + a_off + (long long)m0 * g.sam;
   const T* B = (const T*)g.B + b_off;
-  const bool vec = g.vec != 0;
+  const int vec = g.vec;
   auto rowA = [&](int m) { return A + (long long)m * g.sam; };
   auto rowB = [&](int n) {
     if (g.B_last != nullptr && n0 + n == g.Ndim - 1) return (const T*)g.B_last;
@@ -195,9 +214,9 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   auto fetch = [&](int t) {
     if (t < n_tiles) {
       T* sa = tiles + t % STAGES * STAGE;
-      la.fetch(sa, Kd - t * SPAN, vec, (const T*)g.A);
-      lb.fetch(sa + LA::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
-      if (DUAL) lb2.fetch(sa + LA::ELEMS + LB::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
+      la.template fetch<V16>(sa, Kd - t * SPAN, vec, (const T*)g.A);
+      lb.template fetch<V16>(sa + LA::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
+      if (DUAL) lb2.template fetch<V16>(sa + LA::ELEMS + LB::ELEMS, Kd - t * SPAN, vec, (const T*)g.A);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -340,25 +359,31 @@ __global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
   }
 }
 
-template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int SIMT_THREADS = 256>
-static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
-  constexpr int STAGES = 4, G = SIMT_THREADS / ((TM / 4) * (TN / 4));
+template <int STAGES, bool V16, typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int SIMT_THREADS>
+static int simt_launch_stages(const SimtGemm& g, dim3 grid, cudaStream_t s) {
+  constexpr int G = SIMT_THREADS / ((TM / 4) * (TN / 4));
   constexpr int tiles = STAGES * (int)sizeof(T) * (TileLoad<T, TM, AK, SIMT_THREADS>::ELEMS + (DUAL ? 2 : 1) * TileLoad<T, TN, BN, SIMT_THREADS>::ELEMS);
   constexpr int red = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4) * 4, smem = tiles > red ? tiles : red;
   static int done[64] = {};
-  if (const int rc = allow_smem(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, SIMT_THREADS>, done, smem)) return rc;
-  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, SIMT_THREADS>, dim3(m_tiles, (g.Ndim + TN - 1) / TN, z),
-                          SIMT_THREADS, smem, s, g));
+  if (const int rc = allow_smem(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, V16, SIMT_THREADS>, done, smem)) return rc;
+  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, V16, SIMT_THREADS>, grid, SIMT_THREADS, smem, s, g));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
+template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int SIMT_THREADS = 256>
+static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
+  const dim3 grid(m_tiles, (g.Ndim + TN - 1) / TN, z);
+  return g.vec == 16 ? simt_launch_stages<4, true, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s)
+                     : simt_launch_stages<4, false, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s);
+}
 
-// Whether every 16-byte piece the kernel loads lies on a 16-byte boundary.
+// Bytes of a cp.async that every 16-byte piece the kernel loads is aligned to: 16, 8, 4, or 0 for elements of two bytes that lie on no
+// 4-byte boundary.
 template <typename T>
 static int simt_vec(const SimtGemm& g) {
-  constexpr int EPC = 16 / sizeof(T);
-  const uintptr_t bits = (uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last;
-  return (bits & 15u) == 0 && (g.sak == 1 ? g.sam : g.sak) % EPC == 0 && (g.sbk == 1 ? g.sbn : g.sbk) % EPC == 0 && g.sB % EPC == 0;
+  const uint64_t bits = (uint64_t)(uintptr_t)g.A | (uintptr_t)g.B | (uintptr_t)g.B_last |
+                        sizeof(T) * (uint64_t)((g.sak == 1 ? g.sam : g.sak) | (g.sbk == 1 ? g.sbn : g.sbk) | g.sB);
+  return (bits & 15u) == 0 ? 16 : (bits & 7u) == 0 ? 8 : (bits & 3u) == 0 ? 4 : 0;
 }
 
 // max_m: rows (SIMT_ROWS: of all groups together) or Mdim.  AK / BN: the contraction index is the contiguous one of A / of B.

@@ -33,3 +33,9 @@ def test_unaligned_arrays(counts, d, I, bf16, offset):
         return AB, H, Yp, dAB, dXp, dW13, dW2
 
     assert all(torch.isfinite(a).all() and torch.equal(a, b) for a, b in zip(run(0), run(offset)))
+
+
+# bf16 arrays on a 4-byte boundary and no better one
+@pytest.mark.parametrize("counts,d,I", [([37, 0, 5, 64], 40, 48), ([700, 650, 800], 520, 144)])
+def test_arrays_on_a_four_byte_boundary(counts, d, I):
+    test_unaligned_arrays(counts, d, I, True, 2)
