@@ -93,7 +93,10 @@ inline int spread_smem(int64_t blocks, int need) {
   const int share = per_sm > 0 && per_sm <= 8 ? 227 * 1024 / ((int)per_sm + 1) + 1024 : 0;  // one more does not fit
   return share > need ? share : need;
 }
-// Raises a kernel's limit of dynamic shared memory, once per device (`done`: a flag each).
+// Raises a kernel's limit of dynamic shared memory, once per device (`done`: a flag each), and asks for the largest split of an SM's
+// L1 in its favour: an SM must be empty to change the split, so a chain of kernels that each take the smallest one that
+// holds them cannot overlap (smallest / largest, us: expert calls of a training step of 1500 fp32 tokens 111.4 / 106.4, whole
+// training step of 300 173 / 149).
 template <typename... P>
 inline int allow_smem(void (*kernel)(P...), int (&done)[64], int bytes = SPREAD_SMEM) {
   int dev = 0;
@@ -101,6 +104,7 @@ inline int allow_smem(void (*kernel)(P...), int (&done)[64], int bytes = SPREAD_
   if (dev < 0 || dev >= 64) return C2R_ERR_UNSUPPORTED_SHAPE;
   if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
     C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
   }
   return C2R_OK;

@@ -39,6 +39,7 @@ struct SimtGemm {
   const void* B_last;
   void* C_last;
   int n_groups, vec;
+  int64_t expect_k;        // SIMT_WGRAD: rows a group is expected to have (a hint)
 };
 
 // One grouped SwiGLU evaluation (forward or backward); members a direction does not use stay NULL.

@@ -138,15 +138,17 @@ struct TileLoad {
 // exact sum than one chain is.  STAGES - 1 tiles of both operands are on their way (cp.async) while one is used.  The small
 // configurations this serves are bound by latency and by the operands' way from shared memory (two 16-byte reads per 16 products;
 // 8 x 8 outputs per thread halve those, but leave too few warps: training step of 1500 tokens 159 us, so 222).  Tiles that went
-// through registers, one ahead, transposed on their way, took, in us before / after for whole passes: fp32 forward of 4096 tokens of 512,
-// top-4 of 8 x 512, 982 / 920, training step 2956 / 2716; bf16 off the tensor-core shapes (8192 tokens of 264) 419 / 316 and 1443 / 1091;
-// the expert calls of 512 tokens alone 21.5 / 22.1 and 46.7 / 49.1.
+// through registers, one ahead, transposed on their way, took, in us before / after for expert calls (forward + backward): fp32, top-2 of 8
+// experts of 128, d 256: 100 tokens 50.3 / 41.4, 512 70.7 / 57.0, 1500 120 / 99; 2600 tokens of 512, top-4 of 8 x 512 1767 / 1468; bf16 off
+// the tensor-core shapes (8192 tokens of 264, top-2 of 8 x 512) 2406 / 1583; fp32 arrays on no 16-byte boundary (2600 tokens) 2179 / 1993,
+// bf16 on an 8-byte one (512 tokens of 264) 87 / 65.  Left to itself the compiler holds the 32-wide forms to 60 registers, which costs the
+// small launches a third (512 tokens 57.0 / 74.4), and gives the 64 x 64 ones more than half an SM's.
 // 64 x 64 tiles where they fill the chip, else 32-wide ones; the two SwiGLU products always take 32 x 32, since at 64 x 64 their
 // parts are 128 registers of a thread and one block per SM.
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
 template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int STAGES, bool V16, int SIMT_THREADS>
-__global__ void __launch_bounds__(SIMT_THREADS) simt_gemm_kernel(SimtGemm g) {
+__global__ void __launch_bounds__(SIMT_THREADS, DUAL || (TM == 64 && TN == 64) ? 2 : 1) simt_gemm_kernel(SimtGemm g) {
   chain_begin();
   using LA = TileLoad<T, TM, AK, SIMT_THREADS>;
   using LB = TileLoad<T, TN, BN, SIMT_THREADS>;
@@ -370,11 +372,17 @@ static int simt_launch_stages(const SimtGemm& g, dim3 grid, cudaStream_t s) {
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
+// Four stages, or two where they would be room taken for nothing: small launches, which begin beside the one before them if they fit, and
+// weight gradients over at most two tiles of rows (us, expert calls, four everywhere / so: forward of 100 tokens, top-2 of 8 experts of
+// 128, d 256, 19.8 / 17.6, of 512 23.1 / 21.6; backward of 100 tokens 35.5 / 29.7; two everywhere costs a training step of 1500
+// 106 / 114).
 template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int SIMT_THREADS = 256>
 static int simt_launch_tile(const SimtGemm& g, int m_tiles, int z, cudaStream_t s) {
   const dim3 grid(m_tiles, (g.Ndim + TN - 1) / TN, z);
-  return g.vec == 16 ? simt_launch_stages<4, true, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s)
-                     : simt_launch_stages<4, false, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s);
+  const bool two = g.mode == SIMT_ROWS ? (int64_t)grid.x * grid.y * z <= 3 * 148 : g.expect_k <= 2 * SPAN;
+  if (g.vec != 16) return simt_launch_stages<4, false, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s);
+  return two ? simt_launch_stages<2, true, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s)
+             : simt_launch_stages<4, true, T, TC, TM, TN, DUAL, S, AK, BN, SIMT_THREADS>(g, grid, s);
 }
 
 // Bytes of a cp.async that every 16-byte piece the kernel loads is aligned to: 16, 8, 4, or 0 for elements of two bytes that lie on no
@@ -575,7 +583,7 @@ int simt_swiglu_bwd(const c2r_config* cfg, const SwigluCall& a, cudaStream_t s) 
   if (rc) return rc;
   g.token_acc = nullptr;
   // dW2_e = dYp_e^T H_e   [d, I]
-  g.mode = SIMT_WGRAD; g.accumulate = a.accumulate;
+  g.mode = SIMT_WGRAD; g.accumulate = a.accumulate; g.expect_k = nE == 1 ? max_m : (int64_t)cfg->N * cfg->K / nE;
   g.A = a.dYp; g.sam = 1; g.sak = d; g.B = a.H; g.sbn = 1; g.sbk = I;
   g.C = a.dW2; g.ldc = I; g.sC = (long long)d * I; g.Mdim = d; g.Ndim = I;
   rc = simt_launch<false, false, T>(g, nE, d, s);
