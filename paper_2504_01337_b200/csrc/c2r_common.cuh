@@ -68,18 +68,25 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // forward pass of 1 token 88 / 74, of 64 tokens 233 / 221, fp32 training step of 1500 tokens 206 / 193; calibration, two-stage
 // dispatch and passes past 0.5 ms move by no more than their spread).  No kernel may return, or touch what an earlier one
 // reads or writes, before the wait: the next one relies on this one's completion to imply that of all earlier ones.
+//
+// A launch with dynamic shared memory asks for the largest split of the SM's L1 in its favour: an SM must be empty to change the
+// split, so a chain of kernels that each take the smallest one that holds them cannot overlap (smallest / largest: expert calls of
+// a training step of 1500 fp32 tokens 111.4 / 106.4, whole training step of 300 173 / 149).  A launch without leaves the L1 as it is: the
+// ranking of a very large dispatch reads its counts through it (125000 tokens, top-4, both stages' indices: 64 / 66).
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t c = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
   c.gridDim = grid;
   c.blockDim = block;
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = attr;
-  c.numAttrs = 1;
+  c.numAttrs = smem > 0 ? 2 : 1;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
@@ -87,26 +94,41 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
 // chained kernel become resident as the SMs of the kernel before it fall free, and the first SMs to do so take as many as fit:
 // seven routing blocks on one SM, bound by its issue slots, while most of the chip waits (4096 tokens behind a pair GEMM: 24 us where
 // the kernel alone takes 9).  A block counts with what it asks for, so it asks for its share of an SM.
-constexpr int SPREAD_SMS = 148, SPREAD_SMEM = 120 * 1024;
-inline int spread_smem(int64_t blocks, int need) {
+// Its static shared memory and what the SM keeps for every block are part of the share: left out, with 22 KB of its own a block of the
+// two-stage dispatch's ranking took a third of an SM where a fourth was meant (both stages' indices of 24000 tokens, top-4, 14.3 us; so, and
+// with 14 KB, 12.5; 50000 tokens 22.5 / 19.2).
+constexpr int SPREAD_SMS = 148, SPREAD_SMEM = 120 * 1024, SM_SMEM = 228 * 1024, SM_SMEM_PER_BLOCK = 1024;
+constexpr int spread_share(int per_sm, int static_bytes) {
+  const int dynamic = SM_SMEM / (per_sm + 1) + 512 - SM_SMEM_PER_BLOCK - static_bytes;
+  return dynamic > 0 ? dynamic : 0;
+}
+constexpr bool spread_holds(int per_sm, int static_bytes) {  // so many blocks fit and one more does not
+  const int block = (spread_share(per_sm, static_bytes) + static_bytes + 127) / 128 * 128 + SM_SMEM_PER_BLOCK;
+  return per_sm * block <= SM_SMEM && (per_sm + 1) * block > SM_SMEM;
+}
+static_assert(spread_holds(1, 0) && spread_holds(2, 0) && spread_holds(3, 13824) && spread_holds(4, 13824) && spread_holds(8, 768) && spread_holds(8, 13824),
+              "blocks per SM");
+static_assert(spread_share(1, 0) <= SPREAD_SMEM, "within the kernels' limit");
+inline int spread_smem(int64_t blocks, int need, int static_bytes) {
   const int64_t per_sm = (blocks + SPREAD_SMS - 1) / SPREAD_SMS;
-  const int share = per_sm > 0 && per_sm <= 8 ? 227 * 1024 / ((int)per_sm + 1) + 1024 : 0;  // one more does not fit
+  const int share = per_sm > 0 && per_sm <= 8 ? spread_share((int)per_sm, static_bytes) : 0;
   return share > need ? share : need;
 }
-// Raises a kernel's limit of dynamic shared memory, once per device (`done`: a flag each), and asks for the largest split of an SM's
-// L1 in its favour: an SM must be empty to change the split, so a chain of kernels that each take the smallest one that
-// holds them cannot overlap (smallest / largest, us: expert calls of a training step of 1500 fp32 tokens 111.4 / 106.4, whole
-// training step of 300 173 / 149).
+// Raises a kernel's limit of dynamic shared memory, once per device (`done`: the kernel's static bytes and one more).
 template <typename... P>
-inline int allow_smem(void (*kernel)(P...), int (&done)[64], int bytes = SPREAD_SMEM) {
+inline int allow_smem(void (*kernel)(P...), int (&done)[64], int bytes = SPREAD_SMEM, int* static_bytes = nullptr) {
   int dev = 0;
   C2R_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return C2R_ERR_UNSUPPORTED_SHAPE;
-  if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
+  int known = __atomic_load_n(&done[dev], __ATOMIC_ACQUIRE);
+  if (known == 0) {
+    cudaFuncAttributes a;
+    C2R_CUDA(cudaFuncGetAttributes(&a, kernel));
+    known = (int)a.sharedSizeBytes + 1;
     C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    C2R_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-    __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
+    __atomic_store_n(&done[dev], known, __ATOMIC_RELEASE);
   }
+  if (static_bytes != nullptr) *static_bytes = known - 1;
   return C2R_OK;
 }
 

@@ -510,7 +510,7 @@ static int gate_simt_launch(const c2r_config* cfg, const float* X, const float* 
   const int budget = (blocks <= SPREAD_SMS ? 200 : 100) * 1024;
   int kc = cfg->d;
   if ((tm + cols) * (kc + 4) * 4 > budget) kc = (budget / 2 / 4 / (tm + cols) - 4) / 32 * 32;
-  const int need = (cfg->d > kc ? 2 : 1) * (tm + cols) * (kc + 4) * 4, smem = spread_smem(blocks, need);
+  const int need = (cfg->d > kc ? 2 : 1) * (tm + cols) * (kc + 4) * 4, smem = spread_smem(blocks, need, 0);
   static int done[2][64] = {};
   const int rc = wide ? allow_smem(gate_simt_kernel<2, 4>, done[1], 200 * 1024) : allow_smem(gate_simt_kernel<1, 1>, done[0], 200 * 1024);
   if (rc) return rc;

@@ -1,5 +1,7 @@
 // Dispatch on one device: atomic-free histogram / prefix-scan / stable rank over experts, the
 // 16-byte vectorised row gather, the weighted combine and their backward twins.
+#include <type_traits>
+
 #include "c2r_common.cuh"
 #include "gemm.h"
 
@@ -212,8 +214,17 @@ struct RankArgs {
   long long R;
   int E, row_align;
 };
-template <bool DEDUP>
-__device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int slots_per_block, int n_blocks, int K) {
+struct RankShared {
+  int grp_cnt[PERM_GROUPS][64];
+  int start[64], total[64], by_rank[64], off[65];
+  int part[2][PERM_THREADS / 64][64];  // partial sums: [before | total][share of the blocks][expert]
+  int bad;
+};
+struct RankSharedDedup : RankShared {
+  int row[PERM_THREADS], q[PERM_THREADS];
+};
+template <bool DEDUP, typename Shared>
+__device__ __forceinline__ void rank_block(Shared& sh, const RankArgs& a, long long NK, int slots_per_block, int n_blocks, int K) {
   const int E = a.E, row_align = a.row_align;
   int32_t* __restrict__ slot_of_row = a.slot_of_row;
   int32_t* __restrict__ row_of_slot = a.row_of_slot;
@@ -225,10 +236,9 @@ __device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int 
   const float weight = live && w_row != nullptr ? a.w[slot] : 0.f;
   const int rank_mine = rank_of_thread(a.expert_rank, E);
   constexpr int PARTS = PERM_THREADS / 64;
-  __shared__ int grp_cnt[PERM_GROUPS][64];
-  __shared__ int s_start[64], s_total[64], s_by_rank[64], s_off[65];
-  __shared__ int s_part[2][PARTS][64];  // partial sums: [before | total][share of the blocks][expert]
-  __shared__ int s_bad;
+  auto& grp_cnt = sh.grp_cnt;
+  auto& s_part = sh.part;
+  int *const s_start = sh.start, *const s_total = sh.total, *const s_by_rank = sh.by_rank, *const s_off = sh.off;
   for (int i = threadIdx.x; i < PERM_GROUPS * 64; i += blockDim.x) (&grp_cnt[0][0])[i] = 0;
   {
     const int e = threadIdx.x & 63, part = threadIdx.x >> 6;
@@ -244,7 +254,7 @@ __device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int 
     s_part[0][part][e] = before;
     s_part[1][part][e] = total;
   }
-  layout_order(rank_mine, E, s_by_rank, &s_bad);  // (its barriers also publish s_part and the zeroed grp_cnt)
+  layout_order(rank_mine, E, s_by_rank, &sh.bad);  // (its barriers also publish s_part and the zeroed grp_cnt)
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
     int before = 0, total = 0;
 #pragma unroll
@@ -254,7 +264,7 @@ __device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int 
   }
   __syncthreads();
   segment_offsets(s_by_rank, s_total, E, row_align, s_off);
-  if (threadIdx.x == 0 && blockIdx.x == 0 && s_bad && a.status != nullptr) atomicOr(a.status, C2R_STATUS_BAD_INDEX);
+  if (threadIdx.x == 0 && blockIdx.x == 0 && sh.bad && a.status != nullptr) atomicOr(a.status, C2R_STATUS_BAD_INDEX);
   int flags = 0;
   const int e_mine = group_count(raw, live, E, grp_cnt, flags, DEDUP);
   __syncthreads();
@@ -282,7 +292,7 @@ __device__ __forceinline__ void rank_block(const RankArgs& a, long long NK, int 
   if constexpr (!DEDUP) {
     rank_and_write(e_mine, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, weight, w_row);
   } else {
-    __shared__ int s_row[PERM_THREADS], s_q[PERM_THREADS];
+    int *const s_row = sh.row, *const s_q = sh.q;
     int row = -1;
     rank_and_write(e_mine, E, slots_per_block, grp_cnt, s_start, row_of_slot, slot_of_row, 0.f, nullptr, K, &row);
     s_row[threadIdx.x] = row;
@@ -301,15 +311,19 @@ template <bool TWO>
 __global__ void __launch_bounds__(PERM_THREADS) perm_rank_fused_kernel(const RankArgs a, const RankArgs b, long long NK, int slots_per_block,
                                                                        int n_blocks, int K) {
   chain_begin();
-  if (TWO && blockIdx.y == 1) rank_block<true>(b, NK, slots_per_block, n_blocks, K);
-  else rank_block<false>(a, NK, slots_per_block, n_blocks, K);
+  __shared__ std::conditional_t<TWO, RankSharedDedup, RankShared> sh;  // one for both sides
+  if constexpr (TWO) {
+    if (blockIdx.y == 1) return rank_block<true>(sh, b, NK, slots_per_block, n_blocks, K);
+  }
+  rank_block<false>(sh, a, NK, slots_per_block, n_blocks, K);
 }
 template <bool TWO>
 static int rank_launch(const RankArgs& a, const RankArgs& b, long long NK, int slots_per_block, int n_blocks, int grid, int K, cudaStream_t s) {
   static int done[64] = {};
-  const int rc = allow_smem(perm_rank_fused_kernel<TWO>, done);
+  int own = 0;
+  const int rc = allow_smem(perm_rank_fused_kernel<TWO>, done, SPREAD_SMEM, &own);
   if (rc) return rc;
-  C2R_CUDA(launch_chained(perm_rank_fused_kernel<TWO>, dim3(grid, TWO ? 2 : 1), PERM_THREADS, spread_smem((TWO ? 2 : 1) * grid, 0), s, a, b, NK,
+  C2R_CUDA(launch_chained(perm_rank_fused_kernel<TWO>, dim3(grid, TWO ? 2 : 1), PERM_THREADS, spread_smem((TWO ? 2 : 1) * grid, 0, own), s, a, b, NK,
                           slots_per_block, n_blocks, K));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
@@ -1256,8 +1270,9 @@ static int dispatch_dedup_impl(const c2r_config* cfg, const int32_t* idx, const 
     // Two launches for both indices (eleven took 39 us of 16384 tokens' dispatch, three 17, these 9).  scratch: [nb][P] block counts, which fit:
     // a block but the last owns at least 448 slots and P is at most 64, and the area is a whole number of 256 bytes.
     static int done[64] = {};
-    if (const int rc = allow_smem(dedup_hist_kernel, done)) return rc;
-    C2R_CUDA(launch_chained(dedup_hist_kernel, nb, PERM_THREADS, spread_smem(nb, 0), s, idx, part, NK, E, K, P, spb, block_counts, scratch, key,
+    int own = 0;
+    if (const int rc = allow_smem(dedup_hist_kernel, done, SPREAD_SMEM, &own)) return rc;
+    C2R_CUDA(launch_chained(dedup_hist_kernel, nb, PERM_THREADS, spread_smem(nb, 0, own), s, idx, part, NK, E, K, P, spb, block_counts, scratch, key,
                             status));
     C2R_LAUNCH_CHECK();
     const RankArgs a = {idx, block_counts, expert_rank, counts, offsets, row_of_slot, slot_of_row, nullptr, nullptr, status, R, E, cfg->row_align};

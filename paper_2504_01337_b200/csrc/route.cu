@@ -219,9 +219,10 @@ static int route_launch(const c2r_config* cfg, const float* L, const uint64_t* m
   const int limit = blocks <= SPREAD_SMS ? (FULL ? 512 : 1024) : FULL ? 256 : blocks > 4 * SPREAD_SMS && most > 384 ? 256 : 512;
   const int threads = most > limit ? limit : most < 64 ? 64 : (most + 31) / 32 * 32;  // at least the 64 that handle the mask and the counts
   static int done[64] = {};
-  const int rc = allow_smem(route_kernel<K, LANES, PER, FULL>, done);
+  int own = 0;
+  const int rc = allow_smem(route_kernel<K, LANES, PER, FULL>, done, SPREAD_SMEM, &own);
   if (rc) return rc;
-  C2R_CUDA(launch_chained(route_kernel<K, LANES, PER, FULL>, blocks, threads, spread_smem(blocks, 0), s, L, mask, idx, w, p, status, cfg->N, cfg->E,
+  C2R_CUDA(launch_chained(route_kernel<K, LANES, PER, FULL>, blocks, threads, spread_smem(blocks, 0, own), s, L, mask, idx, w, p, status, cfg->N, cfg->E,
                           cfg->renorm, tpb, block_counts));
   C2R_LAUNCH_CHECK();
   return C2R_OK;

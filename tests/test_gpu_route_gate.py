@@ -179,3 +179,9 @@ def test_full_softmax_of_small_batches(K, E, N, renorm):
     # expf and a division: a few units in the last place of values up to 1
     assert_close_abs(host(w), rw, 1e-6, "w")
     assert_close_abs(host(p), O.softmax_rows(L), 1e-6, "p")
+
+
+# blocks of the ranking at two, three, four, eight and nine per SM, where its share of an SM's shared memory changes
+@pytest.mark.parametrize("N,K,P", [(9600, 4, 3), (19100, 4, 9), (28600, 4, 1), (66300, 4, 3), (75900, 4, 4)])
+def test_two_stage_dispatch_at_the_edges_of_a_share(N, K, P):
+    test_two_stage_dispatch_against_numpy(N, K, P)
