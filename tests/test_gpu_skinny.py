@@ -93,3 +93,24 @@ def test_a_token_gets_the_same_bits_from_either_kernel(n):
         rows = lay.t["row_of_slot"].long()[:n * wl.K]
         got.append([lay.t[x][:n] for x in ("L", "idx", "Ys", "Hs", "Y")] + [lay.t[x][rows] for x in ("H", "Yp")])
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("n", [1, 100, 200])
+def test_a_forward_pass_has_the_same_bits_when_a_backward_pass_follows(n):
+    """The kernels that keep nothing (streaming, alone and with the shared expert in the launch, and pair tiles) against the one that
+    keeps the local derivatives."""
+    from paper_2504_01337_b200.layer import C2RLayer
+    wl = G.Workload("kept", N=n, d=336, E=8, I=400, K=3, T=4, P=2, I_s=528, bf16=True, seed=11)
+    X = G.hidden(wl)
+    Wg, wsg = G.gate_weights(wl)
+    W, sh, sets = G.expert_weights(wl), G.shared_weights(wl), random_sets(wl.E, wl.T, seed=5)
+    got = []
+    for backward in (False, True):
+        lay = C2RLayer(n, wl.d, wl.E, wl.I, wl.K, wl.T, wl.P, wl.I_s, True, backward=backward)
+        lay.set_params(Wg, *W, wsg, sh)
+        lay.set_routing(mask=mask_of(sets, wl.E))
+        lay.set_input(X)
+        lay.forward()
+        rows = lay.t["row_of_slot"].long()
+        got.append([lay.t[x] for x in ("L", "idx", "Ys", "Hs", "Y")] + [lay.t[x][rows] for x in ("H", "Yp")])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
