@@ -69,11 +69,11 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // dispatch and passes past 0.5 ms move by no more than their spread).  No kernel may return, or touch what an earlier one
 // reads or writes, before the wait: the next one relies on this one's completion to imply that of all earlier ones.
 //
-// A launch with dynamic shared memory asks for the largest split of the SM's L1 in its favour: an SM must be empty to change the
+// MAX_SPLIT (the CUDA-core GEMMs): the largest split of the SM's L1 in favour of shared memory.  An SM must be empty to change the
 // split, so a chain of kernels that each take the smallest one that holds them cannot overlap (smallest / largest: expert calls of
-// a training step of 1500 fp32 tokens 111.4 / 106.4, whole training step of 300 173 / 149).  A launch without leaves the L1 as it is: the
-// ranking of a very large dispatch reads its counts through it (125000 tokens, top-4, both stages' indices: 64 / 66).
-template <typename... P, typename... A>
+// a training step of 1500 fp32 tokens 111.4 / 106.4, whole training step of 300 173 / 149).  Routing and dispatch leave it alone: the row
+// pass behind them reads through the L1 that they leave (two-stage dispatch of 25000 tokens of 1536, one expert each, 61.5 / 65.7).
+template <bool MAX_SPLIT = false, typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t c = {};
   cudaLaunchAttribute attr[2];
@@ -86,7 +86,7 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = attr;
-  c.numAttrs = smem > 0 ? 2 : 1;
+  c.numAttrs = MAX_SPLIT ? 2 : 1;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 

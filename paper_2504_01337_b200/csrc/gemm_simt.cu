@@ -368,7 +368,7 @@ static int simt_launch_stages(const SimtGemm& g, dim3 grid, cudaStream_t s) {
   constexpr int red = G == 1 ? 0 : (DUAL ? 2 : 1) * G * TM * (TN + 4) * 4, smem = tiles > red ? tiles : red;
   static int done[64] = {};
   if (const int rc = allow_smem(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, V16, SIMT_THREADS>, done, smem)) return rc;
-  C2R_CUDA(launch_chained(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, V16, SIMT_THREADS>, grid, SIMT_THREADS, smem, s, g));
+  C2R_CUDA(launch_chained<true>(simt_gemm_kernel<T, TC, TM, TN, DUAL, S, AK, BN, STAGES, V16, SIMT_THREADS>, grid, SIMT_THREADS, smem, s, g));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
 }
@@ -514,7 +514,7 @@ static int gate_simt_launch(const c2r_config* cfg, const float* X, const float* 
   static int done[2][64] = {};
   const int rc = wide ? allow_smem(gate_simt_kernel<2, 4>, done[1], 200 * 1024) : allow_smem(gate_simt_kernel<1, 1>, done[0], 200 * 1024);
   if (rc) return rc;
-  C2R_CUDA(launch_chained(wide ? gate_simt_kernel<2, 4> : gate_simt_kernel<1, 1>, blocks, threads, smem, s, X, Wg, wsg, L, z, cfg->N, cfg->d,
+  C2R_CUDA(launch_chained<true>(wide ? gate_simt_kernel<2, 4> : gate_simt_kernel<1, 1>, blocks, threads, smem, s, X, Wg, wsg, L, z, cfg->N, cfg->d,
                           cfg->E, cols, tm, kc, vec));
   C2R_LAUNCH_CHECK();
   return C2R_OK;
