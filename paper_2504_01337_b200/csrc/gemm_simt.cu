@@ -130,6 +130,10 @@ struct TileLoad {
   }
 };
 
+// Blocks per SM that the register limit has to allow.
+template <bool DUAL, int TM, int TN>
+constexpr int simt_min_blocks = DUAL || (TM == 64 && TN == 64) ? 2 : 1;
+
 // C_g(m,n) = sum_k A_g(m,k) B_g(n,k) with arbitrary strides; see SimtGemm for the two modes.
 //
 // A block computes TM x TN outputs; (TM / 4)(TN / 4) threads hold a 4 x 4 share each.  A sum over k is kept as S partial sums,
@@ -148,7 +152,7 @@ struct TileLoad {
 // Blocks: y = tile along N; x = tile along M -- SIMT_ROWS: over all groups' row tiles, found from the counts -- ; z = group
 // (SIMT_WGRAD).
 template <typename T, typename TC, int TM, int TN, bool DUAL, int S, bool AK, bool BN, int STAGES, bool V16, int SIMT_THREADS>
-__global__ void __launch_bounds__(SIMT_THREADS, DUAL || (TM == 64 && TN == 64) ? 2 : 1) simt_gemm_kernel(SimtGemm g) {
+__global__ void __launch_bounds__(SIMT_THREADS, simt_min_blocks<DUAL, TM, TN>) simt_gemm_kernel(SimtGemm g) {
   chain_begin();
   using LA = TileLoad<T, TM, AK, SIMT_THREADS>;
   using LB = TileLoad<T, TN, BN, SIMT_THREADS>;
